@@ -163,7 +163,10 @@ int fdtd_set_spectrum(fdtd_ctx *ctx, double f_max, int n_total_steps);
 
 /* Advance n >= 0 leapfrog steps (H^{n+1/2} from E^n, then E^{n+1} from
  * H^{n+1/2} and J^{n+1/2}, then probes and DFT).  Asynchronous on the
- * context's stream; fields stay on the device between calls. */
+ * context's stream; fields stay on the device between calls.  FP32 boards up
+ * to 24 Mi grid points at depth 1 run many steps per cooperative launch, the
+ * others five launches per step replayed as CUDA graphs; a board's fields and
+ * traces are the same bit for bit either way. */
 int fdtd_step(fdtd_ctx *ctx, int n);
 
 /* fdtd_step with every phase launched directly (no CUDA graph) and timed
@@ -348,7 +351,9 @@ int fdtd_energy_static(const float *const fields[9], const float *const eps_r[3]
 /* ---------------- batching (many boards, one launch per phase) -------------
  * A batch steps many boards with one kernel launch per phase (UPML H, interior
  * fused H+E, UPML E, sources/probes) over a packed list of (board, tile) work
- * items, replayed as one CUDA graph per chunk of steps.  Each board's
+ * items, replayed as one CUDA graph per chunk of steps.  FP32 members up to 24
+ * Mi grid points are worked in groups whose states stay in L2, many steps per
+ * cooperative launch, each member by its own share of the blocks.  Each board's
  * arithmetic is identical to stepping it alone.  Boards keep their own device
  * state and may join or leave between calls.  All boards must share the
  * batch's stream (the batch uses its own; member contexts must not be
@@ -398,7 +403,9 @@ void fdtd_batch_destroy(fdtd_batch *b);
  * depth in effect); batches run depth 1.  pair_zseg is the z-segment length
  * of the two-step pass (default 38, >= 2).  Values <= 0 keep the current
  * setting; unsupported tiles are rejected with FDTD_EINVAL.  Applies to
- * launches queued afterwards. */
+ * launches queued afterwards.  Tile, segment and graph settings shape the
+ * tiled launches; boards that step many times per launch (fdtd_step) do not
+ * use them. */
 typedef struct {
     int tile_x, tile_y, zseg, graph_chunk;
     int depth, pair_zseg;

@@ -28,6 +28,7 @@
 
 #include "../../include/fdtd.h"
 #include "fdtd_internal.h"
+#include "resident_plan.h"
 
 using namespace fdtd;
 
@@ -97,14 +98,23 @@ struct fdtd_ctx {
     fdtd_batch *batch = nullptr;
     // single-board plan and graph
     fdtd_tuning tune{62, 8, 10, 16, 1, 38};
-    bool plan_dirty = true;
-    Plan plan{};
+    bool plan_dirty = true;          // neither plan below holds any more
+    bool plan_ok = false, rplan_ok = false;
+    Plan plan{};                     // tiled launches
     long long *plan_buf = nullptr;   // device [0]=board ptr, then prefixes
     size_t plan_cap = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_chunk = 0;
     cudaGraphExec_t graph2 = nullptr;   // pairs of steps (depth 2)
     int graph2_chunk = 0;
+    ResPlan res{};                      // resident launch, and the plan of its running-DFT update
+    Plan rplan{};
+    long long *rplan_buf = nullptr;
+    size_t rplan_cap = 0;
+    bool ports_in_boxes = true;         // every source and probe edge belongs to a box
+    bool halo = false;                  // a plane of the state was written from outside
+    long long *res_buf = nullptr;
+    size_t res_cap = 0;
     size_t fbytes = 0;                  // bytes of one field component
     double *energy_buf = nullptr;    // partials + 2 outputs
     int energy_n = 0;
@@ -127,6 +137,12 @@ struct fdtd_batch {
     size_t plan_cap = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_chunk = 0;
+    // members stepped by resident launches (the rest step by `plan`)
+    Plan rplan{};
+    long long *rplan_buf = nullptr, *res_buf = nullptr;
+    size_t rplan_cap = 0, res_cap = 0;
+    std::vector<ResPlan> res;
+    int res_chunk = 1, n_active = 0;   // members with steps left when the plans were built
     int prec = -1;
     int grid_cap = 0;
 };
@@ -651,6 +667,7 @@ int upload_board(fdtd_ctx *c)
 
 // Decide the storage scale, upload sources/probes/trace buffers and the
 // descriptor; called once before the first step.
+std::vector<ResAt> res_ports(const fdtd_ctx *c);
 int finalize(fdtd_ctx *c)
 {
     if (c->started) return FDTD_OK;
@@ -698,6 +715,7 @@ int finalize(fdtd_ctx *c)
         c->h.trace = tr;
         c->h.dft = dft;
     }
+    for (const ResAt &a : res_ports(c)) c->ports_in_boxes = c->ports_in_boxes && res_box_of(c->h, a.i, a.j, a.k) >= 0;
     c->started = true;
     c->plan_dirty = true;
     return upload_board(c);
@@ -819,20 +837,20 @@ long long dft_items(const Board &h)
 }
 
 // Lay out plan arrays [boards | int_prefix | zp_prefix | slab_prefix | dft_prefix | work | slab blocks] in buf.
-int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &t, long long *&buf, size_t &cap,
+int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &t, bool tiled, long long *&buf, size_t &cap,
                Plan &plan, cudaStream_t st, std::vector<long long> &host)
 {
     const int nb = (int)boards.size();
-    for (int b = 0; b < nb; ++b)
+    for (int b = 0; b < nb && tiled; ++b)
         if (!fused_maps_match(boards[b]->h, t.tile_x, t.tile_y))
             return fail(FDTD_EINVAL, "fused tile " + std::to_string(t.tile_x) + "x" + std::to_string(t.tile_y) +
                                          " does not match the board's tensor maps (" +
                                          std::to_string(boards[b]->h.tm_tx) + "x" + std::to_string(boards[b]->h.tm_ty) +
                                          "); nothing was launched");
     long long n_slab_blk = 0;
-    for (int b = 0; b < nb; ++b) n_slab_blk += boards[b]->h.slab_blocks;
+    for (int b = 0; b < nb && tiled; ++b) n_slab_blk += boards[b]->h.slab_blocks;
     // a single board's band blocks follow its slab blocks (second step of a pair)
-    const bool band = nb == 1 && boards[0]->h.pair_ok && boards[0]->h.n_band > 0;
+    const bool band = tiled && nb == 1 && boards[0]->h.pair_ok && boards[0]->h.n_band > 0;
     if (band) n_slab_blk += boards[0]->h.band_blocks;
     static_assert(sizeof(SlabBlock) == 4 * sizeof(long long), "slab block descriptor layout");
     const size_t head = ((size_t)nb + 4 * ((size_t)nb + 1) + 2 + 1) & ~(size_t)1;   // + four work counters, 16-byte aligned
@@ -850,10 +868,11 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &t, long
     for (int b = 0; b < nb; ++b) {
         const Board &h = boards[b]->h;
         ptrs[b] = (long long)(uintptr_t)boards[b]->d;
+        dp[b + 1] = dp[b] + dft_items(h);
+        if (!tiled) continue;   // a plan for resident launches: boards and DFT items only
         ip[b + 1] = ip[b] + fused_items(h, t, false);
         zp[b + 1] = zp[b] + fused_items(h, t, true);
         sp[b + 1] = sp[b] + h.slab_blocks;
-        dp[b + 1] = dp[b] + dft_items(h);
         const int ns = h.n_slab + (band ? h.n_band : 0);
         for (int s = 0; s < ns; ++s) {
             const int end = s + 1 < ns ? (int)h.slab[s + 1].block0 : h.slab_blocks + (band ? h.band_blocks : 0);
@@ -918,6 +937,139 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &t, long
     return FDTD_OK;
 }
 
+// Grid points of a board (without the row padding).
+long long grid_points(const Board &h) { return (long long)(h.nx + 1) * (h.ny + 1) * (h.nz + 1); }
+
+// Boards up to this many grid points are stepped by resident launches.  Past
+// L2 (about 4 M points) their two passes move 73 B per node and step against
+// the tiled launches' 49, but without those launches' tails and slab launches.
+constexpr long long kResPoints = 24LL << 20;
+
+std::vector<ResAt> res_ports(const fdtd_ctx *c)
+{
+    std::vector<ResAt> at;
+    for (size_t s = 0; s < c->src.size(); ++s) at.push_back({c->src[s].i, c->src[s].j, c->src[s].k, c->src[s].comp, 0, (int)s});
+    for (size_t p = 0; p < c->probe.size(); ++p)
+        at.push_back({c->probe[p].i, c->probe[p].j, c->probe[p].k, c->probe[p].comp, 1, (int)p});
+    return at;
+}
+
+// Whether n steps of a board go to resident launches.  The limits on ports and
+// extents bound their shared-memory tables; a probe on a high wall plane lies in
+// no box; and a plane written from outside (fdtd_halo_unpack, _copy) may be a
+// wall plane no step writes, whose two sets then differ, so steps that work in
+// place may not follow.
+bool resident_board(const fdtd_ctx *c, long long n)
+{
+    const Board &h = c->h;
+    return c->prec == FDTD_FP32 && !h.pair_ok && grid_points(h) <= kResPoints && 6 * h.nodes < (1LL << 31) &&
+           c->ports_in_boxes && c->src.size() + c->probe.size() <= 1024 && h.nx + h.ny + h.nz <= 3000 && (n <= 1 || !c->halo);
+}
+
+// Upload a resident plan ([arrival counters | teams | blocks | pieces | ports]).
+int upload_resident(const ResHost &R, Board *const *dev_boards, long long *&buf, size_t &cap, ResPlan &plan, cudaStream_t st,
+                    std::vector<long long> &host)
+{
+    size_t words = 0;
+    auto put = [&](size_t bytes) { const size_t at = words; words += (bytes + 15) / 16 * 2; return at; };
+    const size_t oa = put(resident_arrive_bytes((int)R.teams.size())), ot = put(R.teams.size() * sizeof(ResTeam)),
+                 ob = put(R.blocks.size() * sizeof(ResBlock)),
+                 op = put(R.pieces.size() * sizeof(ResPiece)), oq = put(R.ports.size() * sizeof(ResPort));
+    host.assign(words, 0);
+    std::memcpy(host.data() + ot, R.teams.data(), R.teams.size() * sizeof(ResTeam));
+    std::memcpy(host.data() + ob, R.blocks.data(), R.blocks.size() * sizeof(ResBlock));
+    std::memcpy(host.data() + op, R.pieces.data(), R.pieces.size() * sizeof(ResPiece));
+    if (!R.ports.empty()) std::memcpy(host.data() + oq, R.ports.data(), R.ports.size() * sizeof(ResPort));
+    if (words > cap) {
+        if (buf) cudaFree(buf);
+        buf = nullptr;
+        cap = 0;
+        if (cudaMalloc(&buf, words * sizeof(long long)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(FDTD_ENOMEM, "plan allocation failed");
+        }
+        cap = words;
+    }
+    CK(cudaMemcpyAsync(buf, host.data(), words * sizeof(long long), cudaMemcpyHostToDevice, st));
+    plan.n_teams = plan.all_teams = (int)R.teams.size();
+    plan.n_blocks = (int)R.blocks.size();
+    plan.boards = dev_boards;
+    plan.arrive = (unsigned *)(buf + oa);
+    plan.teams = (const ResTeam *)(buf + ot);
+    plan.blocks = (const ResBlock *)(buf + ob);
+    plan.pieces = (const ResPiece *)(buf + op);
+    plan.ports = (const ResPort *)(buf + oq);
+    plan.max_pieces = R.max_pieces;
+    plan.max_ports = R.max_ports;
+    plan.max_factors = R.max_factors;
+    return FDTD_OK;
+}
+
+// One resident launch over a single board.
+int build_resident(fdtd_ctx *c, Board *const *dev_boards, long long *&buf, size_t &cap, ResPlan &plan, cudaStream_t st,
+                   std::vector<long long> &host)
+{
+    int dev = 0, sms = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    ResHost R;
+    res_team(c->h, res_ports(c), 0, sms, R);
+    return upload_resident(R, dev_boards, buf, cap, plan, st, host);
+}
+
+// L2 bytes a board's steps keep in use: one field set, ids and auxiliaries.
+double res_bytes(const fdtd_ctx *c)
+{
+    double b = 25.0 * grid_points(c->h) + 12.0 * (c->zaux_n[0] + c->zaux_n[1]);
+    for (int s = 0; s < c->h.n_slab; ++s)
+        for (int a = 0; a < 6; ++a)
+            if (c->h.slab[s].aux[a]) b += 4.0 * c->h.slab[s].n;
+    return b;
+}
+
+// State of a group of boards that one resident launch works (measured on 24
+// boards of 0.6 to 4 M cells: 30, 60, 90, 120, 200 MB gave 637, 632, 629, 668,
+// 732 us a step).
+constexpr double kResGroupBytes = 90e6;
+
+// Resident launches of a batch: a launch works one group of boards (res_groups),
+// its blocks shared out by the boards' work, and the launches take turns every
+// `chunk` steps.
+int build_resident_batch(const std::vector<fdtd_ctx *> &boards, Board *const *dev_boards, long long *&buf, size_t &cap,
+                         std::vector<ResPlan> &plans, cudaStream_t st, std::vector<long long> &host)
+{
+    int dev = 0, sms = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    std::vector<double> bytes;
+    for (const fdtd_ctx *c : boards) bytes.push_back(res_bytes(c));
+    const std::vector<std::vector<int>> group = res_groups(bytes, kResGroupBytes, sms);
+    ResHost R;
+    plans.assign(group.size(), ResPlan{});
+    for (size_t g = 0; g < group.size(); ++g) {
+        std::vector<double> work;
+        for (int m : group[g]) work.push_back(res_work(boards[m]->h));
+        const std::vector<int> n = res_share(work, sms);
+        plans[g].n_blocks = -(int)R.blocks.size();
+        plans[g].n_teams = -(int)R.teams.size();
+        for (size_t t = 0; t < n.size(); ++t) res_team(boards[group[g][t]]->h, res_ports(boards[group[g][t]]), group[g][t], n[t], R);
+        plans[g].n_blocks += (int)R.blocks.size();
+        plans[g].n_teams += (int)R.teams.size();
+    }
+    ResPlan all{};
+    if (int r = upload_resident(R, dev_boards, buf, cap, all, st, host)) return r;
+    int blk = 0;
+    for (ResPlan &p : plans) {
+        const int nb = p.n_blocks, nt = p.n_teams;
+        p = all;   // (a block names its team by its place among all teams, and so its counter)
+        p.n_blocks = nb;
+        p.blocks = all.blocks + blk;
+        p.n_teams = nt;
+        blk += nb;
+    }
+    return FDTD_OK;
+}
+
 // NVTX range over a host-side call, for profiler timelines (no cost without a tool attached).
 struct NvtxRange {
     explicit NvtxRange(const char *name) { nvtxRangePushA(name); }
@@ -957,6 +1109,21 @@ int run_steps(const Plan &plan, int prec, int grid_cap, int n, int chunk, cudaGr
     }
     return FDTD_OK;
 }
+
+// Run n steps by resident launches of up to `chunk` steps, then the running-DFT
+// update.
+int run_resident(const ResPlan *res, int n_res, const Plan &plan, int grid_cap, int n, int chunk, cudaStream_t st)
+{
+    if (n <= 0) return FDTD_OK;
+    NvtxRange range(plan.nb > 1 ? "fdtd batch steps" : "fdtd steps");
+    for (int left = n; left > 0; left -= chunk)
+        for (int g = 0; g < n_res; ++g) CK(launch_resident(res[g], std::min(left, chunk), st));
+    CK(launch_dft(plan, grid_cap, st));
+    return FDTD_OK;
+}
+// Steps of one resident launch: up to about a millisecond of work; an odd
+// count, so that the set a launch starts from is the one it works in.
+int resident_chunk(long long nodes) { return (int)std::min<long long>(255, std::max<long long>(15, (1LL << 27) / nodes)) | 1; }
 
 // Run n steps of a depth-2 single-board plan: a single step to reach an even
 // step, then pairs (CUDA graphs of chunk / 2 pairs), then one or two single
@@ -1192,6 +1359,7 @@ int fdtd_create(const fdtd_grid *grid, const uint8_t *mat_ids, const double *eps
     static bool smem_limits = false;
     if (!smem_limits) {
         cudaError_t e = fused_set_smem_limits();
+        if (e == cudaSuccess) e = resident_set_smem_limit();
         if (e != cudaSuccess) { cudaGetLastError(); return fail(FDTD_ECUDA, std::string("fused kernel shared memory: ") + cudaGetErrorString(e)); }
         smem_limits = true;
     }
@@ -1418,15 +1586,19 @@ int fdtd_set_tuning(fdtd_ctx *c, const fdtd_tuning *t)
     return FDTD_OK;
 }
 
-static int prepare_single(fdtd_ctx *c);
+static int prepare_single(fdtd_ctx *c, bool tiled);
 
 int fdtd_step(fdtd_ctx *c, int n)
 {
     if (!c) return fail(FDTD_EINVAL, "NULL context");
     if (n < 0) return fail(FDTD_EINVAL, "n must be >= 0");
     if (c->batch) return fail(FDTD_ESTATE, "context is in a batch; step the batch");
-    if (int r = prepare_single(c)) return r;
-    if (c->h.pair_ok) {
+    if (int r = finalize(c)) return r;
+    const bool resident = resident_board(c, n);
+    if (int r = prepare_single(c, !resident)) return r;
+    if (resident) {
+        if (int r = run_resident(&c->res, 1, c->rplan, c->grid_cap, n, resident_chunk(c->h.nodes), c->cur)) return r;
+    } else if (c->h.pair_ok) {
         if (int r = run_depth2(c->plan, c->prec, c->grid_cap, c->host_step, n, c->tune.graph_chunk, c->graph2,
                                c->graph2_chunk, c->cur))
             return r;
@@ -1437,19 +1609,28 @@ int fdtd_step(fdtd_ctx *c, int n)
     return FDTD_OK;
 }
 
-static int prepare_single(fdtd_ctx *c)
+// Build what the next launches of a single board need: the plan of the tiled
+// launches, or that of the resident launches.
+static int prepare_single(fdtd_ctx *c, bool tiled)
 {
     if (int r = finalize(c)) return r;
     if (int r = encode_maps(c, c->tune.tile_x, c->tune.tile_y)) return r;
-    if (c->plan_dirty) {
-        std::vector<long long> host;
-        std::vector<fdtd_ctx *> one{c};
-        if (int r = build_plan(one, c->tune, c->plan_buf, c->plan_cap, c->plan, c->cur, host)) return r;
-        CK(cudaStreamSynchronize(c->cur));
+    if (c->plan_dirty) c->plan_ok = c->rplan_ok = c->plan_dirty = false;
+    if (tiled ? c->plan_ok : c->rplan_ok) return FDTD_OK;
+    std::vector<long long> host, rhost;
+    const std::vector<fdtd_ctx *> one{c};
+    if (tiled) {
+        if (int r = build_plan(one, c->tune, true, c->plan_buf, c->plan_cap, c->plan, c->cur, host)) return r;
+    } else {
+        if (int r = build_plan(one, c->tune, false, c->rplan_buf, c->rplan_cap, c->rplan, c->cur, host)) return r;
+        if (int r = build_resident(c, c->rplan.boards, c->res_buf, c->res_cap, c->res, c->cur, rhost)) return r;
+    }
+    CK(cudaStreamSynchronize(c->cur));
+    if (tiled) {
         if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
         if (c->graph2) { cudaGraphExecDestroy(c->graph2); c->graph2 = nullptr; }
-        c->plan_dirty = false;
     }
+    (tiled ? c->plan_ok : c->rplan_ok) = true;
     return FDTD_OK;
 }
 
@@ -1458,7 +1639,7 @@ int fdtd_step_profiled(fdtd_ctx *c, int n, double *phase_ms)
     if (!c || !phase_ms) return fail(FDTD_EINVAL, "NULL argument");
     if (n < 0) return fail(FDTD_EINVAL, "n must be >= 0");
     if (c->batch) return fail(FDTD_ESTATE, "context is in a batch; step the batch");
-    if (int r = prepare_single(c)) return r;
+    if (int r = prepare_single(c, true)) return r;
     const size_t need = (size_t)n * (kPairLaunches + 1) + 2;
     while (c->events.size() < need) {
         cudaEvent_t e;
@@ -1627,6 +1808,7 @@ int fdtd_reset(fdtd_ctx *c)
     CK(cudaMemsetAsync(h.dft_done, 0, sizeof(long long), c->cur));
     CK(cudaMemsetAsync(h.status, 0, sizeof(int), c->cur));
     c->host_step = 0;
+    c->halo = false;
     return FDTD_OK;
 }
 
@@ -1638,7 +1820,7 @@ struct CkptHeader {
     int32_t version;
     int32_t nx, ny, nz, pitch, prec, n_probe, n_src, n_total, n_bins, n_slab;
     float scale;
-    int32_t pad;
+    int32_t halo;   // a plane of the state was written from outside
     int64_t nodes, step, dft_done;
     double dt;
 };
@@ -1675,6 +1857,7 @@ CkptHeader ckpt_header(const fdtd_ctx *c)
     H.n_probe = (int)c->probe.size(); H.n_src = (int)c->src.size();
     H.n_total = h.n_total; H.n_bins = h.n_bins; H.n_slab = h.n_slab;
     H.scale = h.scale;
+    H.halo = c->halo ? 1 : 0;
     H.nodes = h.nodes;
     H.dt = c->dt;
     return H;
@@ -1741,6 +1924,7 @@ int fdtd_load(fdtd_ctx *c, const void *buf, size_t size)
     CK(cudaMemsetAsync(c->h.status, 0, sizeof(int), c->cur));
     CK(cudaStreamSynchronize(c->cur));
     c->host_step = H.step;
+    c->halo = H.halo != 0;
     return FDTD_OK;
 }
 
@@ -1817,6 +2001,7 @@ int fdtd_halo_unpack(fdtd_ctx *c, int axis, int plane, unsigned comp_mask, const
     if (int r = check_halo(c, axis, plane, comp_mask, g)) return r;
     if (!dev_buf) return fail(FDTD_EINVAL, "NULL buffer");
     if (int r = finalize(c)) return r;
+    c->halo = true;
     const size_t es = elem_size(c->prec);
     const int par = set_of(c->h.tdepth, c->host_step);
     const unsigned char *in = static_cast<const unsigned char *>(dev_buf);
@@ -1843,6 +2028,7 @@ int fdtd_halo_copy(fdtd_ctx *dst, int dst_plane, fdtd_ctx *src, int src_plane, i
     if (int r = finalize(dst)) return r;
     if (int r = finalize(src)) return r;
     if (src->h.scale != dst->h.scale) return fail(FDTD_EINVAL, "the two contexts use different storage scales");
+    dst->halo = true;
     // the copy runs on the destination's stream once the source's queued work is done
     cudaEvent_t ev = nullptr;
     CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -2023,6 +2209,8 @@ void fdtd_destroy(fdtd_ctx *c)
     if (c->graph) cudaGraphExecDestroy(c->graph);
     if (c->graph2) cudaGraphExecDestroy(c->graph2);
     if (c->plan_buf) cudaFree(c->plan_buf);
+    if (c->rplan_buf) cudaFree(c->rplan_buf);
+    if (c->res_buf) cudaFree(c->res_buf);
     for (cudaEvent_t e : c->events) cudaEventDestroy(e);
     for (void *p : c->allocs) cudaFree(p);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -2099,6 +2287,37 @@ int fdtd_batch_remove(fdtd_batch *b, fdtd_ctx *c)
     return FDTD_OK;
 }
 
+// Plans of a batch: members with steps left that resident launches work, and
+// the others for the tiled launches.
+static int prepare_batch(fdtd_batch *b)
+{
+    std::vector<fdtd_ctx *> res, tiled;
+    double work = 0.0;
+    for (size_t m = 0; m < b->members.size(); ++m) {
+        fdtd_ctx *c = b->members[m];
+        if (b->remaining[m] <= 0) continue;
+        const bool r = resident_board(c, 2);
+        (r ? res : tiled).push_back(c);
+        if (r) work += (double)c->h.nodes;
+    }
+    std::vector<long long> host, rhost, rhost2;
+    for (fdtd_ctx *m : tiled)
+        if (int r = encode_maps(m, b->tune.tile_x, b->tune.tile_y)) return r;
+    b->plan.nb = 0;
+    b->res.clear();
+    if (!tiled.empty())
+        if (int r = build_plan(tiled, b->tune, true, b->plan_buf, b->plan_cap, b->plan, b->stream, host)) return r;
+    if (!res.empty()) {
+        if (int r = build_plan(res, b->tune, false, b->rplan_buf, b->rplan_cap, b->rplan, b->stream, rhost)) return r;
+        if (int r = build_resident_batch(res, b->rplan.boards, b->res_buf, b->res_cap, b->res, b->stream, rhost2)) return r;
+        b->res_chunk = resident_chunk((long long)(work / (double)b->res.size()) + 1);
+    }
+    CK(cudaStreamSynchronize(b->stream));
+    if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
+    b->dirty = false;
+    return FDTD_OK;
+}
+
 int fdtd_batch_step(fdtd_batch *b, int n, int *n_done)
 {
     if (!b) return fail(FDTD_EINVAL, "NULL batch");
@@ -2107,18 +2326,18 @@ int fdtd_batch_step(fdtd_batch *b, int n, int *n_done)
     for (long long r : b->remaining) most = std::max(most, r);
     const int run = (int)std::min<long long>(n, most);
     if (run > 0 && !b->members.empty()) {
-        if (b->dirty) {
-            for (fdtd_ctx *m : b->members)
-                if (int r = encode_maps(m, b->tune.tile_x, b->tune.tile_y)) return r;
-            std::vector<long long> host;
-            if (int r = build_plan(b->members, b->tune, b->plan_buf, b->plan_cap, b->plan, b->stream, host)) return r;
-            CK(cudaStreamSynchronize(b->stream));
-            if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
-            b->dirty = false;
+        int active = 0;
+        for (long long r : b->remaining) active += r > 0;
+        if (b->dirty || active != b->n_active) {
+            if (int r = prepare_batch(b)) return r;
+            b->n_active = active;
         }
-        if (int r = run_steps(b->plan, b->prec, b->grid_cap, run, b->tune.graph_chunk, b->graph, b->graph_chunk,
-                              b->stream))
-            return r;
+        if (!b->res.empty())
+            if (int r = run_resident(b->res.data(), (int)b->res.size(), b->rplan, b->grid_cap, run, b->res_chunk, b->stream))
+                return r;
+        if (b->plan.nb > 0)
+            if (int r = run_steps(b->plan, b->prec, b->grid_cap, run, b->tune.graph_chunk, b->graph, b->graph_chunk, b->stream))
+                return r;
         for (size_t m = 0; m < b->members.size(); ++m) {
             const long long did = std::min<long long>(run, b->remaining[m]);
             b->remaining[m] -= did;
@@ -2162,6 +2381,8 @@ void fdtd_batch_destroy(fdtd_batch *b)
     }
     if (b->graph) cudaGraphExecDestroy(b->graph);
     if (b->plan_buf) cudaFree(b->plan_buf);
+    if (b->rplan_buf) cudaFree(b->rplan_buf);
+    if (b->res_buf) cudaFree(b->res_buf);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     cudaGetLastError();
     delete b;

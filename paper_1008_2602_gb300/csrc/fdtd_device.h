@@ -1,0 +1,127 @@
+// fdtd_device.h -- device arithmetic shared by the kernel files: storage
+// access, curls, the UPML component updates, sources.  A value computed by
+// any kernel goes through these (or forms that round alike), so every path
+// gives the same bits.
+#pragma once
+
+#include <cuda_fp16.h>
+
+#include "fdtd_internal.h"
+
+namespace fdtd {
+
+// ------------------------------------------------------------------ storage
+template <typename T>
+struct Io;
+template <>
+struct Io<float> {
+    static __device__ __forceinline__ float ld(const float *p) { return __ldg(p); }
+    static __device__ __forceinline__ float ldw(const float *p) { return *p; }
+    static __device__ __forceinline__ void st(float *p, float v) { *p = v; }
+};
+template <>
+struct Io<__half> {
+    static __device__ __forceinline__ float ld(const __half *p) { return __half2float(__ldg(p)); }
+    static __device__ __forceinline__ float ldw(const __half *p) { return __half2float(*p); }
+    static __device__ __forceinline__ void st(__half *p, float v) { *p = __float2half_rn(v); }
+};
+
+// ------------------------------------------------------------------ arithmetic
+// Sa (a1 - a0) - Sb (b1 - b0): one component of S * curl.
+__device__ __forceinline__ float curl2(float a1, float a0, float b1, float b0, float Sa, float Sb)
+{
+    return __fmaf_rn(-Sb, __fsub_rn(b1, b0), __fmul_rn(Sa, __fsub_rn(a1, a0)));
+}
+
+// Eq. 8 pulse of a source at the half step n + 1/2: J for a current source,
+// Vs for a voltage source.
+__device__ __forceinline__ double src_pulse(const Source &S, long long step, double dt)
+{
+    const double t = ((double)step + 0.5) * dt;
+    const double u = (t - S.t0) / S.tau;
+    return S.J0 * u * exp(-u * u);
+}
+
+// A source applied to the plainly updated edge value ep (as stored), given the
+// edge's previous value en (as stored); returns the new value before storage
+// rounding.  Current source: E -= coef J.  Resistive voltage source: the lumped
+// current (l E^{n+1/2} + Vs) / Rs in Ampere's law turns the plain update
+// E_p = E^n + ce S curl into E^{n+1} = (E_p - beta E^n - gam Vs) / (1 + beta).
+__device__ __forceinline__ float src_apply(const Source &S, double w, float ep, float en)
+{
+    if (S.kind == kSrcCurrent) return __fsub_rn(ep, (float)(S.coef * w));
+    return (float)(((double)ep - S.beta * (double)en - S.gam * w) / (1.0 + S.beta));
+}
+
+// Gedney two-step update of one H~ component (B~ recurrence along w+1, H~
+// recurrence along w+2, B~->H~ along w).  scurl = S * (curl E)_w.  Bo/Bn are
+// the old/new auxiliaries (no auxiliary: pass aux == false).
+__device__ __forceinline__ float upml_h2(float h, float scurl, const Coef &a, const Coef &bb, const Coef &c, bool aux,
+                                         float Bo, float &Bn)
+{
+    if (aux) {
+        Bn = __fmaf_rn(-a.g, scurl, __fmul_rn(a.b1, Bo));
+        return __fmaf_rn(bb.g, __fmaf_rn(c.ap, Bn, -__fmul_rn(c.am, Bo)), __fmul_rn(bb.b1, h));
+    }
+    // no auxiliary: c is trivial and at most one of a, bb is graded, so the
+    // products below are exact
+    return __fmaf_rn(-__fmul_rn(a.g, bb.g), scurl, __fmul_rn(__fmul_rn(a.b1, bb.b1), h));
+}
+
+// Same for E (D~ along w+1, E along w+2, D~->E along w); ce = 1/eps_r.
+__device__ __forceinline__ float upml_e2(float e, float scurl, float ce, const Coef &a, const Coef &bb, const Coef &c,
+                                         bool aux, float Do, float &Dn)
+{
+    if (aux) {
+        Dn = __fmaf_rn(a.g, scurl, __fmul_rn(a.b1, Do));
+        return __fmaf_rn(__fmul_rn(ce, bb.g), __fmaf_rn(c.ap, Dn, -__fmul_rn(c.am, Do)), __fmul_rn(bb.b1, e));
+    }
+    // no auxiliary (see upml_h2)
+    return __fmaf_rn(__fmul_rn(ce, __fmul_rn(a.g, bb.g)), scurl, __fmul_rn(__fmul_rn(a.b1, bb.b1), e));
+}
+
+// Two adjacent elements of one row (8-byte aligned for FP32, 4-byte for the
+// 16-bit storage types), converted to/from FP32.
+template <typename T>
+struct Pair;
+template <>
+struct Pair<float> {
+    static __device__ __forceinline__ float2 lds(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+    static __device__ __forceinline__ float2 ldg(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
+    static __device__ __forceinline__ void st(float *p, float2 v) { *reinterpret_cast<float2 *>(p) = v; }
+};
+template <>
+struct Pair<__half> {
+    static __device__ __forceinline__ float2 lds(const __half *p)
+    {
+        return __half22float2(*reinterpret_cast<const __half2 *>(p));
+    }
+    static __device__ __forceinline__ float2 ldg(const __half *p)
+    {
+        return __half22float2(__ldg(reinterpret_cast<const __half2 *>(p)));
+    }
+    static __device__ __forceinline__ void st(__half *p, float2 v) { *reinterpret_cast<__half2 *>(p) = __float22half2_rn(v); }
+};
+
+// Paired forms of curl2 and of h - s.  Per element they round exactly like
+// the scalar forms: a - b == fma(b, -1, a) (the product is exact), and
+// fma(-Sb, d, x) is the same single rounding either way.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float2 curl2v(float2 a1, float2 a0, float2 b1, float2 b0, float2 Sa, float2 nSb)
+{
+    return __ffma2_rn(nSb, sub2(b1, b0), __fmul2_rn(Sa, sub2(a1, a0)));
+}
+
+// One row of a 1D UPML factor table through the read-only cache (the
+// tables are 16-byte aligned, one Coef per position).
+__device__ __forceinline__ Coef ldcoef(const Coef *p)
+{
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+    return Coef{v.x, v.y, v.z, v.w};
+}
+
+// Factor of the image of tangential H~ across an outer wall for a neighbour
+// `outside` the grid (PMC: odd mirror, -1; PEC: 0).
+__device__ __forceinline__ float hsign(bool outside, int wall) { return outside ? (wall == 1 ? -1.0f : 0.0f) : 1.0f; }
+
+}  // namespace fdtd

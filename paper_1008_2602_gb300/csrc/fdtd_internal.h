@@ -249,6 +249,53 @@ struct Plan {
     PairConst pc;
 };
 
+// Plan of a resident launch (k_resident): one team of blocks per board.  A
+// board's boxes (slab boxes, z-UPML boxes, interior) are cut into pieces, runs
+// of column quads (four nodes of a row) of one box, shared out to the team's
+// blocks; a unit is 32 quads.
+struct ResPiece {
+    int box;                      // slab index, or n_slab + 0, 1, 2: z-UPML below, above, interior
+    int t0, nq;                   // first quad in the box (x, then y, then z) and count
+    int unit0;                    // units of the block before this piece
+};
+struct ResPort {                  // a source or a probe of a block, in the board's order
+    int unit;                     // unit of the block
+    short lane, col;              // lane and node of its quad
+    short comp, probe;
+    int index;                    // in Board::src or Board::probe
+};
+struct ResTeam {
+    int board, n_blocks;
+};
+struct ResBlock {
+    int team, first;              // first block of its team
+    int piece0, n_piece, port0, n_port;
+};
+struct ResPlan {
+    int n_teams, n_blocks, all_teams;
+    Board *const *boards;
+    const ResTeam *teams;
+    const ResBlock *blocks;
+    const ResPiece *pieces;
+    const ResPort *ports;
+    int max_pieces, max_ports, max_factors;   // of a block
+    unsigned *arrive;             // arrivals per team (zeroed before every launch)
+};
+// Length of a UPML factor array in a block's shared memory (n + 1 positions, whole quads).
+__host__ __device__ inline int res_fac_len(int n) { return (n + 1 + 3) & ~3; }
+// Quotients by a fixed divisor d >= 1 for 0 <= t < 2^31: q = (umulhi(t, m) + t) >> s.
+__host__ __device__ inline void res_recip(int d, unsigned &m, int &s)
+{
+    s = 0;
+    while ((1ull << s) < (unsigned long long)d) ++s;
+    m = (unsigned)((((1ull << s) - (unsigned)d) << 32) / (unsigned)d) + 1u;
+}
+__host__ __device__ inline int res_quot(int t, unsigned m, int s)
+{
+    return (int)(((unsigned)(((unsigned long long)(unsigned)t * m) >> 32) + (unsigned)t) >> s);
+}
+constexpr int kResSmem = 200 << 10;   // shared memory a resident launch may ask for
+
 // TMA descriptor slots of a board (3D maps: x, y, plane).
 __host__ __device__ constexpr int tm_e(int set, int c) { return set * 3 + c; }               // E   box_e  x (TY+2)
 __host__ __device__ constexpr int tm_h(int set, int c) { return 9 + set * 3 + c; }           // H   box_h  x (TY+1)
@@ -299,6 +346,10 @@ constexpr int kPairPhase[kPairLaunches] = {kPhaseSlabH, kPhaseFusedZ, kPhaseInte
                                            kPhaseSlabH, kPhaseFusedZ, kPhaseSlabE,    kPhasePost};
 cudaError_t launch_pair(const Plan &plan, int prec, int grid_cap, cudaStream_t st);
 cudaError_t launch_pair_part(const Plan &plan, int prec, int idx, int grid_cap, cudaStream_t st);
+size_t resident_smem(const ResPlan &plan);
+size_t resident_arrive_bytes(int n_teams);
+cudaError_t resident_set_smem_limit();
+cudaError_t launch_resident(const ResPlan &plan, int nsteps, cudaStream_t st);
 cudaError_t launch_dft(const Plan &plan, int grid_cap, cudaStream_t st);
 cudaError_t launch_set_i64(long long *p, long long v, cudaStream_t st);
 cudaError_t launch_energy(const Board *b_dev, const Board &b_host, double *partials, int n_part,

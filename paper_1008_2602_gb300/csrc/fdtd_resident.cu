@@ -1,0 +1,716 @@
+// fdtd_resident.cu -- many leapfrog steps in one launch (Model section:
+// H^{n+1/2} from E^n, then E^{n+1} from H and J; Eqs. 1-5 in the UPML; Eq. 8
+// sources; probe samples).
+//
+// What bounds a small board in the launch-per-phase path is its chain of
+// dependent launches: five per step, each a chain of plane or node marches,
+// 56-62 us a step on boards of 25 k to 250 k cells whatever their size.
+// k_resident is one cooperative launch for many steps: every block keeps the
+// same nodes for all of them, a step is an H phase and an E phase, and a
+// barrier ends each (1.2 us measured over 152 blocks).  Nothing is recomputed
+// and nothing is staged: all reads of a phase are of values the phases before
+// it finished, so every warp issues its loads at once and L2 serves them
+// (12-13.7 TB/s measured up to 90 MB); there a phase is bound by L2 latency
+// (small boards) or L2 bandwidth, past L2 by HBM at 73 B a node and step.
+//
+// Measured (us a step, launch-per-phase path -> here): 38x33x20 57 -> 5.9,
+// 56x48x30 62 -> 6.2, 181x131x6 34 -> 6.7, 232x192x39 90 -> 22.7, 280x230x100
+// 160 -> 96, 480x380x100 294 -> 261; a batch of 24 boards (41 M cells) 852 ->
+// 629.  At 880x680x100 the tiled launches' 49 B a node win (697 against 902).
+//
+// The work is cut into units of 32 column quads (128 nodes), taken in x, y, z
+// order from one box at a time.  The boxes are the board's own (slab boxes,
+// the two z-UPML boxes of the fused region, the interior), because a box
+// decides which auxiliaries its nodes carry and where they lie; the update of
+// a node is the arithmetic of the launch-per-phase kernels, so the fields,
+// auxiliaries and traces come out bit for bit the same and a board may change
+// between the two at any step.
+#include "fdtd_device.h"
+
+namespace fdtd {
+
+namespace {
+
+// Graded: UPML factors along some axis.  GradedX: along x.  Walls: the box
+// touches an outer wall.  Whole: its quads lie whole inside it, and so do
+// those of its auxiliary arrays (16-byte accesses).  Parity: B~z alternates
+// between two arrays.
+enum : int { kGraded = 1, kGradedX = 2, kWalls = 4, kWhole = 8, kParity = 16 };
+
+struct BoxS {     // one box of the board
+    float *aux[6];          // auxiliary read and written (nullptr: none)
+    float *zb[2];           // z-UPML boxes: B~z by step parity (replaces aux[5])
+    int flags;
+    int i0, i1, ie;         // ie: i0 rounded down to a whole quad
+    int j0, k0;
+    int np, nj;             // quads per row, rows per plane
+    unsigned mp, mj;        // reciprocals of np and nj
+    int sp, sj;
+    int apitch;             // row pitch of the auxiliaries (nj rows per plane)
+    int pad;
+};
+
+struct BoardS {   // the block's board, in shared memory
+    float *f[3];                // field sets: six components, NN nodes apart
+    const void *cid;
+    const float4 *ctab;         // rows of 1 / eps_r for 16-bit ids (the block keeps a copy of those of 8-bit ids)
+    const Source *src;
+    float *trace;
+    int *status;
+    double dt;
+    long long step0;
+    float scale;
+    int n_total;
+    int X, P, NN, id16;         // strides of a row, a plane and a component
+    int nact;                   // steps this launch advances the board
+    int first, work, last;      // field sets: read by the first step, kept in place between, written by the last
+    int n[3];
+    int wall[6];
+    float S[3];
+    int fac[3][2];              // UPML factors in shared memory: float offset per axis and position
+    int row;                    // coefficient rows in shared memory: byte offset
+    int port, n_port, pulse;
+    BoxS box[kMaxSlab + 3];
+};
+
+extern __shared__ __align__(16) unsigned char smem[];
+__device__ __forceinline__ BoardS &board_s() { return *reinterpret_cast<BoardS *>(smem); }
+
+constexpr int kResThreads = 512, kWarps = kResThreads / 32;
+
+struct F4 {       // four neighbouring nodes of a row
+    float2 a, b;
+};
+__device__ __forceinline__ float2 two(float x) { return make_float2(x, x); }
+__device__ __forceinline__ F4 four(float x) { return F4{two(x), two(x)}; }
+__device__ __forceinline__ F4 ld4(const float *p)
+{
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    return F4{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ void st4(float *p, const F4 &v, unsigned own)
+{
+    if (own == 15u) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v.a.x, v.a.y, v.b.x, v.b.y);
+    } else {
+        if (own & 1u) p[0] = v.a.x;
+        if (own & 2u) p[1] = v.a.y;
+        if (own & 4u) p[2] = v.b.x;
+        if (own & 8u) p[3] = v.b.y;
+    }
+}
+__device__ __forceinline__ F4 neg4(const F4 &x) { return F4{make_float2(-x.a.x, -x.a.y), make_float2(-x.b.x, -x.b.y)}; }
+__device__ __forceinline__ F4 mul4(const F4 &x, const F4 &y) { return F4{__fmul2_rn(x.a, y.a), __fmul2_rn(x.b, y.b)}; }
+__device__ __forceinline__ F4 fma4(const F4 &x, const F4 &y, const F4 &z)
+{
+    return F4{__ffma2_rn(x.a, y.a, z.a), __ffma2_rn(x.b, y.b, z.b)};
+}
+__device__ __forceinline__ F4 sub4(const F4 &x, const F4 &y) { return F4{sub2(x.a, y.a), sub2(x.b, y.b)}; }
+__device__ __forceinline__ F4 curl4(const F4 &a1, const F4 &a0, const F4 &b1, const F4 &b0, float Sa, float Sb)
+{
+    return F4{curl2v(a1.a, a0.a, b1.a, b0.a, two(Sa), two(-Sb)), curl2v(a1.b, a0.b, b1.b, b0.b, two(Sa), two(-Sb))};
+}
+__device__ __forceinline__ float get(const F4 &v, int q) { return q == 0 ? v.a.x : q == 1 ? v.a.y : q == 2 ? v.b.x : v.b.y; }
+__device__ __forceinline__ void set(F4 &v, int q, float x)
+{
+    if (q == 0) v.a.x = x;
+    else if (q == 1) v.a.y = x;
+    else if (q == 2) v.b.x = x;
+    else v.b.y = x;
+}
+
+// UPML factors of a quad.  The block's copies are four arrays (b1, g, ap, am)
+// per axis and position, so a quad's factors along x are four 16-byte reads
+// and a row's along y or z four scalars.
+struct C4 {
+    F4 b1, g, ap, am;
+};
+__device__ __forceinline__ C4 fac_quad(int at, int n, int i)
+{
+    const float *f = reinterpret_cast<const float *>(smem) + at + i;
+    const int m = res_fac_len(n);
+    return C4{ld4(f), ld4(f + m), ld4(f + 2 * m), ld4(f + 3 * m)};
+}
+__device__ __forceinline__ C4 fac_row(int at, int n, int j)
+{
+    const float *f = reinterpret_cast<const float *>(smem) + at + j;
+    const int m = res_fac_len(n);
+    return C4{four(f[0]), four(f[m]), four(f[2 * m]), four(f[3 * m])};
+}
+__device__ __forceinline__ C4 fac_one() { return C4{four(1.f), four(1.f), four(1.f), four(1.f)}; }
+
+// upml_h2 and upml_e2 on a quad: the same operations, element by element.
+__device__ __forceinline__ F4 upml_h4(const F4 &h, const F4 &sc, const C4 &a, const C4 &b, const C4 &c, bool aux, const F4 &Bo,
+                                      F4 &Bn)
+{
+    if (aux) {
+        Bn = fma4(neg4(a.g), sc, mul4(a.b1, Bo));
+        return fma4(b.g, fma4(c.ap, Bn, neg4(mul4(c.am, Bo))), mul4(b.b1, h));
+    }
+    return fma4(neg4(mul4(a.g, b.g)), sc, mul4(mul4(a.b1, b.b1), h));
+}
+__device__ __forceinline__ F4 upml_e4(const F4 &e, const F4 &sc, const F4 &ce, const C4 &a, const C4 &b, const C4 &c, bool aux,
+                                      const F4 &Do, F4 &Dn)
+{
+    if (aux) {
+        Dn = fma4(a.g, sc, mul4(a.b1, Do));
+        return fma4(mul4(ce, b.g), fma4(c.ap, Dn, neg4(mul4(c.am, Do))), mul4(b.b1, e));
+    }
+    return fma4(mul4(ce, mul4(a.g, b.g)), sc, mul4(mul4(a.b1, b.b1), e));
+}
+
+// Walk of a warp through its units of a piece: quads t0 + 32 u + lane below end.
+struct Walk {
+    int np, nj, ie, i0, i1, apitch;
+    unsigned mp, mj;
+    int sp, sj, at0, row, plane;   // node index of a quad: at0 + 4 p + r row + kk plane (r: row of the box, kk: plane)
+    __device__ __forceinline__ explicit Walk(const BoxS &x)
+    {
+        const BoardS &B = board_s();
+        np = x.np; nj = x.nj; ie = x.ie; i0 = x.i0; i1 = x.i1; apitch = x.apitch;
+        mp = x.mp; mj = x.mj; sp = x.sp; sj = x.sj;
+        at0 = x.k0 * B.P + x.j0 * B.X + x.ie;
+        row = B.X;
+        plane = B.P - x.nj * B.X;
+    }
+};
+struct Pos {
+    int p, r, kk;           // quad of the row, row of the box, plane of the box
+    int at, ax;             // node and auxiliary index
+    unsigned own;           // bit q: node q of the quad belongs to the box
+};
+__device__ __forceinline__ Pos locate(const Walk &w, int t, int end, bool whole)
+{
+    Pos q;
+    const bool live = t < end;
+    t = min(t, end - 1);
+    q.r = res_quot(t, w.mp, w.sp);
+    q.p = t - q.r * w.np;
+    q.kk = res_quot(q.r, w.mj, w.sj);
+    q.at = w.at0 + 4 * q.p + q.r * w.row + q.kk * w.plane;
+    q.own = 15u;
+    if (!whole) {
+        const int i = w.ie + 4 * q.p;
+        q.own = (15u << max(w.i0 - i, 0)) & (15u >> max(i + 4 - w.i1, 0));
+    }
+    if (!live) q.own = 0;
+    q.ax = q.r * w.apitch + 4 * q.p + (w.ie - w.i0);
+    return q;
+}
+
+// Auxiliaries of a quad (only the box's own nodes lie in the array).
+__device__ __forceinline__ F4 ldaux(const float *p, const Pos &q, bool whole)
+{
+    if (!p) return four(0.f);
+    p += q.ax;
+    if (whole) return ld4(p);
+    F4 v = four(0.f);
+    if (q.own & 1u) v.a.x = p[0];
+    if (q.own & 2u) v.a.y = p[1];
+    if (q.own & 4u) v.b.x = p[2];
+    if (q.own & 8u) v.b.y = p[3];
+    return v;
+}
+__device__ __forceinline__ void staux(float *p, const Pos &q, const F4 &v, unsigned own, bool whole)
+{
+    if (!p) return;
+    p += q.ax;
+    if (whole) {
+        if (own) *reinterpret_cast<float4 *>(p) = make_float4(v.a.x, v.a.y, v.b.x, v.b.y);
+        return;
+    }
+    if (own & 1u) p[0] = v.a.x;
+    if (own & 2u) p[1] = v.a.y;
+    if (own & 4u) p[2] = v.b.x;
+    if (own & 8u) p[3] = v.b.y;
+}
+
+// Auxiliary array of component c of a box, read from shared memory at each use
+// (held in registers, the six pointers of a graded box would spill); B~z of the
+// z-UPML boxes by parity.
+__device__ __forceinline__ float *aux_of(const BoxS &x, int c, int par = -1)
+{
+    unsigned long long v;
+    float *const *p = par >= 0 && (x.flags & kParity) ? &x.zb[par] : &x.aux[c];
+    asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"((unsigned)__cvta_generic_to_shared(p)));
+    return (float *)v;
+}
+
+// Nodes of the quad at column i below the last column n (where x-directed samples exist).
+__device__ __forceinline__ unsigned below(int i, int n) { return 15u >> min(max(i + 4 - n, 0), 4); }
+
+// H~^{n+1/2} of the units turn, turn + kWarps, ... < nu of a piece, from field
+// set I into set O.  G: the box is graded or touches an outer wall.
+template <bool G>
+__device__ __forceinline__ void run_h(const BoxS &x, int t0, int end, int turn, int nu, const float *I, float *O, int par)
+{
+    const BoardS &B = board_s();
+    const int lane = threadIdx.x & 31;
+    const Walk w(x);
+    const bool whole = (x.flags & kWhole) != 0, GX = (x.flags & kGradedX) != 0;
+    const int X = B.X, P = B.P, N = B.NN;
+    for (int u = turn; u < nu; u += kWarps) {
+        const Pos q = locate(w, t0 + 32 * u + lane, end, whole);
+        const int at = q.at;
+        // neighbours past the grid's last column, row or plane read the next
+        // component's memory: in bounds, and used only by nodes that are not stored
+        const F4 ex = ld4(I + at), ey = ld4(I + (at + N)), ez = ld4(I + (at + 2 * N));
+        const float eyi = I[at + N + 4], ezi = I[at + 2 * N + 4];
+        const F4 exj = ld4(I + (at + X)), ezj = ld4(I + (at + 2 * N + X));
+        const F4 exk = ld4(I + (at + P)), eyk = ld4(I + (at + N + P));
+        const F4 ox = ld4(I + (at + 3 * N)), oy = ld4(I + (at + 4 * N)), oz = ld4(I + (at + 5 * N));
+        F4 b0, b1, b2;
+        if (G) {
+            b0 = ldaux(aux_of(x, 3), q, whole);
+            b1 = ldaux(aux_of(x, 4), q, whole);
+            b2 = ldaux(aux_of(x, 5, par), q, whole);
+        }
+        const float Sx = B.S[0], Sy = B.S[1], Sz = B.S[2];
+        const F4 eyr{make_float2(ey.a.y, ey.b.x), make_float2(ey.b.y, eyi)};   // E_y, E_z at i + 1
+        const F4 ezr{make_float2(ez.a.y, ez.b.x), make_float2(ez.b.y, ezi)};
+        const F4 cx = curl4(ezj, ez, eyk, ey, Sy, Sz);
+        const F4 cy = curl4(exk, ex, ezr, ez, Sz, Sx);
+        const F4 cz = curl4(eyr, ey, exj, ex, Sx, Sy);
+        if (!G) {
+            st4(O + (at + 3 * N), sub4(ox, cx), q.own);
+            st4(O + (at + 4 * N), sub4(oy, cy), q.own);
+            st4(O + (at + 5 * N), sub4(oz, cz), q.own);
+            continue;
+        }
+        const int i = w.ie + 4 * q.p, j = x.j0 + q.r - q.kk * w.nj, k = x.k0 + q.kk;
+        unsigned mx = q.own, my = q.own, mz = q.own;
+        if (x.flags & kWalls) {   // samples that exist: not past the last row, column or plane
+            const bool yin = j < B.n[1], zin = k < B.n[2];
+            const unsigned xin = below(i, B.n[0]);
+            if (!(yin && zin)) mx = 0;
+            my = zin ? my & xin : 0u;
+            mz = yin ? mz & xin : 0u;
+        }
+        F4 n;
+        {
+            float *const a = aux_of(x, 3);
+            const F4 h = upml_h4(ox, cx, fac_row(B.fac[1][1], B.n[1], j), fac_row(B.fac[2][1], B.n[2], k),
+                                 GX ? fac_quad(B.fac[0][0], B.n[0], i) : fac_one(), a != nullptr, b0, n);
+            st4(O + (at + 3 * N), h, mx);
+            staux(a, q, n, mx, whole);
+        }
+        {
+            float *const a = aux_of(x, 4);
+            const F4 h = upml_h4(oy, cy, fac_row(B.fac[2][1], B.n[2], k), GX ? fac_quad(B.fac[0][1], B.n[0], i) : fac_one(),
+                                 fac_row(B.fac[1][0], B.n[1], j), a != nullptr, b1, n);
+            st4(O + (at + 4 * N), h, my);
+            staux(a, q, n, my, whole);
+        }
+        {
+            float *const a = aux_of(x, 5, par ^ 1);
+            const F4 h = upml_h4(oz, cz, GX ? fac_quad(B.fac[0][1], B.n[0], i) : fac_one(), fac_row(B.fac[1][1], B.n[1], j),
+                                 fac_row(B.fac[2][0], B.n[2], k), a != nullptr, b2, n);
+            st4(O + (at + 5 * N), h, mz);
+            staux(a, q, n, mz, whole);
+        }
+    }
+}
+
+// Images of tangential H~ across the outer walls: a low wall mirrors the
+// node's own value, a high wall its - neighbour's.
+__device__ __forceinline__ void image(bool lo, bool hi, int wlo, int whi, float &p, float &m)
+{
+    if (hi) p = hsign(true, whi) * m;
+    if (lo) m = hsign(true, wlo) * p;
+}
+__device__ __forceinline__ void image4(bool lo, bool hi, int wlo, int whi, F4 &p, F4 &m)
+{
+    image(lo, hi, wlo, whi, p.a.x, m.a.x);
+    image(lo, hi, wlo, whi, p.a.y, m.a.y);
+    image(lo, hi, wlo, whi, p.b.x, m.b.x);
+    image(lo, hi, wlo, whi, p.b.y, m.b.y);
+}
+
+// E^{n+1} of the units turn, turn - kWarps, ... > stop of a piece: E^n from set
+// I, H~^{n+1/2} from set O, into set O.  PORTS: the units hold sources or probes
+// (unit `base + u` of the block, local step s).
+template <bool G, bool PORTS>
+__device__ __forceinline__ void run_e(const BoxS &x, int t0, int end, int turn, int stop, const float *I, float *O, int s, int base)
+{
+    const BoardS &B = board_s();
+    const int lane = threadIdx.x & 31;
+    const Walk w(x);
+    const bool whole = (x.flags & kWhole) != 0, GX = (x.flags & kGradedX) != 0;
+    const int X = B.X, P = B.P, N = B.NN;
+    const void *const cid = B.cid;
+    const bool id16 = B.id16 != 0;
+    for (int u = turn; u > stop; u -= kWarps) {
+        const Pos q = locate(w, t0 + 32 * u + lane, end, whole);
+        const int at = q.at;
+        uint2 id;
+        if (id16) id = *reinterpret_cast<const uint2 *>((const uint16_t *)cid + at);
+        else id.x = *reinterpret_cast<const unsigned *>((const uint8_t *)cid + at);
+        // neighbours before the grid's first column, row or plane read the
+        // previous component's memory: in bounds, and replaced by the wall's image below
+        const F4 hx = ld4(O + (at + 3 * N)), hy = ld4(O + (at + 4 * N)), hz = ld4(O + (at + 5 * N));
+        const float hyi = O[at + 4 * N - 1], hzi = O[at + 5 * N - 1];
+        F4 hxj = ld4(O + (at + 3 * N - X)), hzj = ld4(O + (at + 5 * N - X));
+        F4 hxk = ld4(O + (at + 3 * N - P)), hyk = ld4(O + (at + 4 * N - P));
+        const F4 ex = ld4(I + at), ey = ld4(I + (at + N)), ez = ld4(I + (at + 2 * N));
+        F4 d0, d1, d2;
+        if (G) {
+            d0 = ldaux(aux_of(x, 0), q, whole);
+            d1 = ldaux(aux_of(x, 1), q, whole);
+            d2 = ldaux(aux_of(x, 2), q, whole);
+        }
+        const float Sx = B.S[0], Sy = B.S[1], Sz = B.S[2];
+        F4 hyl{make_float2(hyi, hy.a.x), make_float2(hy.a.y, hy.b.x)};   // H~y, H~z at i - 1
+        F4 hzl{make_float2(hzi, hz.a.x), make_float2(hz.a.y, hz.b.x)};
+        unsigned mx = q.own, my = q.own, mz = q.own;
+        const int i = w.ie + 4 * q.p, j = x.j0 + q.r - q.kk * w.nj, k = x.k0 + q.kk;
+        F4 cx, cy, cz;
+        if (G && (x.flags & kWalls)) {
+            const int n = B.n[0], w0 = B.wall[0], w1 = B.wall[1];
+            // H~ on the + side of the node, per axis of difference
+            F4 hyx = hy, hzx = hz, hxy = hx, hzy = hz, hxz = hx, hyz = hy;
+            image(i == 0, i == n, w0, w1, hyx.a.x, hyl.a.x);
+            image(i == 0, i == n, w0, w1, hzx.a.x, hzl.a.x);
+            image(false, i + 1 == n, w0, w1, hyx.a.y, hyl.a.y);
+            image(false, i + 1 == n, w0, w1, hzx.a.y, hzl.a.y);
+            image(false, i + 2 == n, w0, w1, hyx.b.x, hyl.b.x);
+            image(false, i + 2 == n, w0, w1, hzx.b.x, hzl.b.x);
+            image(false, i + 3 == n, w0, w1, hyx.b.y, hyl.b.y);
+            image(false, i + 3 == n, w0, w1, hzx.b.y, hzl.b.y);
+            image4(j == 0, j == B.n[1], B.wall[2], B.wall[3], hxy, hxj);
+            image4(j == 0, j == B.n[1], B.wall[2], B.wall[3], hzy, hzj);
+            image4(k == 0, k == B.n[2], B.wall[4], B.wall[5], hxz, hxk);
+            image4(k == 0, k == B.n[2], B.wall[4], B.wall[5], hyz, hyk);
+            mx &= below(i, n);
+            if (j >= B.n[1]) my = 0;
+            if (k >= B.n[2]) mz = 0;
+            cx = curl4(hzy, hzj, hyz, hyk, Sy, Sz);
+            cy = curl4(hxz, hxk, hzx, hzl, Sz, Sx);
+            cz = curl4(hyx, hyl, hxy, hxj, Sx, Sy);
+        } else {
+            cx = curl4(hz, hzj, hy, hyk, Sy, Sz);
+            cy = curl4(hx, hxk, hz, hzl, Sz, Sx);
+            cz = curl4(hy, hyl, hx, hxj, Sx, Sy);
+        }
+        float4 r0, r1, r2, r3;   // 1 / eps_r of the quad's edges
+        if (id16) {
+            const float4 *const r = B.ctab;
+            r0 = __ldg(r + (id.x & 0xffffu)); r1 = __ldg(r + (id.x >> 16));
+            r2 = __ldg(r + (id.y & 0xffffu)); r3 = __ldg(r + (id.y >> 16));
+        } else {
+            const float4 *const r = reinterpret_cast<const float4 *>(smem + B.row);
+            r0 = r[id.x & 0xffu]; r1 = r[(id.x >> 8) & 0xffu]; r2 = r[(id.x >> 16) & 0xffu]; r3 = r[id.x >> 24];
+        }
+        const F4 kx{make_float2(r0.x, r1.x), make_float2(r2.x, r3.x)}, ky{make_float2(r0.y, r1.y), make_float2(r2.y, r3.y)},
+            kz{make_float2(r0.z, r1.z), make_float2(r2.z, r3.z)};
+        F4 nx, ny, nz;
+        if (!G) {
+            nx = fma4(kx, cx, ex);
+            ny = fma4(ky, cy, ey);
+            nz = fma4(kz, cz, ez);
+        } else {
+            F4 n;
+            {
+                float *const a = aux_of(x, 0);
+                nx = upml_e4(ex, cx, kx, fac_row(B.fac[1][0], B.n[1], j), fac_row(B.fac[2][0], B.n[2], k),
+                             GX ? fac_quad(B.fac[0][1], B.n[0], i) : fac_one(), a != nullptr, d0, n);
+                staux(a, q, n, mx, whole);
+            }
+            {
+                float *const a = aux_of(x, 1);
+                ny = upml_e4(ey, cy, ky, fac_row(B.fac[2][0], B.n[2], k), GX ? fac_quad(B.fac[0][0], B.n[0], i) : fac_one(),
+                             fac_row(B.fac[1][1], B.n[1], j), a != nullptr, d1, n);
+                staux(a, q, n, my, whole);
+            }
+            {
+                float *const a = aux_of(x, 2);
+                nz = upml_e4(ez, cz, kz, GX ? fac_quad(B.fac[0][0], B.n[0], i) : fac_one(), fac_row(B.fac[1][0], B.n[1], j),
+                             fac_row(B.fac[2][1], B.n[2], k), a != nullptr, d2, n);
+                staux(a, q, n, mz, whole);
+            }
+        }
+        // sources on edges of this unit, in order (several may share an edge), then probe samples
+        const ResPort *const list = reinterpret_cast<const ResPort *>(smem + B.port);
+        for (int v0 = 0; PORTS && v0 < B.n_port; v0 += 32) {
+            const int mine = v0 + lane;
+            unsigned hit = __ballot_sync(0xffffffffu, mine < B.n_port && list[mine].unit == base + u);
+            for (; hit; hit &= hit - 1) {
+                const int v = v0 + __ffs(hit) - 1;
+                const ResPort &p = list[v];
+                if (p.lane != lane) continue;
+                const int e = p.col;
+                const float now = get(p.comp == 0 ? nx : p.comp == 1 ? ny : nz, e);
+                if (p.probe) {
+                    const float f = now * B.scale;
+                    const long long n = B.step0 + s;
+                    if (n < (long long)B.n_total) B.trace[(long long)p.index * B.n_total + n] = f;
+                    if (!isfinite(f)) atomicOr(B.status, 1);
+                } else {
+                    const double pulse = reinterpret_cast<const double *>(smem + B.pulse)[v];
+                    const float f = src_apply(B.src[p.index], pulse, now, get(p.comp == 0 ? ex : p.comp == 1 ? ey : ez, e));
+                    if (p.comp == 0) set(nx, e, f);
+                    else if (p.comp == 1) set(ny, e, f);
+                    else set(nz, e, f);
+                }
+            }
+        }
+        st4(O + at, nx, mx);
+        st4(O + (at + N), ny, my);
+        st4(O + (at + 2 * N), nz, mz);
+    }
+}
+
+// A unit that holds sources or probes: out of line, so that the others carry none of its state.
+__device__ __noinline__ void port_unit(int bx, int t0, int end, int u, int si, int so, int s, int base)
+{
+    const BoardS &B = board_s();
+    const BoxS &x = B.box[bx];
+    if (x.flags & (kGraded | kWalls)) run_e<true, true>(x, t0, end, u, u - 1, B.f[si], B.f[so], s, base);
+    else run_e<false, true>(x, t0, end, u, u - 1, B.f[si], B.f[so], s, base);
+}
+
+// Shared tables of a block, built from the board's descriptor at the start of
+// a launch (a descriptor may change between launches).
+__device__ void fill_board(const Board *B, BoardS &o, int nsteps)
+{
+    for (int s = 0; s < 3; ++s) o.f[s] = (float *)B->f[s][0];
+    o.n[0] = B->nx; o.n[1] = B->ny; o.n[2] = B->nz;
+    for (int a = 0; a < 3; ++a) o.S[a] = B->S[a];
+    o.cid = B->cid;
+    o.ctab = B->ctab;
+    o.src = B->src;
+    o.trace = B->trace;
+    o.status = B->status;
+    o.dt = B->dt;
+    o.scale = B->scale;
+    o.n_total = B->n_total;
+    o.P = (int)B->plane;
+    o.X = B->pitch;
+    o.NN = (int)B->nodes;
+    o.id16 = B->id16;
+    for (int w = 0; w < 6; ++w) o.wall[w] = B->wall[w];
+    o.step0 = *((volatile long long *)B->step);
+    const long long left = *((volatile long long *)B->stop) - o.step0;
+    o.nact = (int)(left < 0 ? 0 : (left < nsteps ? left : nsteps));
+    // H of a node is written over by its own update alone, and so is E: all
+    // steps but the last work in place in the set that has to hold the state
+    // before the last (for the energy and checkpoints), so one field set and
+    // not two has to stay in L2
+    o.first = set_of(B->tdepth, o.step0);
+    o.work = set_of(B->tdepth, o.step0 + o.nact - 1);
+    o.last = set_of(B->tdepth, o.step0 + o.nact);
+}
+__device__ void fill_box(const Board *B, int kind, BoxS &o)
+{
+    int lo[3], hi[3];
+    for (int c = 0; c < 6; ++c) o.aux[c] = nullptr;
+    o.zb[0] = o.zb[1] = nullptr;
+    o.flags = 0;
+    if (kind < B->n_slab) {
+        const Slab &s = B->slab[kind];
+        lo[0] = s.i0; hi[0] = s.i1; lo[1] = s.j0; hi[1] = s.j1; lo[2] = s.k0; hi[2] = s.k1;
+        for (int c = 0; c < 6; ++c) o.aux[c] = s.aux[c];
+        o.apitch = s.ni;
+        o.flags = kGraded;
+        if (lo[0] < B->depth[0] || hi[0] > B->nx - B->depth[1]) o.flags |= kGradedX;
+    } else {
+        lo[0] = B->ix0; hi[0] = B->ix1; lo[1] = B->iy0; hi[1] = B->iy1;
+        const int z = kind - B->n_slab;   // 0: below, 1: above, 2: between the z-UPML layers
+        lo[2] = z == 0 ? B->zlo : (z == 1 ? max(B->iz1, B->iz0) : B->iz0);
+        hi[2] = z == 0 ? B->iz0 : (z == 1 ? B->nz : B->iz1);
+        if (z < 2) {
+            o.aux[2] = B->zD[z];
+            o.aux[5] = B->zB[z][0];
+            o.zb[0] = B->zB[z][0];
+            o.zb[1] = B->zB[z][1];
+            o.flags = kGraded | kParity;
+        }
+        o.apitch = B->zpitch;
+    }
+    const int n[3] = {B->nx, B->ny, B->nz};
+    for (int a = 0; a < 3; ++a)
+        if (lo[a] == 0 || hi[a] > n[a]) o.flags |= kWalls;
+    if ((lo[0] & 3) == 0 && (hi[0] & 3) == 0 && (o.apitch & 3) == 0) o.flags |= kWhole;
+    o.i0 = lo[0]; o.i1 = hi[0]; o.ie = lo[0] & ~3; o.j0 = lo[1]; o.k0 = lo[2];
+    o.np = max((hi[0] - o.ie + 3) / 4, 1);
+    o.nj = max(hi[1] - lo[1], 1);
+    res_recip(o.np, o.mp, o.sp);
+    res_recip(o.nj, o.mj, o.sj);
+}
+
+// Shared memory, in this order: the board with its boxes, pieces, ports,
+// pulses, coefficient rows, UPML factors.
+struct Layout {
+    int piece, port, pulse, row, fac, bytes;
+};
+__host__ __device__ inline Layout layout_of(const ResPlan &p)
+{
+    Layout l;
+    auto up = [](size_t x) { return (int)((x + 15) & ~(size_t)15); };
+    l.piece = up(sizeof(BoardS));
+    l.port = up(l.piece + sizeof(ResPiece) * p.max_pieces);
+    l.pulse = up(l.port + sizeof(ResPort) * p.max_ports);
+    l.row = up(l.pulse + sizeof(double) * p.max_ports);
+    l.fac = l.row + (int)sizeof(float4) * kMaxCombo;
+    l.bytes = l.fac + (int)sizeof(float) * p.max_factors;
+    return l;
+}
+
+// Barrier of a team of blocks: `target` arrivals on a counter zeroed before
+// the launch (release on arrival, acquire on the way out).  The wait is
+// bounded; a block that gives up reports it and returns false, and the other
+// blocks' waits run out alike.
+__device__ __forceinline__ void team_arrive(unsigned *bar)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+}
+__device__ __forceinline__ bool team_wait(unsigned *bar, unsigned target, int *status, int *gave_up)
+{
+    if (threadIdx.x == 0) {
+        unsigned v = 0;
+        int it = 0;
+        do asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        while (v < target && ++it < (1 << 22));
+        if (v < target) {
+            atomicOr(status, 2);
+            *gave_up = 1;
+        }
+    }
+    __syncthreads();
+    return *(volatile int *)gave_up == 0;
+}
+
+// A team of blocks advances one board; a launch holds one team per board.
+// Every block updates H on its own pieces, waits for the team, updates E on
+// them, waits, and so on.  The E phase takes the pieces and their units
+// backwards, so that it starts with what the H phase left in L2 last, and the
+// next H phase with what the E phase left last.
+__global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int nsteps)
+{
+    const Layout l = layout_of(plan);
+    BoardS &B = board_s();
+    ResPiece *const piece = reinterpret_cast<ResPiece *>(smem + l.piece);
+    ResPort *const port = reinterpret_cast<ResPort *>(smem + l.port);
+    double *const pulse = reinterpret_cast<double *>(smem + l.pulse);
+    __shared__ int gave_up;
+    __shared__ unsigned marks[32];     // units with a source or probe, by unit number modulo 1024
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const ResBlock blk = plan.blocks[blockIdx.x];
+    const ResTeam team = plan.teams[blk.team];
+    const Board *const board = plan.boards[team.board];
+    unsigned *const bar = plan.arrive + (size_t)blk.team * 32;   // a 128-byte line of its own
+
+    if (tid == 0) {
+        fill_board(board, B, nsteps);
+        int at = l.fac / 4;
+        for (int a = 0; a < 3; ++a)
+            for (int h = 0; h < 2; ++h) {
+                B.fac[a][h] = at;
+                at += 4 * res_fac_len(B.n[a]);
+            }
+        B.row = l.row;
+        B.port = l.port;
+        B.n_port = blk.n_port;
+        B.pulse = l.pulse;
+        gave_up = 0;
+    }
+    for (int x = tid; x < board->n_slab + 3; x += kResThreads) fill_box(board, x, B.box[x]);
+    for (int x = tid; x < blk.n_piece; x += kResThreads) piece[x] = plan.pieces[blk.piece0 + x];
+    for (int x = tid; x < blk.n_port; x += kResThreads) port[x] = plan.ports[blk.port0 + x];
+    if (tid < 32) marks[tid] = 0;
+    __syncthreads();
+    for (int p = tid; p < blk.n_port; p += kResThreads) atomicOr(&marks[(port[p].unit >> 5) & 31], 1u << (port[p].unit & 31));
+    if (!B.id16)
+        for (int r = tid; r < kMaxCombo; r += kResThreads) reinterpret_cast<float4 *>(smem + l.row)[r] = board->ctab[r];
+    for (int a = 0; a < 3; ++a)
+        for (int h = 0; h < 2; ++h) {
+            const int m = res_fac_len(B.n[a]);
+            float *const f = reinterpret_cast<float *>(smem) + B.fac[a][h];
+            for (int r = tid; r < m; r += kResThreads) {
+                const Coef c = ldcoef(board->cw[a][h] + min(r, B.n[a]));
+                f[r] = c.b1;
+                f[m + r] = c.g;
+                f[2 * m + r] = c.ap;
+                f[3 * m + r] = c.am;
+            }
+        }
+    __syncthreads();
+    const int nact = B.nact;
+    unsigned target = 0;
+    for (int s = 0; s < nact; ++s) {
+        const float *const I = B.f[s == 0 ? B.first : B.work];
+        float *const O = B.f[s == nact - 1 ? B.last : B.work];
+        int turn = warp;   // units go round the warps, on from piece to piece
+        for (int p = 0; p < blk.n_piece; ++p) {
+            const ResPiece pc = piece[p];
+            const int nu = (pc.nq + 31) >> 5;
+            if (turn < nu) {
+                const BoxS &x = B.box[pc.box];
+                if (x.flags & (kGraded | kWalls)) run_h<true>(x, pc.t0, pc.t0 + pc.nq, turn, nu, I, O, (int)((B.step0 + s) & 1));
+                else run_h<false>(x, pc.t0, pc.t0 + pc.nq, turn, nu, I, O, 0);
+                turn += (nu - turn + kWarps - 1) / kWarps * kWarps;
+            }
+            turn -= nu;
+        }
+        team_arrive(bar);
+        if (warp == 1)   // Eq. 8 at this step, while the block waits
+            for (int q = lane; q < blk.n_port; q += 32)
+                if (!port[q].probe) pulse[q] = src_pulse(B.src[port[q].index], B.step0 + s, B.dt);
+        target += team.n_blocks;
+        if (!team_wait(bar, target, B.status, &gave_up)) return;
+        turn = warp;
+        for (int p = blk.n_piece - 1; p >= 0; --p) {
+            const ResPiece pc = piece[p];
+            const int nu = (pc.nq + 31) >> 5;
+            if (turn < nu) {
+                const BoxS &x = B.box[pc.box];
+                for (int v = nu - 1 - turn; v >= 0;) {
+                    // units with a source or probe one by one, the others in runs between them
+                    int f = v;
+                    if (blk.n_port)
+                        while (f >= 0 && !((marks[((pc.unit0 + f) >> 5) & 31] >> ((pc.unit0 + f) & 31)) & 1u)) f -= kWarps;
+                    else f = -1;
+                    if (f < v) {
+                        const int stop = max(f, -1);
+                        if (x.flags & (kGraded | kWalls)) run_e<true, false>(x, pc.t0, pc.t0 + pc.nq, v, stop, I, O, s, 0);
+                        else run_e<false, false>(x, pc.t0, pc.t0 + pc.nq, v, stop, I, O, s, 0);
+                    }
+                    if (f >= 0)
+                        port_unit(pc.box, pc.t0, pc.t0 + pc.nq, f, s == 0 ? B.first : B.work, s == nact - 1 ? B.last : B.work, s,
+                                  pc.unit0);
+                    v = f - kWarps;
+                }
+                turn += (nu - turn + kWarps - 1) / kWarps * kWarps;
+            }
+            turn -= nu;
+        }
+        team_arrive(bar);
+        target += team.n_blocks;
+        if (!team_wait(bar, target, B.status, &gave_up)) return;
+    }
+    // every block of the team has read the counters (before its first barrier)
+    if (tid == 0 && nact > 0 && blk.first) *((volatile long long *)board->step) = B.step0 + nact;
+}
+
+}  // namespace
+
+size_t resident_smem(const ResPlan &p) { return (size_t)layout_of(p).bytes; }
+
+cudaError_t resident_set_smem_limit()
+{
+    return cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
+}
+
+size_t resident_arrive_bytes(int n_teams) { return (size_t)n_teams * 128; }
+
+cudaError_t launch_resident(const ResPlan &plan, int nsteps, cudaStream_t st)
+{
+    cudaError_t e = cudaMemsetAsync(plan.arrive, 0, resident_arrive_bytes(plan.all_teams), st);
+    if (e != cudaSuccess) return e;
+    ResPlan p = plan;
+    void *args[] = {&p, &nsteps};
+    return cudaLaunchCooperativeKernel((const void *)k_resident, dim3(plan.n_blocks), dim3(kResThreads), args,
+                                       resident_smem(plan), st);
+}
+
+}  // namespace fdtd
