@@ -31,11 +31,12 @@ namespace fdtd {
 
 namespace {
 
-// Graded: UPML factors along some axis.  GradedX: along x.  Walls: the box
-// touches an outer wall.  Whole: its quads lie whole inside it, and so do
+// Graded: UPML factors along some axis.  GradedX: along x.  Low: the box holds
+// nodes on a low wall plane behind a PEC wall (their image is 0).  Walls: it
+// holds nodes on a high wall plane, or on a low one behind a PMC wall.  Whole: its quads lie whole inside it, and so do
 // those of its auxiliary arrays (16-byte accesses).  Parity: B~z alternates
 // between two arrays.
-enum : int { kGraded = 1, kGradedX = 2, kWalls = 4, kWhole = 8, kParity = 16 };
+enum : int { kGraded = 1, kGradedX = 2, kWalls = 4, kWhole = 8, kParity = 16, kLow = 32 };
 
 struct BoxS {     // one box of the board
     float *aux[6];          // auxiliary read and written (nullptr: none)
@@ -54,7 +55,6 @@ struct BoardS {   // the block's board, in shared memory
     float *f[3];                // field sets: six components, NN nodes apart
     const void *cid;
     const float4 *ctab;         // rows of 1 / eps_r for 16-bit ids (the block keeps a copy of those of 8-bit ids)
-    const Source *src;
     float *trace;
     int *status;
     double dt;
@@ -69,8 +69,14 @@ struct BoardS {   // the block's board, in shared memory
     float S[3];
     int fac[3][2];              // UPML factors in shared memory: float offset per axis and position
     int row;                    // coefficient rows in shared memory: byte offset
-    int port, n_port, pulse;
+    int port, n_port, drive;    // sources and probes: offsets of their places and drives, and count
     BoxS box[kMaxSlab + 3];
+};
+
+struct Drive {    // a source of the block, its Eq. 8 value at the current step, and what a current source takes off E
+    Source s;
+    double w;
+    float take;
 };
 
 extern __shared__ __align__(16) unsigned char smem[];
@@ -387,6 +393,11 @@ __device__ __forceinline__ void run_e(const BoxS &x, int t0, int end, int turn, 
             cy = curl4(hxz, hxk, hzx, hzl, Sz, Sx);
             cz = curl4(hyx, hyl, hxy, hxj, Sx, Sy);
         } else {
+            if (G && (x.flags & kLow)) {   // what lies across a low PEC wall counts as 0
+                if (i == 0) hyl.a.x = hzl.a.x = 0.f;
+                if (j == 0) hxj = hzj = four(0.f);
+                if (k == 0) hxk = hyk = four(0.f);
+            }
             cx = curl4(hz, hzj, hy, hyk, Sy, Sz);
             cy = curl4(hx, hxk, hz, hzl, Sz, Sx);
             cz = curl4(hy, hyl, hx, hxj, Sx, Sy);
@@ -445,8 +456,10 @@ __device__ __forceinline__ void run_e(const BoxS &x, int t0, int end, int turn, 
                     if (n < (long long)B.n_total) B.trace[(long long)p.index * B.n_total + n] = f;
                     if (!isfinite(f)) atomicOr(B.status, 1);
                 } else {
-                    const double pulse = reinterpret_cast<const double *>(smem + B.pulse)[v];
-                    const float f = src_apply(B.src[p.index], pulse, now, get(p.comp == 0 ? ex : p.comp == 1 ? ey : ez, e));
+                    const Drive &d = reinterpret_cast<const Drive *>(smem + B.drive)[v];
+                    const float f = d.s.kind == kSrcCurrent
+                                        ? __fsub_rn(now, d.take)
+                                        : src_apply(d.s, d.w, now, get(p.comp == 0 ? ex : p.comp == 1 ? ey : ez, e));
                     if (p.comp == 0) set(nx, e, f);
                     else if (p.comp == 1) set(ny, e, f);
                     else set(nz, e, f);
@@ -464,7 +477,7 @@ __device__ __noinline__ void port_unit(int bx, int t0, int end, int u, int si, i
 {
     const BoardS &B = board_s();
     const BoxS &x = B.box[bx];
-    if (x.flags & (kGraded | kWalls)) run_e<true, true>(x, t0, end, u, u - 1, B.f[si], B.f[so], s, base);
+    if (x.flags & (kGraded | kWalls | kLow)) run_e<true, true>(x, t0, end, u, u - 1, B.f[si], B.f[so], s, base);
     else run_e<false, true>(x, t0, end, u, u - 1, B.f[si], B.f[so], s, base);
 }
 
@@ -477,7 +490,6 @@ __device__ void fill_board(const Board *B, BoardS &o, int nsteps)
     for (int a = 0; a < 3; ++a) o.S[a] = B->S[a];
     o.cid = B->cid;
     o.ctab = B->ctab;
-    o.src = B->src;
     o.trace = B->trace;
     o.status = B->status;
     o.dt = B->dt;
@@ -528,7 +540,8 @@ __device__ void fill_box(const Board *B, int kind, BoxS &o)
     }
     const int n[3] = {B->nx, B->ny, B->nz};
     for (int a = 0; a < 3; ++a)
-        if (lo[a] == 0 || hi[a] > n[a]) o.flags |= kWalls;
+        if (hi[a] > n[a] || (lo[a] == 0 && B->wall[2 * a] != 0)) o.flags |= kWalls;
+        else if (lo[a] == 0) o.flags |= kLow;
     if ((lo[0] & 3) == 0 && (hi[0] & 3) == 0 && (o.apitch & 3) == 0) o.flags |= kWhole;
     o.i0 = lo[0]; o.i1 = hi[0]; o.ie = lo[0] & ~3; o.j0 = lo[1]; o.k0 = lo[2];
     o.np = max((hi[0] - o.ie + 3) / 4, 1);
@@ -538,9 +551,9 @@ __device__ void fill_box(const Board *B, int kind, BoxS &o)
 }
 
 // Shared memory, in this order: the board with its boxes, pieces, ports,
-// pulses, coefficient rows, UPML factors.
+// drives, coefficient rows, UPML factors.
 struct Layout {
-    int piece, port, pulse, row, fac, bytes;
+    int piece, port, drive, row, fac, bytes;
 };
 __host__ __device__ inline Layout layout_of(const ResPlan &p)
 {
@@ -548,8 +561,8 @@ __host__ __device__ inline Layout layout_of(const ResPlan &p)
     auto up = [](size_t x) { return (int)((x + 15) & ~(size_t)15); };
     l.piece = up(sizeof(BoardS));
     l.port = up(l.piece + sizeof(ResPiece) * p.max_pieces);
-    l.pulse = up(l.port + sizeof(ResPort) * p.max_ports);
-    l.row = up(l.pulse + sizeof(double) * p.max_ports);
+    l.drive = up(l.port + sizeof(ResPort) * p.max_ports);
+    l.row = up(l.drive + sizeof(Drive) * p.max_ports);
     l.fac = l.row + (int)sizeof(float4) * kMaxCombo;
     l.bytes = l.fac + (int)sizeof(float) * p.max_factors;
     return l;
@@ -591,7 +604,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
     BoardS &B = board_s();
     ResPiece *const piece = reinterpret_cast<ResPiece *>(smem + l.piece);
     ResPort *const port = reinterpret_cast<ResPort *>(smem + l.port);
-    double *const pulse = reinterpret_cast<double *>(smem + l.pulse);
+    Drive *const drive = reinterpret_cast<Drive *>(smem + l.drive);
     __shared__ int gave_up;
     __shared__ unsigned marks[32];     // units with a source or probe, by unit number modulo 1024
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -611,7 +624,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
         B.row = l.row;
         B.port = l.port;
         B.n_port = blk.n_port;
-        B.pulse = l.pulse;
+        B.drive = l.drive;
         gave_up = 0;
     }
     for (int x = tid; x < board->n_slab + 3; x += kResThreads) fill_box(board, x, B.box[x]);
@@ -619,6 +632,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
     for (int x = tid; x < blk.n_port; x += kResThreads) port[x] = plan.ports[blk.port0 + x];
     if (tid < 32) marks[tid] = 0;
     __syncthreads();
+    for (int p = tid; p < blk.n_port; p += kResThreads)
+        if (!port[p].probe) drive[p].s = board->src[port[p].index];
     for (int p = tid; p < blk.n_port; p += kResThreads) atomicOr(&marks[(port[p].unit >> 5) & 31], 1u << (port[p].unit & 31));
     if (!B.id16)
         for (int r = tid; r < kMaxCombo; r += kResThreads) reinterpret_cast<float4 *>(smem + l.row)[r] = board->ctab[r];
@@ -646,7 +661,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
             const int nu = (pc.nq + 31) >> 5;
             if (turn < nu) {
                 const BoxS &x = B.box[pc.box];
-                if (x.flags & (kGraded | kWalls)) run_h<true>(x, pc.t0, pc.t0 + pc.nq, turn, nu, I, O, (int)((B.step0 + s) & 1));
+                if (x.flags & (kGraded | kWalls | kLow)) run_h<true>(x, pc.t0, pc.t0 + pc.nq, turn, nu, I, O, (int)((B.step0 + s) & 1));
                 else run_h<false>(x, pc.t0, pc.t0 + pc.nq, turn, nu, I, O, 0);
                 turn += (nu - turn + kWarps - 1) / kWarps * kWarps;
             }
@@ -655,7 +670,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
         team_arrive(bar);
         if (warp == 1)   // Eq. 8 at this step, while the block waits
             for (int q = lane; q < blk.n_port; q += 32)
-                if (!port[q].probe) pulse[q] = src_pulse(B.src[port[q].index], B.step0 + s, B.dt);
+                if (!port[q].probe) {
+                    drive[q].w = src_pulse(drive[q].s, B.step0 + s, B.dt);
+                    drive[q].take = (float)(drive[q].s.coef * drive[q].w);
+                }
         target += team.n_blocks;
         if (!team_wait(bar, target, B.status, &gave_up)) return;
         turn = warp;
@@ -672,7 +690,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
                     else f = -1;
                     if (f < v) {
                         const int stop = max(f, -1);
-                        if (x.flags & (kGraded | kWalls)) run_e<true, false>(x, pc.t0, pc.t0 + pc.nq, v, stop, I, O, s, 0);
+                        if (x.flags & (kGraded | kWalls | kLow)) run_e<true, false>(x, pc.t0, pc.t0 + pc.nq, v, stop, I, O, s, 0);
                         else run_e<false, false>(x, pc.t0, pc.t0 + pc.nq, v, stop, I, O, s, 0);
                     }
                     if (f >= 0)
