@@ -1005,6 +1005,7 @@ int upload_resident(const ResHost &R, Board *const *dev_boards, long long *&buf,
     plan.max_pieces = R.max_pieces;
     plan.max_ports = R.max_ports;
     plan.max_factors = R.max_factors;
+    plan.max_units = R.max_units;
     return FDTD_OK;
 }
 
@@ -1055,19 +1056,22 @@ int build_resident_batch(const std::vector<fdtd_ctx *> &boards, Board *const *de
         const std::vector<int> n = res_share(work, sms);
         plans[g].n_blocks = -(int)R.blocks.size();
         plans[g].n_teams = -(int)R.teams.size();
+        R.max_units = 0;
         for (size_t t = 0; t < n.size(); ++t) res_team(boards[group[g][t]]->h, res_ports(boards[group[g][t]]), group[g][t], n[t], R);
         plans[g].n_blocks += (int)R.blocks.size();
         plans[g].n_teams += (int)R.teams.size();
+        plans[g].max_units = R.max_units;
     }
     ResPlan all{};
     if (int r = upload_resident(R, dev_boards, buf, cap, all, st, host)) return r;
     int blk = 0;
     for (ResPlan &p : plans) {
-        const int nb = p.n_blocks, nt = p.n_teams;
+        const int nb = p.n_blocks, nt = p.n_teams, nu = p.max_units;
         p = all;   // (a block names its team by its place among all teams, and so its counter)
         p.n_blocks = nb;
         p.blocks = all.blocks + blk;
         p.n_teams = nt;
+        p.max_units = nu;
         blk += nb;
     }
     return FDTD_OK;

@@ -279,6 +279,7 @@ struct ResPlan {
     const ResPiece *pieces;
     const ResPort *ports;
     int max_pieces, max_ports, max_factors;   // of a block
+    int max_units;                // of a block; at most kPinWarps: each warp keeps its unit (k_pinned)
     unsigned *arrive;             // arrivals per team (zeroed before every launch)
 };
 // Length of a UPML factor array in a block's shared memory (n + 1 positions, whole quads).
@@ -294,6 +295,10 @@ __host__ __device__ inline int res_quot(int t, unsigned m, int s)
 {
     return (int)(((unsigned)(((unsigned long long)(unsigned)t * m) >> 32) + (unsigned)t) >> s);
 }
+// Warps of a block of k_pinned (one unit each; 912 units on 152 blocks).  Measured
+// us a step against k_resident: 4.5 against 5.65-5.95 at 216 to 630 units, 6.4
+// against 5.9 at 1151 units with eight warps.
+constexpr int kPinWarps = 6;
 constexpr int kResSmem = 200 << 10;   // shared memory a resident launch may ask for
 
 // TMA descriptor slots of a board (3D maps: x, y, plane).

@@ -13,10 +13,11 @@
 // (12-13.7 TB/s measured up to 90 MB); there a phase is bound by L2 latency
 // (small boards) or L2 bandwidth, past L2 by HBM at 73 B a node and step.
 //
-// Measured (us a step, launch-per-phase path -> here): 38x33x20 57 -> 5.9,
-// 56x48x30 62 -> 6.2, 181x131x6 34 -> 6.7, 232x192x39 90 -> 22.7, 280x230x100
-// 160 -> 96, 480x380x100 294 -> 261; a batch of 24 boards (41 M cells) 852 ->
-// 629.  At 880x680x100 the tiled launches' 49 B a node win (697 against 902).
+// Measured (us a step, launch-per-phase path -> here): 38x33x20 57 -> 4.5 and
+// 56x48x30 62 -> 4.5 (k_pinned), 181x131x6 34 -> 5.9, 232x192x39 90 -> 22.1,
+// 280x230x100 160 -> 95, 480x380x100 294 -> 259; a batch of 24 boards (41 M
+// cells) 852 -> 618.  At 880x680x100 the tiled launches' 49 B a node win (697
+// against 902).
 //
 // The work is cut into units of 32 column quads (128 nodes), taken in x, y, z
 // order from one box at a time.  The boxes are the board's own (slab boxes,
@@ -82,7 +83,7 @@ struct Drive {    // a source of the block, its Eq. 8 value at the current step,
 extern __shared__ __align__(16) unsigned char smem[];
 __device__ __forceinline__ BoardS &board_s() { return *reinterpret_cast<BoardS *>(smem); }
 
-constexpr int kResThreads = 512, kWarps = kResThreads / 32;
+constexpr int kWarps = 16, kResThreads = 32 * kWarps, kPinThreads = 32 * kPinWarps;
 
 struct F4 {       // four neighbouring nodes of a row
     float2 a, b;
@@ -332,6 +333,76 @@ __device__ __forceinline__ void image4(bool lo, bool hi, int wlo, int whi, F4 &p
     image(lo, hi, wlo, whi, p.b.y, m.b.y);
 }
 
+__device__ __forceinline__ void images(const BoardS &B, int i, int j, int k, F4 &hyx, F4 &hzx, F4 &hxy, F4 &hzy, F4 &hxz, F4 &hyz,
+                                       F4 &hyl, F4 &hzl, F4 &hxj, F4 &hzj, F4 &hxk, F4 &hyk)
+{
+    const int n = B.n[0], w0 = B.wall[0], w1 = B.wall[1];
+    image(i == 0, i == n, w0, w1, hyx.a.x, hyl.a.x);
+    image(i == 0, i == n, w0, w1, hzx.a.x, hzl.a.x);
+    image(false, i + 1 == n, w0, w1, hyx.a.y, hyl.a.y);
+    image(false, i + 1 == n, w0, w1, hzx.a.y, hzl.a.y);
+    image(false, i + 2 == n, w0, w1, hyx.b.x, hyl.b.x);
+    image(false, i + 2 == n, w0, w1, hzx.b.x, hzl.b.x);
+    image(false, i + 3 == n, w0, w1, hyx.b.y, hyl.b.y);
+    image(false, i + 3 == n, w0, w1, hzx.b.y, hzl.b.y);
+    image4(j == 0, j == B.n[1], B.wall[2], B.wall[3], hxy, hxj);
+    image4(j == 0, j == B.n[1], B.wall[2], B.wall[3], hzy, hzj);
+    image4(k == 0, k == B.n[2], B.wall[4], B.wall[5], hxz, hxk);
+    image4(k == 0, k == B.n[2], B.wall[4], B.wall[5], hyz, hyk);
+}
+
+// 1 / eps_r of a quad's edges from its ids.
+__device__ __forceinline__ void rows_of(const BoardS &B, bool id16, const uint2 &id, F4 &kx, F4 &ky, F4 &kz)
+{
+    float4 r0, r1, r2, r3;
+    if (id16) {
+        const float4 *const r = B.ctab;
+        r0 = __ldg(r + (id.x & 0xffffu)); r1 = __ldg(r + (id.x >> 16));
+        r2 = __ldg(r + (id.y & 0xffffu)); r3 = __ldg(r + (id.y >> 16));
+    } else {
+        const float4 *const r = reinterpret_cast<const float4 *>(smem + B.row);
+        r0 = r[id.x & 0xffu]; r1 = r[(id.x >> 8) & 0xffu]; r2 = r[(id.x >> 16) & 0xffu]; r3 = r[id.x >> 24];
+    }
+    kx = F4{make_float2(r0.x, r1.x), make_float2(r2.x, r3.x)};
+    ky = F4{make_float2(r0.y, r1.y), make_float2(r2.y, r3.y)};
+    kz = F4{make_float2(r0.z, r1.z), make_float2(r2.z, r3.z)};
+}
+
+// The block's sources on edges of unit `unit`, in order (several may share an
+// edge), then its probe samples: nx, ny, nz is the new E of the lane's quad, ex,
+// ey, ez its E before.
+__device__ __forceinline__ void work_ports(int unit, int s, F4 &nx, F4 &ny, F4 &nz, const F4 &ex, const F4 &ey, const F4 &ez)
+{
+    const BoardS &B = board_s();
+    const int lane = threadIdx.x & 31;
+    const ResPort *const list = reinterpret_cast<const ResPort *>(smem + B.port);
+    for (int v0 = 0; v0 < B.n_port; v0 += 32) {
+        const int mine = v0 + lane;
+        unsigned hit = __ballot_sync(0xffffffffu, mine < B.n_port && list[mine].unit == unit);
+        for (; hit; hit &= hit - 1) {
+            const int v = v0 + __ffs(hit) - 1;
+            const ResPort &p = list[v];
+            if (p.lane != lane) continue;
+            const int e = p.col;
+            const float now = get(p.comp == 0 ? nx : p.comp == 1 ? ny : nz, e);
+            if (p.probe) {
+                const float f = now * B.scale;
+                const long long n = B.step0 + s;
+                if (n < (long long)B.n_total) B.trace[(long long)p.index * B.n_total + n] = f;
+                if (!isfinite(f)) atomicOr(B.status, 1);
+            } else {
+                const Drive &d = reinterpret_cast<const Drive *>(smem + B.drive)[v];
+                const float f = d.s.kind == kSrcCurrent
+                                    ? __fsub_rn(now, d.take)
+                                    : src_apply(d.s, d.w, now, get(p.comp == 0 ? ex : p.comp == 1 ? ey : ez, e));
+                if (p.comp == 0) set(nx, e, f);
+                else if (p.comp == 1) set(ny, e, f);
+                else set(nz, e, f);
+            }
+        }
+    }
+}
+
 // E^{n+1} of the units turn, turn - kWarps, ... > stop of a piece: E^n from set
 // I, H~^{n+1/2} from set O, into set O.  PORTS: the units hold sources or probes
 // (unit `base + u` of the block, local step s).
@@ -371,22 +442,10 @@ __device__ __forceinline__ void run_e(const BoxS &x, int t0, int end, int turn, 
         const int i = w.ie + 4 * q.p, j = x.j0 + q.r - q.kk * w.nj, k = x.k0 + q.kk;
         F4 cx, cy, cz;
         if (G && (x.flags & kWalls)) {
-            const int n = B.n[0], w0 = B.wall[0], w1 = B.wall[1];
             // H~ on the + side of the node, per axis of difference
             F4 hyx = hy, hzx = hz, hxy = hx, hzy = hz, hxz = hx, hyz = hy;
-            image(i == 0, i == n, w0, w1, hyx.a.x, hyl.a.x);
-            image(i == 0, i == n, w0, w1, hzx.a.x, hzl.a.x);
-            image(false, i + 1 == n, w0, w1, hyx.a.y, hyl.a.y);
-            image(false, i + 1 == n, w0, w1, hzx.a.y, hzl.a.y);
-            image(false, i + 2 == n, w0, w1, hyx.b.x, hyl.b.x);
-            image(false, i + 2 == n, w0, w1, hzx.b.x, hzl.b.x);
-            image(false, i + 3 == n, w0, w1, hyx.b.y, hyl.b.y);
-            image(false, i + 3 == n, w0, w1, hzx.b.y, hzl.b.y);
-            image4(j == 0, j == B.n[1], B.wall[2], B.wall[3], hxy, hxj);
-            image4(j == 0, j == B.n[1], B.wall[2], B.wall[3], hzy, hzj);
-            image4(k == 0, k == B.n[2], B.wall[4], B.wall[5], hxz, hxk);
-            image4(k == 0, k == B.n[2], B.wall[4], B.wall[5], hyz, hyk);
-            mx &= below(i, n);
+            images(B, i, j, k, hyx, hzx, hxy, hzy, hxz, hyz, hyl, hzl, hxj, hzj, hxk, hyk);
+            mx &= below(i, B.n[0]);
             if (j >= B.n[1]) my = 0;
             if (k >= B.n[2]) mz = 0;
             cx = curl4(hzy, hzj, hyz, hyk, Sy, Sz);
@@ -402,17 +461,8 @@ __device__ __forceinline__ void run_e(const BoxS &x, int t0, int end, int turn, 
             cy = curl4(hx, hxk, hz, hzl, Sz, Sx);
             cz = curl4(hy, hyl, hx, hxj, Sx, Sy);
         }
-        float4 r0, r1, r2, r3;   // 1 / eps_r of the quad's edges
-        if (id16) {
-            const float4 *const r = B.ctab;
-            r0 = __ldg(r + (id.x & 0xffffu)); r1 = __ldg(r + (id.x >> 16));
-            r2 = __ldg(r + (id.y & 0xffffu)); r3 = __ldg(r + (id.y >> 16));
-        } else {
-            const float4 *const r = reinterpret_cast<const float4 *>(smem + B.row);
-            r0 = r[id.x & 0xffu]; r1 = r[(id.x >> 8) & 0xffu]; r2 = r[(id.x >> 16) & 0xffu]; r3 = r[id.x >> 24];
-        }
-        const F4 kx{make_float2(r0.x, r1.x), make_float2(r2.x, r3.x)}, ky{make_float2(r0.y, r1.y), make_float2(r2.y, r3.y)},
-            kz{make_float2(r0.z, r1.z), make_float2(r2.z, r3.z)};
+        F4 kx, ky, kz;
+        rows_of(B, id16, id, kx, ky, kz);
         F4 nx, ny, nz;
         if (!G) {
             nx = fma4(kx, cx, ex);
@@ -439,33 +489,7 @@ __device__ __forceinline__ void run_e(const BoxS &x, int t0, int end, int turn, 
                 staux(a, q, n, mz, whole);
             }
         }
-        // sources on edges of this unit, in order (several may share an edge), then probe samples
-        const ResPort *const list = reinterpret_cast<const ResPort *>(smem + B.port);
-        for (int v0 = 0; PORTS && v0 < B.n_port; v0 += 32) {
-            const int mine = v0 + lane;
-            unsigned hit = __ballot_sync(0xffffffffu, mine < B.n_port && list[mine].unit == base + u);
-            for (; hit; hit &= hit - 1) {
-                const int v = v0 + __ffs(hit) - 1;
-                const ResPort &p = list[v];
-                if (p.lane != lane) continue;
-                const int e = p.col;
-                const float now = get(p.comp == 0 ? nx : p.comp == 1 ? ny : nz, e);
-                if (p.probe) {
-                    const float f = now * B.scale;
-                    const long long n = B.step0 + s;
-                    if (n < (long long)B.n_total) B.trace[(long long)p.index * B.n_total + n] = f;
-                    if (!isfinite(f)) atomicOr(B.status, 1);
-                } else {
-                    const Drive &d = reinterpret_cast<const Drive *>(smem + B.drive)[v];
-                    const float f = d.s.kind == kSrcCurrent
-                                        ? __fsub_rn(now, d.take)
-                                        : src_apply(d.s, d.w, now, get(p.comp == 0 ? ex : p.comp == 1 ? ey : ez, e));
-                    if (p.comp == 0) set(nx, e, f);
-                    else if (p.comp == 1) set(ny, e, f);
-                    else set(nz, e, f);
-                }
-            }
-        }
+        if (PORTS) work_ports(base + u, s, nx, ny, nz, ex, ey, ez);
         st4(O + at, nx, mx);
         st4(O + (at + N), ny, my);
         st4(O + (at + 2 * N), nz, mz);
@@ -593,26 +617,16 @@ __device__ __forceinline__ bool team_wait(unsigned *bar, unsigned target, int *s
     return *(volatile int *)gave_up == 0;
 }
 
-// A team of blocks advances one board; a launch holds one team per board.
-// Every block updates H on its own pieces, waits for the team, updates E on
-// them, waits, and so on.  The E phase takes the pieces and their units
-// backwards, so that it starts with what the H phase left in L2 last, and the
-// next H phase with what the E phase left last.
-__global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int nsteps)
+// Fills a block's shared memory; ends with a barrier.  marks: units with a
+// source or probe, by unit number modulo 1024.
+__device__ __forceinline__ void set_up(const ResPlan &plan, const Layout &l, const ResBlock &blk, const Board *board, int nsteps,
+                                       int *gave_up, unsigned *marks)
 {
-    const Layout l = layout_of(plan);
     BoardS &B = board_s();
     ResPiece *const piece = reinterpret_cast<ResPiece *>(smem + l.piece);
     ResPort *const port = reinterpret_cast<ResPort *>(smem + l.port);
     Drive *const drive = reinterpret_cast<Drive *>(smem + l.drive);
-    __shared__ int gave_up;
-    __shared__ unsigned marks[32];     // units with a source or probe, by unit number modulo 1024
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const ResBlock blk = plan.blocks[blockIdx.x];
-    const ResTeam team = plan.teams[blk.team];
-    const Board *const board = plan.boards[team.board];
-    unsigned *const bar = plan.arrive + (size_t)blk.team * 32;   // a 128-byte line of its own
-
+    const int tid = threadIdx.x, nt = blockDim.x;
     if (tid == 0) {
         fill_board(board, B, nsteps);
         int at = l.fac / 4;
@@ -625,23 +639,23 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
         B.port = l.port;
         B.n_port = blk.n_port;
         B.drive = l.drive;
-        gave_up = 0;
+        *gave_up = 0;
     }
-    for (int x = tid; x < board->n_slab + 3; x += kResThreads) fill_box(board, x, B.box[x]);
-    for (int x = tid; x < blk.n_piece; x += kResThreads) piece[x] = plan.pieces[blk.piece0 + x];
-    for (int x = tid; x < blk.n_port; x += kResThreads) port[x] = plan.ports[blk.port0 + x];
+    for (int x = tid; x < board->n_slab + 3; x += nt) fill_box(board, x, B.box[x]);
+    for (int x = tid; x < blk.n_piece; x += nt) piece[x] = plan.pieces[blk.piece0 + x];
+    for (int x = tid; x < blk.n_port; x += nt) port[x] = plan.ports[blk.port0 + x];
     if (tid < 32) marks[tid] = 0;
     __syncthreads();
-    for (int p = tid; p < blk.n_port; p += kResThreads)
+    for (int p = tid; p < blk.n_port; p += nt)
         if (!port[p].probe) drive[p].s = board->src[port[p].index];
-    for (int p = tid; p < blk.n_port; p += kResThreads) atomicOr(&marks[(port[p].unit >> 5) & 31], 1u << (port[p].unit & 31));
+    for (int p = tid; p < blk.n_port; p += nt) atomicOr(&marks[(port[p].unit >> 5) & 31], 1u << (port[p].unit & 31));
     if (!B.id16)
-        for (int r = tid; r < kMaxCombo; r += kResThreads) reinterpret_cast<float4 *>(smem + l.row)[r] = board->ctab[r];
+        for (int r = tid; r < kMaxCombo; r += nt) reinterpret_cast<float4 *>(smem + l.row)[r] = board->ctab[r];
     for (int a = 0; a < 3; ++a)
         for (int h = 0; h < 2; ++h) {
             const int m = res_fac_len(B.n[a]);
             float *const f = reinterpret_cast<float *>(smem) + B.fac[a][h];
-            for (int r = tid; r < m; r += kResThreads) {
+            for (int r = tid; r < m; r += nt) {
                 const Coef c = ldcoef(board->cw[a][h] + min(r, B.n[a]));
                 f[r] = c.b1;
                 f[m + r] = c.g;
@@ -650,6 +664,39 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
             }
         }
     __syncthreads();
+}
+
+// Eq. 8 of the block's sources at local step s (by one warp).
+__device__ __forceinline__ void pulses(const Layout &l, const ResBlock &blk, int s)
+{
+    const BoardS &B = board_s();
+    const ResPort *const port = reinterpret_cast<const ResPort *>(smem + l.port);
+    Drive *const drive = reinterpret_cast<Drive *>(smem + l.drive);
+    for (int q = threadIdx.x & 31; q < blk.n_port; q += 32)
+        if (!port[q].probe) {
+            drive[q].w = src_pulse(drive[q].s, B.step0 + s, B.dt);
+            drive[q].take = (float)(drive[q].s.coef * drive[q].w);
+        }
+}
+
+// A team of blocks advances one board; a launch holds one team per board.
+// Every block updates H on its own pieces, waits for the team, updates E on
+// them, waits, and so on.  The E phase takes the pieces and their units
+// backwards, so that it starts with what the H phase left in L2 last, and the
+// next H phase with what the E phase left last.
+__global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int nsteps)
+{
+    const Layout l = layout_of(plan);
+    BoardS &B = board_s();
+    const ResPiece *const piece = reinterpret_cast<const ResPiece *>(smem + l.piece);
+    __shared__ int gave_up;
+    __shared__ unsigned marks[32];
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const ResBlock blk = plan.blocks[blockIdx.x];
+    const ResTeam team = plan.teams[blk.team];
+    const Board *const board = plan.boards[team.board];
+    unsigned *const bar = plan.arrive + (size_t)blk.team * 32;   // a 128-byte line of its own
+    set_up(plan, l, blk, board, nsteps, &gave_up, marks);
     const int nact = B.nact;
     unsigned target = 0;
     for (int s = 0; s < nact; ++s) {
@@ -668,12 +715,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
             turn -= nu;
         }
         team_arrive(bar);
-        if (warp == 1)   // Eq. 8 at this step, while the block waits
-            for (int q = lane; q < blk.n_port; q += 32)
-                if (!port[q].probe) {
-                    drive[q].w = src_pulse(drive[q].s, B.step0 + s, B.dt);
-                    drive[q].take = (float)(drive[q].s.coef * drive[q].w);
-                }
+        if (warp == 1) pulses(l, blk, s);   // while the block waits
         target += team.n_blocks;
         if (!team_wait(bar, target, B.status, &gave_up)) return;
         turn = warp;
@@ -710,13 +752,172 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResPlan plan, int n
     if (tid == 0 && nact > 0 && blk.first) *((volatile long long *)board->step) = B.step0 + nact;
 }
 
+// The same for boards of at most kPinWarps units a block.  There a step of
+// k_resident is latency: two barriers, and in each phase the way from the
+// barrier to the loads, L2, and back to the barrier.  Here a warp has one unit
+// and a lane keeps its quad for the whole launch, its E, H~, auxiliaries and
+// ids in registers, so that a phase is the six loads of its neighbours, the
+// update and three stores.  (A quad cut by the box's edge reads itself again:
+// its other nodes are some other lane's.)  38x33x20 5.65 -> 4.5, 56x48x30 5.95
+// -> 4.5 us a step, of which the two barriers take 2.4.  Auxiliaries go back to memory at the
+// end; B~z of the z-UPML boxes alternates between two arrays, so its last two
+// values do.
+__global__ void __launch_bounds__(kPinThreads, 1) k_pinned(ResPlan plan, int nsteps)
+{
+    const Layout l = layout_of(plan);
+    BoardS &B = board_s();
+    __shared__ int gave_up;
+    __shared__ unsigned marks[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const ResBlock blk = plan.blocks[blockIdx.x];
+    const ResTeam team = plan.teams[blk.team];
+    const Board *const board = plan.boards[team.board];
+    unsigned *const bar = plan.arrive + (size_t)blk.team * 32;
+    set_up(plan, l, blk, board, nsteps, &gave_up, marks);
+    const int nact = B.nact, X = B.X, P = B.P, N = B.NN;
+    // the warp's unit and the lane's quad
+    ResPiece pc{0, 0, 0, 0};
+    bool live = false;
+    for (int p = 0; p < blk.n_piece && !live; ++p) {
+        pc = reinterpret_cast<const ResPiece *>(smem + l.piece)[p];
+        live = warp >= pc.unit0 && warp < pc.unit0 + ((pc.nq + 31) >> 5);
+    }
+    live = live && nact > 0;
+    const BoxS &x = B.box[live ? pc.box : 0];
+    const bool whole = (x.flags & kWhole) != 0, gx = (x.flags & kGradedX) != 0;
+    const bool graded = (x.flags & (kGraded | kWalls | kLow)) != 0;
+    const bool ports = live && ((marks[warp >> 5] >> (warp & 31)) & 1u);
+    Pos q{};
+    int i = 0, j = 0, k = 0;
+    unsigned mh[3] = {0, 0, 0}, me[3] = {0, 0, 0};   // nodes of the quad whose H~, E exist
+    F4 ex{}, ey{}, ez{}, hx{}, hy{}, hz{}, b0{}, b1{}, b2{}, d0{}, d1{}, d2{};
+    unsigned kept = 0;                               // auxiliaries the box keeps (bit c)
+    uint2 id = make_uint2(0, 0);
+    const bool id16 = B.id16 != 0;
+    if (live) {
+        const Walk w(x);
+        q = locate(w, pc.t0 + 32 * (warp - pc.unit0) + lane, pc.t0 + pc.nq, whole);
+        i = w.ie + 4 * q.p; j = x.j0 + q.r - q.kk * w.nj; k = x.k0 + q.kk;
+        const bool yin = j < B.n[1], zin = k < B.n[2];
+        const unsigned bx = below(i, B.n[0]);
+        mh[0] = yin && zin ? q.own : 0u; mh[1] = zin ? q.own & bx : 0u; mh[2] = yin ? q.own & bx : 0u;
+        me[0] = q.own & bx; me[1] = yin ? q.own : 0u; me[2] = zin ? q.own : 0u;
+        const float *const I = B.f[B.first];
+        ex = ld4(I + q.at); ey = ld4(I + (q.at + N)); ez = ld4(I + (q.at + 2 * N));
+        hx = ld4(I + (q.at + 3 * N)); hy = ld4(I + (q.at + 4 * N)); hz = ld4(I + (q.at + 5 * N));
+        for (int c = 0; c < 6; ++c) kept |= (x.aux[c] != nullptr ? 1u : 0u) << c;
+        const int par = (int)(B.step0 & 1);
+        d0 = ldaux(x.aux[0], q, whole); d1 = ldaux(x.aux[1], q, whole); d2 = ldaux(x.aux[2], q, whole);
+        b0 = ldaux(x.aux[3], q, whole); b1 = ldaux(x.aux[4], q, whole);
+        b2 = ldaux(x.flags & kParity ? x.zb[par] : x.aux[5], q, whole);
+        if (id16) id = *reinterpret_cast<const uint2 *>((const uint16_t *)B.cid + q.at);
+        else id.x = *reinterpret_cast<const unsigned *>((const uint8_t *)B.cid + q.at);
+    }
+    const bool cut = q.own != 15u && q.own != 0u;
+    const int at = q.at;
+    unsigned target = 0;
+    for (int s = 0; s < nact; ++s) {
+        const float *const I = B.f[s == 0 ? B.first : B.work];
+        float *const O = B.f[s == nact - 1 ? B.last : B.work];
+        if (live) {
+            const F4 exj = ld4(I + (at + X)), ezj = ld4(I + (at + 2 * N + X));
+            const F4 exk = ld4(I + (at + P)), eyk = ld4(I + (at + N + P));
+            const float eyi = I[at + N + 4], ezi = I[at + 2 * N + 4];
+            F4 vy = ey, vz = ez;
+            if (cut) { vy = ld4(I + (at + N)); vz = ld4(I + (at + 2 * N)); }
+            const F4 cx = curl4(ezj, ez, eyk, ey, B.S[1], B.S[2]);
+            const F4 cy = curl4(exk, ex, F4{make_float2(vz.a.y, vz.b.x), make_float2(vz.b.y, ezi)}, ez, B.S[2], B.S[0]);
+            const F4 cz = curl4(F4{make_float2(vy.a.y, vy.b.x), make_float2(vy.b.y, eyi)}, ey, exj, ex, B.S[0], B.S[1]);
+            if (!graded) {
+                hx = sub4(hx, cx);
+                hy = sub4(hy, cy);
+                hz = sub4(hz, cz);
+            } else {
+                const C4 y1 = fac_row(B.fac[1][1], B.n[1], j), z1 = fac_row(B.fac[2][1], B.n[2], k);
+                const C4 x1 = gx ? fac_quad(B.fac[0][1], B.n[0], i) : fac_one();
+                F4 n;
+                hx = upml_h4(hx, cx, y1, z1, gx ? fac_quad(B.fac[0][0], B.n[0], i) : fac_one(), kept & 8u, b0, n);
+                if (kept & 8u) b0 = n;
+                hy = upml_h4(hy, cy, z1, x1, fac_row(B.fac[1][0], B.n[1], j), kept & 16u, b1, n);
+                if (kept & 16u) b1 = n;
+                hz = upml_h4(hz, cz, x1, y1, fac_row(B.fac[2][0], B.n[2], k), kept & 32u, b2, n);
+                if (kept & 32u) b2 = n;
+            }
+            st4(O + (at + 3 * N), hx, mh[0]);
+            st4(O + (at + 4 * N), hy, mh[1]);
+            st4(O + (at + 5 * N), hz, mh[2]);
+        }
+        team_arrive(bar);
+        if (warp == 1) pulses(l, blk, s);   // while the block waits
+        target += team.n_blocks;
+        if (!team_wait(bar, target, B.status, &gave_up)) return;
+        if (live) {
+            F4 hxj = ld4(O + (at + 3 * N - X)), hzj = ld4(O + (at + 5 * N - X));
+            F4 hxk = ld4(O + (at + 3 * N - P)), hyk = ld4(O + (at + 4 * N - P));
+            const float hyi = O[at + 4 * N - 1], hzi = O[at + 5 * N - 1];
+            F4 vy = hy, vz = hz;
+            if (cut) { vy = ld4(O + (at + 4 * N)); vz = ld4(O + (at + 5 * N)); }
+            F4 hyl{make_float2(hyi, vy.a.x), make_float2(vy.a.y, vy.b.x)};   // H~y, H~z at i - 1
+            F4 hzl{make_float2(hzi, vz.a.x), make_float2(vz.a.y, vz.b.x)};
+            // H~ on the + side of the node, per axis of difference
+            F4 hyx = hy, hzx = hz, hxy = hx, hzy = hz, hxz = hx, hyz = hy;
+            if (x.flags & kWalls) images(B, i, j, k, hyx, hzx, hxy, hzy, hxz, hyz, hyl, hzl, hxj, hzj, hxk, hyk);
+            else if (x.flags & kLow) {
+                if (i == 0) hyl.a.x = hzl.a.x = 0.f;
+                if (j == 0) hxj = hzj = four(0.f);
+                if (k == 0) hxk = hyk = four(0.f);
+            }
+            F4 kx, ky, kz;
+            rows_of(B, id16, id, kx, ky, kz);
+            const F4 cx = curl4(hzy, hzj, hyz, hyk, B.S[1], B.S[2]);
+            const F4 cy = curl4(hxz, hxk, hzx, hzl, B.S[2], B.S[0]);
+            const F4 cz = curl4(hyx, hyl, hxy, hxj, B.S[0], B.S[1]);
+            F4 nx, ny, nz;
+            if (!graded) {
+                nx = fma4(kx, cx, ex);
+                ny = fma4(ky, cy, ey);
+                nz = fma4(kz, cz, ez);
+            } else {
+                const C4 y0 = fac_row(B.fac[1][0], B.n[1], j), z0 = fac_row(B.fac[2][0], B.n[2], k);
+                const C4 x0 = gx ? fac_quad(B.fac[0][0], B.n[0], i) : fac_one();
+                F4 n;
+                nx = upml_e4(ex, cx, kx, y0, z0, gx ? fac_quad(B.fac[0][1], B.n[0], i) : fac_one(), kept & 1u, d0, n);
+                if (kept & 1u) d0 = n;
+                ny = upml_e4(ey, cy, ky, z0, x0, fac_row(B.fac[1][1], B.n[1], j), kept & 2u, d1, n);
+                if (kept & 2u) d1 = n;
+                nz = upml_e4(ez, cz, kz, x0, y0, fac_row(B.fac[2][1], B.n[2], k), kept & 4u, d2, n);
+                if (kept & 4u) d2 = n;
+            }
+            if (ports) work_ports(warp, s, nx, ny, nz, ex, ey, ez);
+            ex = nx; ey = ny; ez = nz;
+            st4(O + at, ex, me[0]);
+            st4(O + (at + N), ey, me[1]);
+            st4(O + (at + 2 * N), ez, me[2]);
+            if (s >= nact - 2 && (x.flags & kParity)) staux(x.zb[(B.step0 + s + 1) & 1], q, b2, mh[2], whole);
+            if (s == nact - 1) {
+                staux(x.aux[0], q, d0, me[0], whole);
+                staux(x.aux[1], q, d1, me[1], whole);
+                staux(x.aux[2], q, d2, me[2], whole);
+                staux(x.aux[3], q, b0, mh[0], whole);
+                staux(x.aux[4], q, b1, mh[1], whole);
+                if (!(x.flags & kParity)) staux(x.aux[5], q, b2, mh[2], whole);
+            }
+        }
+        team_arrive(bar);
+        target += team.n_blocks;
+        if (!team_wait(bar, target, B.status, &gave_up)) return;
+    }
+    if (tid == 0 && nact > 0 && blk.first) *((volatile long long *)board->step) = B.step0 + nact;
+}
+
 }  // namespace
 
 size_t resident_smem(const ResPlan &p) { return (size_t)layout_of(p).bytes; }
 
 cudaError_t resident_set_smem_limit()
 {
-    return cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
+    const cudaError_t e = cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_pinned, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
 }
 
 size_t resident_arrive_bytes(int n_teams) { return (size_t)n_teams * 128; }
@@ -727,7 +928,9 @@ cudaError_t launch_resident(const ResPlan &plan, int nsteps, cudaStream_t st)
     if (e != cudaSuccess) return e;
     ResPlan p = plan;
     void *args[] = {&p, &nsteps};
-    return cudaLaunchCooperativeKernel((const void *)k_resident, dim3(plan.n_blocks), dim3(kResThreads), args,
+    const bool pin = plan.max_units <= kPinWarps;
+    const void *const kernel = pin ? (const void *)k_pinned : (const void *)k_resident;
+    return cudaLaunchCooperativeKernel(kernel, dim3(plan.n_blocks), dim3(pin ? kPinThreads : kResThreads), args,
                                        resident_smem(plan), st);
 }
 

@@ -84,23 +84,34 @@ struct ResHost {
     std::vector<ResBlock> blocks;
     std::vector<ResPiece> pieces;
     std::vector<ResPort> ports;
-    int max_pieces = 1, max_ports = 1, max_factors = 1;
+    int max_pieces = 1, max_ports = 1, max_factors = 1, max_units = 0;
 };
 
+// Whether a board's units fit nblk blocks at one a warp.
+inline bool res_pinned(const Board &h, int nblk)
+{
+    int units = 0;
+    for (int x = 0; x < res_boxes(h); ++x) units += ResRange(h, x).units();
+    return units <= nblk * kPinWarps;
+}
+
 // Add the team that advances board number b on nblk blocks: the boxes' units
-// go to the blocks in turn, each up to its share of the weight.
+// go to the blocks in turn, each up to its share of the weight, or of the
+// units' number where each warp keeps one unit.
 inline void res_team(const Board &h, const std::vector<ResAt> &at, int b, int nblk, ResHost &R)
 {
     const int nbox = res_boxes(h);
     std::vector<ResRange> box;
     for (int x = 0; x < nbox; ++x) box.emplace_back(h, x);
-    const double total = res_work(h);
+    const bool pinned = res_pinned(h, nblk);
+    double total = 0.0;
+    for (int x = 0; x < nbox; ++x) total += (double)box[x].units() * (pinned ? 1 : res_weight(h, x));
     std::vector<std::vector<ResPiece>> mine(nblk);
     std::vector<int> count(nblk, 0);
     double done = 0.0;
     int blk = 0;
     for (int x = 0; x < nbox; ++x) {
-        const int units = box[x].units(), w = res_weight(h, x);
+        const int units = box[x].units(), w = pinned ? 1 : res_weight(h, x);
         for (int u = 0; u < units;) {
             const double want = total * (blk + 1) / nblk;
             const int take = blk == nblk - 1 ? units - u
@@ -131,6 +142,7 @@ inline void res_team(const Board &h, const std::vector<ResAt> &at, int b, int nb
         R.blocks.push_back({team, q == 0, (int)R.pieces.size(), (int)mine[q].size(), (int)R.ports.size(), (int)port[q].size()});
         R.pieces.insert(R.pieces.end(), mine[q].begin(), mine[q].end());
         R.ports.insert(R.ports.end(), port[q].begin(), port[q].end());
+        R.max_units = std::max(R.max_units, count[q]);
         R.max_pieces = std::max(R.max_pieces, (int)mine[q].size());
         R.max_ports = std::max(R.max_ports, (int)port[q].size());
     }

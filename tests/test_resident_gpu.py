@@ -52,6 +52,12 @@ CASES = {
     "voltage": W.add_voltage_sources(_r(11, 37, 29, 23), [(10, 10, 10, 2), (10, 10, 10, 2)]),
     "many_ports": _ports(_r(14, 37, 29, 23), 3, 12, 150),
     "table1": W.table1_board(n_steps=80),
+    # past one unit a warp (the boards above but two have at most that)
+    "large_odd": _r(31, 97, 61, 43, upml=5, n_steps=40).replace(upml_kappa_max=5.0),
+    "large_pmc": _r(32, 121, 75, 31, upml=0, n_steps=40).replace(walls=(1,) * 6),
+    "large_mixed": _r(33, 118, 66, 44, upml=4, n_steps=40).replace(upml_depth=(4, 0, 3, 5, 0, 6), walls=(0, 1, 0, 0, 1, 0)),
+    "large_ports": _ports(_r(34, 97, 61, 43, upml=5, n_steps=40), 4, 12, 150),
+    "large_8bit": W.realistic_board(n_steps=40),
 }
 
 

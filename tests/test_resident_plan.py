@@ -118,7 +118,8 @@ int main()
                     bad += pieces != R.pieces.size() || ports != R.ports.size() || ports != at.size();
                     for (const auto &v : hit)
                         for (int n : v) bad += n != 1;
-                    bad += most > res_work(h) / nblk + 2 * heaviest;
+                    bad += !res_pinned(h, nblk) && most > res_work(h) / nblk + 2 * heaviest;
+                    bad += res_pinned(h, nblk) != (R.max_units <= kPinWarps);   // one unit a warp, or balanced
                     // ports: the node they name is theirs
                     std::map<int, int> seen;
                     for (const ResBlock &b : R.blocks)
