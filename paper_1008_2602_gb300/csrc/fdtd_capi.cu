@@ -314,10 +314,7 @@ bool layout_board(const fdtd_grid &g, const fdtd_boundary &bnd, const Axes &A, B
         sl.ni = sl.i1 - sl.i0; sl.nj = sl.j1 - sl.j0;
         sl.n = (long long)sl.ni * sl.nj * (sl.k1 - sl.k0);
         sl.block0 = blocks;
-        // threads: (i, j) columns marching z, or (i, k) columns marching y for a single plane
-        const long long cols = sl.k1 - sl.k0 == 1 ? (long long)sl.ni * ((sl.nj + kSlabKz - 1) / kSlabKz)
-                                                  : (long long)sl.ni * sl.nj * ((sl.k1 - sl.k0 + kSlabKz - 1) / kSlabKz);
-        blocks += (int)((cols + kSlabThreads - 1) / kSlabThreads);
+        blocks += (int)((slab_threads(sl) + kSlabThreads - 1) / kSlabThreads);
         const int lo[3] = {sl.i0, sl.j0, sl.k0}, hi[3] = {sl.i1, sl.j1, sl.k1};
         auto any_nontrivial = [&](int axis, int half, bool need_b1g, bool need_apam) {
             for (int t = lo[axis]; t < hi[axis]; ++t) {
@@ -379,9 +376,7 @@ void layout_band(Board &h)
         sl.n = (long long)sl.ni * sl.nj * (sl.k1 - sl.k0);
         sl.block0 = blocks;
         for (int a = 0; a < 6; ++a) sl.aux[a] = nullptr;
-        const long long cols = sl.k1 - sl.k0 == 1 ? (long long)sl.ni * ((sl.nj + kSlabKz - 1) / kSlabKz)
-                                                  : (long long)sl.ni * sl.nj * ((sl.k1 - sl.k0 + kSlabKz - 1) / kSlabKz);
-        blocks += (int)((cols + kSlabThreads - 1) / kSlabThreads);
+        blocks += (int)((slab_threads(sl) + kSlabThreads - 1) / kSlabThreads);
         if (b == 1) h.band_h_blocks = blocks - h.slab_blocks;
     }
     h.band_blocks = blocks - h.slab_blocks;

@@ -76,8 +76,7 @@ struct Slab {
     int ni, nj;                   // i1 - i0, j1 - j0
     long long n;                  // nodes in the box
     long long block0;             // first slab-kernel block of this slab (board-local)
-                                  // (blocks cover ni * nj * ceil(nk / kSlabKz) threads, or
-                                  // ni * ceil(nj / kSlabKz) for a single plane)
+                                  // (blocks cover slab_threads)
     float *aux[6];                // D~x, D~y, D~z, B~x, B~y, B~z or nullptr
 };
 
@@ -337,7 +336,13 @@ inline bool fused_maps_match(const Board &h, int tile_x, int tile_y)
 }
 
 constexpr int kSlabThreads = 128;
-constexpr int kSlabKz = 8;          // planes per slab-kernel thread
+constexpr int kSlabKz = 4;          // planes per slab-kernel thread
+constexpr int kSlabBlocks = 3;      // resident blocks per SM
+// Threads of a box: one per column quad (rows cut at multiples of four) and run of kSlabKz planes.
+inline long long slab_threads(const Slab &s)
+{
+    return (long long)((s.i1 - (s.i0 & ~3) + 3) / 4) * s.nj * ((s.k1 - s.k0 + kSlabKz - 1) / kSlabKz);
+}
 constexpr int kDftProbeGroup = 4;
 
 enum Phase : int { kPhaseSlabH = 0, kPhaseFusedZ = 1, kPhaseInterior = 2, kPhaseSlabE = 3, kPhasePost = 4, kNumPhases = 5 };

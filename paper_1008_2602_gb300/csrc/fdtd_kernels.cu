@@ -1243,416 +1243,238 @@ __global__ void __launch_bounds__(PairLayout<T>::THREADS, 2) k_pair(Plan plan)
 }
 
 // ------------------------------------------------------------------ slabs
-// A slab thread marches kSlabKz consecutive nodes of its slab: along z for
-// slabs more than one plane thick (an (i, j) column), along y for the two
-// single-plane z slabs (an (i, k) column).  Consecutive threads take
-// consecutive i, so rows are coalesced, and the per-column UPML factors and
-// index arithmetic are paid once per column.
-struct SlabCol {
+// The slab kernels update everything outside the fused region, box by box.  A
+// thread has a column quad (four nodes of a row, aligned to four) and marches
+// kSlabKz planes: the plane above of one step is the node's own plane of the
+// next, so a plane costs seven quads and two scalars (H) or seven and two and
+// the ids (E), plus the auxiliaries, as 16-byte loads (8-byte for 16-bit
+// storage) without staging.  Bound by the latency of those loads: 12 warps an
+// SM at 168 registers keep some 60 KB in flight.  (One node a thread with
+// 4-byte cp.async words into shared-memory rings, as before, took slab H + E
+// 68.5 + 82.6 us on the 880x680x100 board, now 56.5 + 66.9; FP16 at 480x380x100
+// 42.7 + 47.7, now 39.4 + 41.0.  Four blocks an SM at 128 registers spill: 58 +
+// 80; runs of 8 planes instead of 4: the same in FP32, 43.6 + 44.8 in FP16.)
+//
+// Neighbours past the grid's last column, row or plane, or before its first,
+// are read from the adjoining component's memory: in bounds (a set's six
+// components are contiguous and E comes first, so E never reads past them nor
+// H~ before them), and used only by samples that do not exist or replaced by
+// the wall's image.
+struct SlabThread {
+    const Board *B;
     const Slab *sl;
-    long long t;          // slab-local (aux) index of the first node; + tstep per node
-    int tstep;
-    bool ym;              // marching along y (else z)
-    int i, j, k, count;   // first node, nodes to march
+    int in, out;          // field sets
+    int i, j, k, count;   // first node of the quad, planes to march
+    unsigned own;         // bit q: node i + q belongs to the box
+    int ax, astep;        // auxiliary index of node i (may lie before the box's first column), per plane
+    bool whole, gx;       // 16-byte auxiliary accesses; factors along x
+    bool walls, low;      // see slab walls
 };
 
-// Block set-up from the plan's per-block descriptor: the step counters, the
-// slab's box and every set's field pointers are independent loads.
-template <typename T>
-__device__ __forceinline__ bool slab_locate(const Plan &plan, long long blk, const Board *&B, SlabCol &sc,
-                                            Fields<T> &F)
+__device__ __forceinline__ bool slab_locate(const Plan &plan, long long blk, SlabThread &t)
 {
     const SlabBlock d = plan.slab_blk[blk];
-    B = d.B;
+    const Board *const B = t.B = d.B;
     const long long step = __ldg(d.step), stop = __ldg(d.stop);
-    const Slab *sl = &B->slab[d.slab];
-    const int ni = sl->ni, nj = sl->nj, i0 = sl->i0, j0 = sl->j0, k0 = sl->k0, k1 = sl->k1, j1 = sl->j1;
-    const void *f0[6], *f1[6], *f2[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        f0[c] = B->f[0][c];
-        f1[c] = B->f[1][c];
-        f2[c] = B->f[2][c];
-    }
-    const int depth = B->tdepth;
+    const Slab *const sl = t.sl = &B->slab[d.slab];
+    const int i0 = sl->i0, i1 = sl->i1, j0 = sl->j0, k0 = sl->k0, k1 = sl->k1, nj = sl->nj, ni = sl->ni;
+    const int depth = B->tdepth, nx = B->nx, ny = B->ny, nz = B->nz;
     if (step >= stop) return false;
-    const bool ym = (k1 - k0 == 1);
-    const int nij = ni * nj;
-    const int tt = d.t0 + (int)threadIdx.x;
-    if (ym) {
-        const int nrow = (nj + kSlabKz - 1) / kSlabKz;
-        if (tt >= ni * nrow) return false;
-        const int jr = tt / ni, ii = tt - jr * ni;
-        sc.i = i0 + ii;
-        sc.j = j0 + jr * kSlabKz;
-        sc.k = k0;
-        sc.count = min(kSlabKz, j1 - sc.j);
-        sc.t = (long long)jr * kSlabKz * ni + ii;
-        sc.tstep = ni;
-    } else {
-        const int nkz = (k1 - k0 + kSlabKz - 1) / kSlabKz;
-        if (tt >= nij * nkz) return false;
-        const int kz = tt / nij, ij = tt - kz * nij;
-        const int jj = ij / ni;
-        sc.i = i0 + (ij - jj * ni);
-        sc.j = j0 + jj;
-        sc.k = k0 + kz * kSlabKz;
-        sc.count = min(kSlabKz, k1 - sc.k);
-        sc.t = (long long)kz * kSlabKz * nij + ij;
-        sc.tstep = nij;
-    }
-    sc.ym = ym;
-    sc.sl = sl;
-    const int si = set_of(depth, step), so = set_of(depth, step + 1);
-    auto pick = [&](int set, int c) -> const void * { return set == 0 ? f0[c] : (set == 1 ? f1[c] : f2[c]); };
-    F.ex = (const T *)pick(si, 0); F.ey = (const T *)pick(si, 1); F.ez = (const T *)pick(si, 2);
-    F.hx = (const T *)pick(si, 3); F.hy = (const T *)pick(si, 4); F.hz = (const T *)pick(si, 5);
-    F.oex = (T *)pick(so, 0); F.oey = (T *)pick(so, 1); F.oez = (T *)pick(so, 2);
-    F.ohx = (T *)pick(so, 3); F.ohy = (T *)pick(so, 4); F.ohz = (T *)pick(so, 5);
+    const int ie = i0 & ~3, np = (i1 - ie + 3) >> 2;
+    const int tt = d.t0 + (int)threadIdx.x, r = tt / np, kz = r / nj;
+    if (kz * kSlabKz >= k1 - k0) return false;
+    t.i = ie + 4 * (tt - r * np);
+    t.j = j0 + r - kz * nj;
+    t.k = k0 + kz * kSlabKz;
+    t.count = min(kSlabKz, k1 - t.k);
+    t.own = (15u << max(i0 - t.i, 0)) & (15u >> max(t.i + 4 - i1, 0)) & 15u;
+    t.ax = ((t.k - k0) * nj + (t.j - j0)) * ni + (t.i - i0);
+    t.astep = ni * nj;
+    t.whole = ((i0 | i1 | ni) & 3) == 0;
+    t.gx = i0 < B->depth[0] || i1 > nx - B->depth[1];
+    const int *const w = B->wall;
+    t.walls = i1 > nx || sl->j1 > ny || k1 > nz || (i0 == 0 && w[0]) || (j0 == 0 && w[2]) || (k0 == 0 && w[4]);
+    t.low = !t.walls && (i0 == 0 || j0 == 0 || k0 == 0);
+    t.in = set_of(depth, step);
+    t.out = set_of(depth, step + 1);
     return true;
 }
 
-// Gedney two-step update of one H~ component (B~ recurrence along w+1, H~
-// recurrence along w+2, B~->H~ along w).  scurl = S * (curl E)_w.
-__device__ __forceinline__ float upml_h(float h, float scurl, const Coef &a, const Coef &bb, const Coef &c,
-                                        float *aux, long long t)
+// Auxiliaries of a quad (only the box's own nodes lie in the array).
+__device__ __forceinline__ F4 slab_aux(const float *p, int at, unsigned own, bool whole)
 {
-    if (aux) {
-        const float Bo = aux[t];
-        const float Bn = __fmaf_rn(-a.g, scurl, __fmul_rn(a.b1, Bo));
-        aux[t] = Bn;
-        return __fmaf_rn(bb.g, __fmaf_rn(c.ap, Bn, -__fmul_rn(c.am, Bo)), __fmul_rn(bb.b1, h));
+    if (!p) return four(0.f);
+    p += at;
+    if (whole) return ld4(p);
+    F4 v = four(0.f);
+    if (own & 1u) v.a.x = p[0];
+    if (own & 2u) v.a.y = p[1];
+    if (own & 4u) v.b.x = p[2];
+    if (own & 8u) v.b.y = p[3];
+    return v;
+}
+__device__ __forceinline__ void slab_staux(float *p, int at, const F4 &v, unsigned own, bool whole)
+{
+    if (!p) return;
+    p += at;
+    if (whole) {
+        st4(p, v, own);
+        return;
     }
-    return __fmaf_rn(-bb.g, scurl, __fmul_rn(bb.b1, h));
+    if (own & 1u) p[0] = v.a.x;
+    if (own & 2u) p[1] = v.a.y;
+    if (own & 4u) p[2] = v.b.x;
+    if (own & 8u) p[3] = v.b.y;
 }
 
-// Same for E (D~ recurrence along w+1, E recurrence along w+2, D~->E along
-// w); ce = 1/eps_r of the edge (0 on PEC).
-__device__ __forceinline__ float upml_e(float e, float scurl, float ce, const Coef &a, const Coef &bb,
-                                        const Coef &c, float *aux, long long t)
+// Factors of a row along y or z, and of a quad along x (1 where not graded).
+__device__ __forceinline__ C4 row_factors(const Coef *p)
 {
-    if (aux) {
-        const float Do = aux[t];
-        const float Dn = __fmaf_rn(a.g, scurl, __fmul_rn(a.b1, Do));
-        aux[t] = Dn;
-        return __fmaf_rn(__fmul_rn(ce, bb.g), __fmaf_rn(c.ap, Dn, -__fmul_rn(c.am, Do)), __fmul_rn(bb.b1, e));
-    }
-    return __fmaf_rn(__fmul_rn(ce, bb.g), scurl, __fmul_rn(bb.b1, e));
+    const Coef c = ldcoef(p);
+    return C4{four(c.b1), four(c.g), four(c.ap), four(c.am)};
 }
-
-// The slab kernels issue every load of a node unconditionally, with the
-// offsets of neighbours that do not exist (i = nx, j = ny, k = nz, or the
-// image across an outer wall) clamped to an in-bounds node; only the stores
-// are conditional.  A thread streams the inputs of its next nodes into a
-// per-thread ring of shared-memory slots with cp.async (one commit group
-// per node), so several nodes' loads are in flight while it updates the
-// current one, without holding them in registers.
-
-// cp.async of the 32-bit word at src (4-byte aligned) into shared memory.
-__device__ __forceinline__ void cp_word(float *dst, const void *src)
+__device__ __forceinline__ C4 quad_factors(const Coef *p, int i, int n, bool graded)
 {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+    if (!graded) return fac_one();
+    const Coef a = ldcoef(p + i), b = ldcoef(p + min(i + 1, n)), c = ldcoef(p + min(i + 2, n)), d = ldcoef(p + min(i + 3, n));
+    return C4{F4{make_float2(a.b1, b.b1), make_float2(c.b1, d.b1)}, F4{make_float2(a.g, b.g), make_float2(c.g, d.g)},
+              F4{make_float2(a.ap, b.ap), make_float2(c.ap, d.ap)}, F4{make_float2(a.am, b.am), make_float2(c.am, d.am)}};
 }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// Storage element <-> 32-bit word: a 16-bit element is copied with its
-// neighbour (the aligned word holding it) and picked by its index parity.
-// Field arrays start 128-byte aligned and node offsets keep the element
-// index, so the parity of the node index selects the half.
-template <typename T>
-struct Word;
-template <>
-struct Word<float> {
-    static __device__ __forceinline__ const void *at(const float *p) { return p; }
-    static __device__ __forceinline__ float get(float w, long long) { return w; }
-};
-template <>
-struct Word<__half> {
-    static __device__ __forceinline__ const void *at(const __half *p)
-    {
-        return (const void *)((uintptr_t)p & ~(uintptr_t)3);
-    }
-    static __device__ __forceinline__ float get(float w, long long e)
-    {
-        const unsigned b = __float_as_uint(w);
-        return __half2float(__ushort_as_half((unsigned short)((e & 1) ? b >> 16 : b & 0xffffu)));
-    }
-};
-
-// Coefficient id of node idx from the word holding it (8- or 16-bit ids).
-__device__ __forceinline__ const void *cid_word(const void *cid, int id16, long long idx)
-{
-    return id16 ? (const void *)((uintptr_t)((const uint16_t *)cid + idx) & ~(uintptr_t)3)
-                : (const void *)((uintptr_t)((const uint8_t *)cid + idx) & ~(uintptr_t)3);
-}
-__device__ __forceinline__ int cid_get(int id16, float w, long long idx)
-{
-    const unsigned b = __float_as_uint(w);
-    return id16 ? (int)((idx & 1) ? b >> 16 : b & 0xffffu) : (int)((b >> (8 * (int)(idx & 3))) & 0xffu);
-}
-
-// Ring slots per thread (nodes in flight + 1), words per node and resident
-// blocks per SM of the two slab kernels; the rings are sized so that the
-// blocks' shared memory fits an SM.  With 128-thread blocks, four nodes in
-// flight per thread at the same occupancy measured 2 % faster than three
-// with 256-thread blocks.
-constexpr int kSlabHStages = 5, kSlabHWords = 15, kSlabHBlocks = 5;
-constexpr int kSlabEStages = 5, kSlabEWords = 16, kSlabEBlocks = 4;
-constexpr int kSlabHSmem = kSlabHStages * kSlabHWords * kSlabThreads * 4;
-constexpr int kSlabESmem = kSlabEStages * kSlabEWords * kSlabThreads * 4;
-static_assert(kSlabHBlocks * (kSlabHSmem + 1024) <= 232448 && kSlabEBlocks * (kSlabESmem + 1024) <= 232448,
-              "slab rings exceed an SM's shared memory");
-
-// Slot w of node m in a thread's ring of S slots of NW words (words of one
-// slot are kSlabThreads apart, so a warp's accesses to a word are conflict-free).
-template <int S, int NW>
-__device__ __forceinline__ float *ring_at(float *my, int m, int w)
-{
-    return my + ((m % S) * NW + w) * kSlabThreads;
-}
-
-enum SlabHWord { hEYC, hEXC, hEYU, hEXU, hEZC, hEZJ, hEZI, hEYI, hEXJ, hHX, hHY, hHZ, hBX, hBY, hBZ };
 
 template <typename T>
-__global__ void __launch_bounds__(kSlabThreads, kSlabHBlocks) k_slab_h(Plan plan)
+__global__ void __launch_bounds__(kSlabThreads, kSlabBlocks) k_slab_h(Plan plan)
 {
-    extern __shared__ float slab_ring[];
-    float *const my = slab_ring + threadIdx.x;
     for (long long blk = blockIdx.x; blk < plan.n_slab; blk += gridDim.x) {
-        const Board *B;
-        SlabCol sc;
-        Fields<T> F;
-        if (!slab_locate(plan, blk, B, sc, F)) continue;
-        const int i = sc.i, ny = B->ny, nz = B->nz;
-        const int X = B->pitch;
-        const long long P = B->plane;
+        SlabThread t;
+        if (!slab_locate(plan, blk, t)) continue;
+        const Board *const B = t.B;
+        const int X = B->pitch, nx = B->nx, ny = B->ny, nz = B->nz;
+        const long long P = B->plane, N = B->nodes;
         const float Sx = B->S[0], Sy = B->S[1], Sz = B->S[2];
-        const Slab &sl = *sc.sl;
-        float *const ax = sl.aux[3], *const ay = sl.aux[4], *const az = sl.aux[5];
-        const bool xin = i < B->nx;
-        const int di = xin ? 1 : 0;   // clamped +x neighbour offset
-        // x factors fixed along the column: H_x (x integer), H_y, H_z (x half)
-        const Coef x0 = B->cw[0][0][i], x1 = B->cw[0][1][i];
-        const int j0 = sc.j, k0 = sc.k, cnt = sc.count;
-        const bool ym = sc.ym;
-        const long long idx0 = (long long)k0 * P + (long long)j0 * X + i;
-        const long long didx = ym ? X : P;
-        // y and z factors: only the marching axis' change from node to node
-        const Coef *const cy0 = B->cw[1][0], *const cy1 = B->cw[1][1];
-        const Coef *const cz0 = B->cw[2][0], *const cz1 = B->cw[2][1];
-        Coef y0 = ldcoef(cy0 + j0), y1 = ldcoef(cy1 + j0), z0 = ldcoef(cz0 + k0), z1 = ldcoef(cz1 + k0);
-        // issue the loads of node m (empty group past the column's end)
-        auto issue = [&](int m) {
-            if (m < cnt) {
-                const long long idx = idx0 + m * didx, t = sc.t + (long long)m * sc.tstep;
-                const int j = ym ? j0 + m : j0, k = ym ? k0 : k0 + m;
-                const int dj = j < ny ? X : 0;
-                const long long dk = k < nz ? P : 0;
-                if (ym || m == 0) {   // marching z, E_y and E_x at the node are the previous +z loads
-                    cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEYC), Word<T>::at(F.ey + idx));
-                    cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEXC), Word<T>::at(F.ex + idx));
-                }
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEYU), Word<T>::at(F.ey + idx + dk));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEXU), Word<T>::at(F.ex + idx + dk));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEZC), Word<T>::at(F.ez + idx));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEZJ), Word<T>::at(F.ez + idx + dj));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEZI), Word<T>::at(F.ez + idx + di));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEYI), Word<T>::at(F.ey + idx + di));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hEXJ), Word<T>::at(F.ex + idx + dj));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hHX), Word<T>::at(F.hx + idx));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hHY), Word<T>::at(F.hy + idx));
-                cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hHZ), Word<T>::at(F.hz + idx));
-                if (ax) cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hBX), ax + t);
-                if (ay) cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hBY), ay + t);
-                if (az) cp_word(ring_at<kSlabHStages, kSlabHWords>(my, m, hBZ), az + t);
+        float *const a0 = t.sl->aux[3], *const a1 = t.sl->aux[4], *const a2 = t.sl->aux[5];
+        const long long at = (long long)t.k * P + (long long)t.j * X + t.i;
+        const T *e = (const T *)B->f[t.in][0] + at;   // E_x of the quad; the other components N apart
+        T *o = (T *)B->f[t.out][0] + (at + 3 * N);
+        const C4 x0 = quad_factors(B->cw[0][0], t.i, nx, t.gx), x1 = quad_factors(B->cw[0][1], t.i, nx, t.gx);
+        const Coef *const fy0 = B->cw[1][0] + t.j, *const fy1 = B->cw[1][1] + t.j, *fz0 = B->cw[2][0] + t.k, *fz1 = B->cw[2][1] + t.k;
+        F4 ex = ld4(e), ey = ld4(e + N);
+        int ax = t.ax;
+        for (int m = 0; m < t.count; ++m, e += P, o += P, ax += t.astep) {
+            const F4 exk = ld4(e + P), eyk = ld4(e + N + P);
+            const F4 ez = ld4(e + 2 * N), exj = ld4(e + X), ezj = ld4(e + 2 * N + X);
+            const float eyi = Io<T>::ldw(e + N + 4), ezi = Io<T>::ldw(e + 2 * N + 4);
+            const F4 hx = ld4(e + 3 * N), hy = ld4(e + 4 * N), hz = ld4(e + 5 * N);
+            const F4 b0 = slab_aux(a0, ax, t.own, t.whole), b1 = slab_aux(a1, ax, t.own, t.whole), b2 = slab_aux(a2, ax, t.own, t.whole);
+            const int k = t.k + m;
+            const C4 y0 = row_factors(fy0), y1 = row_factors(fy1), z0 = row_factors(fz0 + m), z1 = row_factors(fz1 + m);
+            unsigned mx = t.own, my = t.own, mz = t.own;
+            if (t.walls) {   // samples that exist: not past the last row, column or plane
+                const unsigned xin = below(t.i, nx);
+                if (!(t.j < ny && k < nz)) mx = 0;
+                my = k < nz ? my & xin : 0u;
+                mz = t.j < ny ? mz & xin : 0u;
             }
-            cp_commit();
-        };
-#pragma unroll
-        for (int m = 0; m < kSlabHStages - 1; ++m) issue(m);
-        float eyc = 0.f, exc = 0.f;   // E_y, E_x at the node (carried along z)
-#pragma unroll
-        for (int m = 0; m < kSlabKz; ++m) {
-            if (m >= cnt) break;
-            issue(m + kSlabHStages - 1);
-            cp_wait<kSlabHStages - 1>();
-            const long long idx = idx0 + m * didx, t = sc.t + (long long)m * sc.tstep;
-            const int j = ym ? j0 + m : j0, k = ym ? k0 : k0 + m;
-            const int dj = j < ny ? X : 0;
-            const long long dk = k < nz ? P : 0;
-            auto w = [&](int word) { return *ring_at<kSlabHStages, kSlabHWords>(my, m, word); };
-            if (ym || m == 0) {
-                eyc = Word<T>::get(w(hEYC), idx);
-                exc = Word<T>::get(w(hEXC), idx);
-            }
-            const float eyu = Word<T>::get(w(hEYU), idx + dk), exu = Word<T>::get(w(hEXU), idx + dk);
-            const float ezc = Word<T>::get(w(hEZC), idx);
-            const float ezj = Word<T>::get(w(hEZJ), idx + dj), ezi = Word<T>::get(w(hEZI), idx + di);
-            const float eyi = Word<T>::get(w(hEYI), idx + di), exj = Word<T>::get(w(hEXJ), idx + dj);
-            const float hxo = Word<T>::get(w(hHX), idx), hyo = Word<T>::get(w(hHY), idx);
-            const float hzo = Word<T>::get(w(hHZ), idx);
-            const bool yin = j < ny, zin = k < nz;
-            if (m > 0) {
-                if (ym) { y0 = ldcoef(cy0 + j); y1 = ldcoef(cy1 + j); }
-                else { z0 = ldcoef(cz0 + k); z1 = ldcoef(cz1 + k); }
-            }
-            float bn;
-            if (yin && zin) {   // H_x(i, j+1/2, k+1/2)
-                const float h = upml_h2(hxo, curl2(ezj, ezc, eyu, eyc, Sy, Sz), y1, z1, x0, ax != nullptr,
-                                        ax ? w(hBX) : 0.f, bn);
-                Io<T>::st(F.ohx + idx, h);
-                if (ax) ax[t] = bn;
-            }
-            if (xin && zin) {   // H_y(i+1/2, j, k+1/2)
-                const float h = upml_h2(hyo, curl2(exu, exc, ezi, ezc, Sz, Sx), z1, x1, y0, ay != nullptr,
-                                        ay ? w(hBY) : 0.f, bn);
-                Io<T>::st(F.ohy + idx, h);
-                if (ay) ay[t] = bn;
-            }
-            if (xin && yin) {   // H_z(i+1/2, j+1/2, k)
-                const float h = upml_h2(hzo, curl2(eyi, eyc, exj, exc, Sx, Sy), x1, y1, z0, az != nullptr,
-                                        az ? w(hBZ) : 0.f, bn);
-                Io<T>::st(F.ohz + idx, h);
-                if (az) az[t] = bn;
-            }
-            eyc = eyu;
-            exc = exu;
+            F4 n;
+            F4 h = upml_h4(hx, curl4(ezj, ez, eyk, ey, Sy, Sz), y1, z1, x0, a0 != nullptr, b0, n);
+            st4(o, h, mx);
+            slab_staux(a0, ax, n, mx, t.whole);
+            h = upml_h4(hy, curl4(exk, ex, F4{make_float2(ez.a.y, ez.b.x), make_float2(ez.b.y, ezi)}, ez, Sz, Sx), z1, x1, y0,
+                        a1 != nullptr, b1, n);
+            st4(o + N, h, my);
+            slab_staux(a1, ax, n, my, t.whole);
+            h = upml_h4(hz, curl4(F4{make_float2(ey.a.y, ey.b.x), make_float2(ey.b.y, eyi)}, ey, exj, ex, Sx, Sy), x1, y1, z0,
+                        a2 != nullptr, b2, n);
+            st4(o + 2 * N, h, mz);
+            slab_staux(a2, ax, n, mz, t.whole);
+            ex = exk;
+            ey = eyk;
         }
-        cp_wait<0>();   // no copy into the ring may be outstanding when the next block reuses it
     }
 }
 
-// Ring words of a slab E node: H~ at the node and at its -x, -y, -z
-// neighbours (each loaded once; a neighbour across the low wall is clamped to
-// the node itself, and the image of H~ across a high wall is the -x/-y/-z
-// neighbour's value, picked after the load), E^n, the D~ auxiliaries, the id.
-enum SlabEWord { eHZ, eHZJ, eHZI, eHY, eHYI, eHYK, eHX, eHXJ, eHXK, eEX, eEY, eEZ, eDX, eDY, eDZ, eID };
-
 template <typename T>
-__global__ void __launch_bounds__(kSlabThreads, kSlabEBlocks) k_slab_e(Plan plan)
+__global__ void __launch_bounds__(kSlabThreads, kSlabBlocks) k_slab_e(Plan plan)
 {
-    extern __shared__ float slab_ring[];
-    float *const my = slab_ring + threadIdx.x;
     for (long long blk = blockIdx.x; blk < plan.n_slab; blk += gridDim.x) {
-        const Board *B;
-        SlabCol sc;
-        Fields<T> F;
-        if (!slab_locate(plan, blk, B, sc, F)) continue;
-        const int i = sc.i;
-        const int nx = B->nx, ny = B->ny, nz = B->nz;
-        const int X = B->pitch;
-        const long long P = B->plane;
+        SlabThread t;
+        if (!slab_locate(plan, blk, t)) continue;
+        const Board *const B = t.B;
+        const int X = B->pitch, nx = B->nx, ny = B->ny, nz = B->nz;
+        const long long P = B->plane, N = B->nodes;
         const float Sx = B->S[0], Sy = B->S[1], Sz = B->S[2];
-        const Slab &sl = *sc.sl;
-        float *const ax = sl.aux[0], *const ay = sl.aux[1], *const az = sl.aux[2];
-        const int *wl = B->wall;
-        const int w2 = wl[2], w3 = wl[3], w4 = wl[4], w5 = wl[5];
-        // images across the x walls (fixed along the column)
-        const bool xhi = i == nx, xlo = i == 0;
-        const float sxh = hsign(xhi, wl[1]), sxl = hsign(xlo, wl[0]);
-        const int ox0 = xlo ? 0 : -1;   // offset of H at i-1 (clamped at the low wall)
-        // x factors fixed along the column: E_x (x half), E_y, E_z (x integer)
-        const Coef x1 = B->cw[0][1][i], x0 = B->cw[0][0][i];
-        const int j0 = sc.j, k0 = sc.k, cnt = sc.count;
-        const bool ym = sc.ym;
-        const long long idx0 = (long long)k0 * P + (long long)j0 * X + i;
-        const long long didx = ym ? X : P;
-        const Coef *const cy0 = B->cw[1][0], *const cy1 = B->cw[1][1];
-        const Coef *const cz0 = B->cw[2][0], *const cz1 = B->cw[2][1];
-        Coef y0 = ldcoef(cy0 + j0), y1 = ldcoef(cy1 + j0), z0 = ldcoef(cz0 + k0), z1 = ldcoef(cz1 + k0);
-        const void *const cid = B->cid;
+        float *const a0 = t.sl->aux[0], *const a1 = t.sl->aux[1], *const a2 = t.sl->aux[2];
+        const long long at = (long long)t.k * P + (long long)t.j * X + t.i;
+        const T *e = (const T *)B->f[t.in][0] + at;
+        T *o = (T *)B->f[t.out][0] + at;
         const int id16 = B->id16;
+        const unsigned char *cid = (const unsigned char *)B->cid + (id16 ? 2 * at : at);
         const float4 *const ctab = B->ctab;
-        auto issue = [&](int m) {
-            if (m < cnt) {
-                const long long idx = idx0 + m * didx, t = sc.t + (long long)m * sc.tstep;
-                const int j = ym ? j0 + m : j0, k = ym ? k0 : k0 + m;
-                const int oy0 = j == 0 ? 0 : -X;
-                const long long oz0 = k == 0 ? 0 : -P;
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eID), cid_word(cid, id16, idx));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHZ), Word<T>::at(F.ohz + idx));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHZJ), Word<T>::at(F.ohz + idx + oy0));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHZI), Word<T>::at(F.ohz + idx + ox0));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHY), Word<T>::at(F.ohy + idx));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHYI), Word<T>::at(F.ohy + idx + ox0));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHX), Word<T>::at(F.ohx + idx));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHXJ), Word<T>::at(F.ohx + idx + oy0));
-                if (ym || m == 0) {   // marching z, H~y and H~x at -z are the previous node's values
-                    cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHYK), Word<T>::at(F.ohy + idx + oz0));
-                    cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eHXK), Word<T>::at(F.ohx + idx + oz0));
+        const C4 x0 = quad_factors(B->cw[0][0], t.i, nx, t.gx), x1 = quad_factors(B->cw[0][1], t.i, nx, t.gx);
+        const Coef *const fy0 = B->cw[1][0] + t.j, *const fy1 = B->cw[1][1] + t.j, *fz0 = B->cw[2][0] + t.k, *fz1 = B->cw[2][1] + t.k;
+        F4 hxk = ld4(o + 3 * N - P), hyk = ld4(o + 4 * N - P);   // H~ of the plane below
+        int ax = t.ax;
+        for (int m = 0; m < t.count; ++m, e += P, o += P, cid += id16 ? 2 * P : P, ax += t.astep) {
+            uint2 id = make_uint2(0, 0);
+            if (id16) id = *reinterpret_cast<const uint2 *>(cid);
+            else id.x = *reinterpret_cast<const unsigned *>(cid);
+            const F4 hx = ld4(o + 3 * N), hy = ld4(o + 4 * N), hz = ld4(o + 5 * N);
+            const float hyi = Io<T>::ldw(o + 4 * N - 1), hzi = Io<T>::ldw(o + 5 * N - 1);
+            F4 hxj = ld4(o + 3 * N - X), hzj = ld4(o + 5 * N - X);
+            const F4 ex = ld4(e), ey = ld4(e + N), ez = ld4(e + 2 * N);
+            const F4 d0 = slab_aux(a0, ax, t.own, t.whole), d1 = slab_aux(a1, ax, t.own, t.whole), d2 = slab_aux(a2, ax, t.own, t.whole);
+            const int k = t.k + m;
+            const C4 y0 = row_factors(fy0), y1 = row_factors(fy1), z0 = row_factors(fz0 + m), z1 = row_factors(fz1 + m);
+            F4 hyl{make_float2(hyi, hy.a.x), make_float2(hy.a.y, hy.b.x)};   // H~y, H~z at i - 1
+            F4 hzl{make_float2(hzi, hz.a.x), make_float2(hz.a.y, hz.b.x)};
+            unsigned mx = t.own, my = t.own, mz = t.own;
+            F4 cx, cy, cz;
+            if (t.walls) {
+                // H~ on the + side of the node, per axis of difference
+                F4 hyx = hy, hzx = hz, hxy = hx, hzy = hz, hxz = hx, hyz = hy;
+                const int *const w = B->wall;
+                image_x(t.i, nx, w[0], w[1], hyx, hyl);
+                image_x(t.i, nx, w[0], w[1], hzx, hzl);
+                image4(t.j == 0, t.j == ny, w[2], w[3], hxy, hxj);
+                image4(t.j == 0, t.j == ny, w[2], w[3], hzy, hzj);
+                image4(k == 0, k == nz, w[4], w[5], hxz, hxk);
+                image4(k == 0, k == nz, w[4], w[5], hyz, hyk);
+                cx = curl4(hzy, hzj, hyz, hyk, Sy, Sz);
+                cy = curl4(hxz, hxk, hzx, hzl, Sz, Sx);
+                cz = curl4(hyx, hyl, hxy, hxj, Sx, Sy);
+                mx &= below(t.i, nx);
+                if (t.j >= ny) my = 0;
+                if (k >= nz) mz = 0;
+            } else {
+                if (t.low) {   // what lies across a low PEC wall counts as 0
+                    if (t.i == 0) hyl.a.x = hzl.a.x = 0.f;
+                    if (t.j == 0) hxj = hzj = four(0.f);
+                    if (k == 0) hxk = hyk = four(0.f);
                 }
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eEX), Word<T>::at(F.ex + idx));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eEY), Word<T>::at(F.ey + idx));
-                cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eEZ), Word<T>::at(F.ez + idx));
-                if (ax) cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eDX), ax + t);
-                if (ay) cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eDY), ay + t);
-                if (az) cp_word(ring_at<kSlabEStages, kSlabEWords>(my, m, eDZ), az + t);
+                cx = curl4(hz, hzj, hy, hyk, Sy, Sz);
+                cy = curl4(hx, hxk, hz, hzl, Sz, Sx);
+                cz = curl4(hy, hyl, hx, hxj, Sx, Sy);
             }
-            cp_commit();
-        };
-#pragma unroll
-        for (int m = 0; m < kSlabEStages - 1; ++m) issue(m);
-        float hyk = 0.f, hxk = 0.f;   // H~y, H~x at -z (carried along z)
-#pragma unroll
-        for (int m = 0; m < kSlabKz; ++m) {
-            if (m >= cnt) break;
-            issue(m + kSlabEStages - 1);
-            cp_wait<kSlabEStages - 1>();
-            const long long idx = idx0 + m * didx, t = sc.t + (long long)m * sc.tstep;
-            const int j = ym ? j0 + m : j0, k = ym ? k0 : k0 + m;
-            const int oy0 = j == 0 ? 0 : -X;
-            const long long oz0 = k == 0 ? 0 : -P;
-            auto w = [&](int word) { return *ring_at<kSlabEStages, kSlabEWords>(my, m, word); };
-            const bool yhi = j == ny, ylo = j == 0, zhi = k == nz, zlo = k == 0;
-            const float syh = hsign(yhi, w3), syl = hsign(ylo, w2), szh = hsign(zhi, w5), szl = hsign(zlo, w4);
-            const float4 ce = __ldg(ctab + cid_get(id16, w(eID), idx));
-            if (m > 0) {
-                if (ym) { y0 = ldcoef(cy0 + j); y1 = ldcoef(cy1 + j); }
-                else { z0 = ldcoef(cz0 + k); z1 = ldcoef(cz1 + k); }
+            float4 r0, r1, r2, r3;   // 1 / eps_r of the quad's edges
+            if (id16) {
+                r0 = __ldg(ctab + (id.x & 0xffffu)); r1 = __ldg(ctab + (id.x >> 16));
+                r2 = __ldg(ctab + (id.y & 0xffffu)); r3 = __ldg(ctab + (id.y >> 16));
+            } else {
+                r0 = __ldg(ctab + (id.x & 0xffu)); r1 = __ldg(ctab + ((id.x >> 8) & 0xffu));
+                r2 = __ldg(ctab + ((id.x >> 16) & 0xffu)); r3 = __ldg(ctab + (id.x >> 24));
             }
-            if (ym || m == 0) {
-                hyk = Word<T>::get(w(eHYK), idx + oz0);
-                hxk = Word<T>::get(w(eHXK), idx + oz0);
-            }
-            const float hz = Word<T>::get(w(eHZ), idx), hzj = Word<T>::get(w(eHZJ), idx + oy0);
-            const float hzi = Word<T>::get(w(eHZI), idx + ox0);
-            const float hy = Word<T>::get(w(eHY), idx), hyi = Word<T>::get(w(eHYI), idx + ox0);
-            const float hx = Word<T>::get(w(eHX), idx), hxj = Word<T>::get(w(eHXJ), idx + oy0);
-            float dn;
-            if (i < nx) {   // E_x(i+1/2, j, k)
-                const float e = upml_e2(Word<T>::get(w(eEX), idx),
-                                        curl2(syh * (yhi ? hzj : hz), syl * hzj, szh * (zhi ? hyk : hy), szl * hyk,
-                                              Sy, Sz),
-                                        ce.x, y0, z0, x1, ax != nullptr, ax ? w(eDX) : 0.f, dn);
-                Io<T>::st(F.oex + idx, e);
-                if (ax) ax[t] = dn;
-            }
-            if (j < ny) {   // E_y(i, j+1/2, k)
-                const float e = upml_e2(Word<T>::get(w(eEY), idx),
-                                        curl2(szh * (zhi ? hxk : hx), szl * hxk, sxh * (xhi ? hzi : hz), sxl * hzi,
-                                              Sz, Sx),
-                                        ce.y, z0, x0, y1, ay != nullptr, ay ? w(eDY) : 0.f, dn);
-                Io<T>::st(F.oey + idx, e);
-                if (ay) ay[t] = dn;
-            }
-            if (k < nz) {   // E_z(i, j, k+1/2)
-                const float e = upml_e2(Word<T>::get(w(eEZ), idx),
-                                        curl2(sxh * (xhi ? hyi : hy), sxl * hyi, syh * (yhi ? hxj : hx), syl * hxj,
-                                              Sx, Sy),
-                                        ce.z, x0, y0, z1, az != nullptr, az ? w(eDZ) : 0.f, dn);
-                Io<T>::st(F.oez + idx, e);
-                if (az) az[t] = dn;
-            }
-            hyk = hy;   // the next node (k + 1 <= nz) reads H at k
+            F4 n;
+            F4 v = upml_e4(ex, cx, F4{make_float2(r0.x, r1.x), make_float2(r2.x, r3.x)}, y0, z0, x1, a0 != nullptr, d0, n);
+            st4(o, v, mx);
+            slab_staux(a0, ax, n, mx, t.whole);
+            v = upml_e4(ey, cy, F4{make_float2(r0.y, r1.y), make_float2(r2.y, r3.y)}, z0, x0, y1, a1 != nullptr, d1, n);
+            st4(o + N, v, my);
+            slab_staux(a1, ax, n, my, t.whole);
+            v = upml_e4(ez, cz, F4{make_float2(r0.z, r1.z), make_float2(r2.z, r3.z)}, x0, y0, z1, a2 != nullptr, d2, n);
+            st4(o + 2 * N, v, mz);
+            slab_staux(a2, ax, n, mz, t.whole);
             hxk = hx;
+            hyk = hy;
         }
-        cp_wait<0>();
     }
 }
 
@@ -1984,7 +1806,7 @@ static cudaError_t phase_t(const Plan &plan, int phase, int grid_cap, cudaStream
     switch (phase) {
     case kPhaseSlabH:
         if (plan.n_slab > 0)
-            k_slab_h<T><<<(int)(plan.n_slab < kMaxGrid ? plan.n_slab : kMaxGrid), kSlabThreads, kSlabHSmem, st>>>(plan);
+            k_slab_h<T><<<(int)(plan.n_slab < kMaxGrid ? plan.n_slab : kMaxGrid), kSlabThreads, 0, st>>>(plan);
         break;
     case kPhaseFusedZ:
         if (plan.n_zp > 0) {
@@ -2000,7 +1822,7 @@ static cudaError_t phase_t(const Plan &plan, int phase, int grid_cap, cudaStream
         break;
     case kPhaseSlabE:
         if (plan.n_slab > 0)
-            k_slab_e<T><<<(int)(plan.n_slab < kMaxGrid ? plan.n_slab : kMaxGrid), kSlabThreads, kSlabESmem, st>>>(plan);
+            k_slab_e<T><<<(int)(plan.n_slab < kMaxGrid ? plan.n_slab : kMaxGrid), kSlabThreads, 0, st>>>(plan);
         break;
     default:
         k_post<T><<<plan.nb, 128, 0, st>>>(plan);
@@ -2076,9 +1898,7 @@ bool fused_tile_supported(int tx, int ty) { return (tx == 62 || tx == 124) && (t
 template <typename T>
 static cudaError_t limits_t()
 {
-    cudaError_t e[11] = {PairCfg<T>::set_limit(),
-                         cudaFuncSetAttribute(k_slab_h<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlabHSmem),
-                         cudaFuncSetAttribute(k_slab_e<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlabESmem),
+    cudaError_t e[9] = {PairCfg<T>::set_limit(),
                          FusedCfg<T, 4, 1, false, 1>::set_limit(), FusedCfg<T, 8, 1, false, 4>::set_limit(),
                          FusedCfg<T, 4, 2, false, 1>::set_limit(), FusedCfg<T, 8, 2, false, 2>::set_limit(),
                          FusedCfg<T, 4, 1, true, 1>::set_limit(),  FusedCfg<T, 8, 1, true, 4>::set_limit(),
