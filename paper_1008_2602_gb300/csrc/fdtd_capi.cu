@@ -103,6 +103,7 @@ struct fdtd_ctx {
     Plan plan{};                     // tiled launches
     long long *plan_buf = nullptr;   // device [0]=board ptr, then prefixes
     size_t plan_cap = 0;
+    SideStream side;
     cudaGraphExec_t graph = nullptr;
     int graph_chunk = 0;
     cudaGraphExec_t graph2 = nullptr;   // pairs of steps (depth 2)
@@ -138,6 +139,7 @@ struct fdtd_batch {
     Plan plan{};
     long long *plan_buf = nullptr;
     size_t plan_cap = 0;
+    SideStream side;
     cudaGraphExec_t graph = nullptr;
     int graph_chunk = 0;
     // members stepped by resident launches (the rest step by `plan`)
@@ -1078,12 +1080,29 @@ struct NvtxRange {
     ~NvtxRange() { nvtxRangePop(); }
 };
 
+// The side stream of a context or batch, made on its first tiled step.
+int open_side(SideStream &s)
+{
+    if (!s.stream) CK(cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking));
+    if (!s.start) CK(cudaEventCreateWithFlags(&s.start, cudaEventDisableTiming));
+    if (!s.done) CK(cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming));
+    return FDTD_OK;
+}
+void close_side(SideStream &s)
+{
+    if (s.start) cudaEventDestroy(s.start);
+    if (s.done) cudaEventDestroy(s.done);
+    if (s.stream) cudaStreamDestroy(s.stream);
+    s = SideStream{};
+}
+
 // Run n steps of `plan` on stream st: CUDA graphs of `chunk` steps (each
 // ending with the running-DFT update), direct launches for the remainder.
 int run_steps(const Plan &plan, int prec, int grid_cap, int n, int chunk, cudaGraphExec_t &graph, int &graph_chunk,
-              cudaStream_t st)
+              cudaStream_t st, SideStream &side)
 {
     if (n <= 0) return FDTD_OK;
+    if (int r = open_side(side)) return r;
     NvtxRange range(plan.nb > 1 ? "fdtd batch steps" : "fdtd steps");
     if (chunk > 1 && n >= chunk) {
         if (!graph || graph_chunk != chunk) {
@@ -1092,7 +1111,7 @@ int run_steps(const Plan &plan, int prec, int grid_cap, int n, int chunk, cudaGr
             cudaGraph_t gr = nullptr;
             CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
             cudaError_t e = cudaSuccess;
-            for (int s = 0; s < chunk && e == cudaSuccess; ++s) e = launch_step(plan, prec, grid_cap, st);
+            for (int s = 0; s < chunk && e == cudaSuccess; ++s) e = launch_step(plan, prec, grid_cap, st, side);
             if (e == cudaSuccess) e = launch_dft(plan, grid_cap, st);
             cudaError_t e2 = cudaStreamEndCapture(st, &gr);
             if (e != cudaSuccess) { if (gr) cudaGraphDestroy(gr); return cuda_fail(e, "capture"); }
@@ -1106,7 +1125,7 @@ int run_steps(const Plan &plan, int prec, int grid_cap, int n, int chunk, cudaGr
         n %= chunk;
     }
     if (n > 0) {
-        for (int s = 0; s < n; ++s) CK(launch_step(plan, prec, grid_cap, st));
+        for (int s = 0; s < n; ++s) CK(launch_step(plan, prec, grid_cap, st, side));
         CK(launch_dft(plan, grid_cap, st));
     }
     return FDTD_OK;
@@ -1133,12 +1152,13 @@ int resident_chunk(long long nodes) { return (int)std::min<long long>(255, std::
 // (the state in the middle of a pair is kept only where later launches read
 // it).
 int run_depth2(const Plan &plan, int prec, int grid_cap, long long step, int n, int chunk, cudaGraphExec_t &graph2,
-               int &graph2_chunk, cudaStream_t st)
+               int &graph2_chunk, cudaStream_t st, SideStream &side)
 {
     if (n <= 0) return FDTD_OK;
+    if (int r = open_side(side)) return r;
     NvtxRange range("fdtd step pairs");
     const PairSplit sp = pair_split(step, n);
-    if (sp.lead) CK(launch_step(plan, prec, grid_cap, st));
+    if (sp.lead) CK(launch_step(plan, prec, grid_cap, st, side));
     const bool direct = sp.lead != 0;
     int pairs = sp.pairs;
     const int left = sp.tail;
@@ -1164,7 +1184,7 @@ int run_depth2(const Plan &plan, int prec, int grid_cap, long long step, int n, 
         pairs %= cp;
     }
     for (int p = 0; p < pairs; ++p) CK(launch_pair(plan, prec, grid_cap, st));
-    for (int s = 0; s < left; ++s) CK(launch_step(plan, prec, grid_cap, st));
+    for (int s = 0; s < left; ++s) CK(launch_step(plan, prec, grid_cap, st, side));
     if (direct || pairs > 0 || left > 0) CK(launch_dft(plan, grid_cap, st));
     return FDTD_OK;
 }
@@ -1614,9 +1634,9 @@ int fdtd_step(fdtd_ctx *c, int n)
         if (int r = run_resident(&c->res, 1, c->rplan, c->grid_cap, n, resident_chunk(c->h.nodes), c->cur)) return r;
     } else if (c->h.pair_ok) {
         if (int r = run_depth2(c->plan, c->prec, c->grid_cap, c->host_step, n, c->tune.graph_chunk, c->graph2,
-                               c->graph2_chunk, c->cur))
+                               c->graph2_chunk, c->cur, c->side))
             return r;
-    } else if (int r = run_steps(c->plan, c->prec, c->grid_cap, n, c->tune.graph_chunk, c->graph, c->graph_chunk, c->cur)) {
+    } else if (int r = run_steps(c->plan, c->prec, c->grid_cap, n, c->tune.graph_chunk, c->graph, c->graph_chunk, c->cur, c->side)) {
         return r;
     }
     c->host_step += n;
@@ -2211,6 +2231,7 @@ void fdtd_destroy(fdtd_ctx *c)
     if (c->cur) cudaStreamSynchronize(c->cur);
     if (c->graph) cudaGraphExecDestroy(c->graph);
     if (c->graph2) cudaGraphExecDestroy(c->graph2);
+    close_side(c->side);
     if (c->plan_buf) cudaFree(c->plan_buf);
     if (c->rplan_buf) cudaFree(c->rplan_buf);
     if (c->res_buf) cudaFree(c->res_buf);
@@ -2339,7 +2360,7 @@ int fdtd_batch_step(fdtd_batch *b, int n, int *n_done)
             if (int r = run_resident(b->res.data(), (int)b->res.size(), b->rplan, b->grid_cap, run, b->res_chunk, b->stream))
                 return r;
         if (b->plan.nb > 0)
-            if (int r = run_steps(b->plan, b->prec, b->grid_cap, run, b->tune.graph_chunk, b->graph, b->graph_chunk, b->stream))
+            if (int r = run_steps(b->plan, b->prec, b->grid_cap, run, b->tune.graph_chunk, b->graph, b->graph_chunk, b->stream, b->side))
                 return r;
         for (size_t m = 0; m < b->members.size(); ++m) {
             const long long did = std::min<long long>(run, b->remaining[m]);
@@ -2383,6 +2404,7 @@ void fdtd_batch_destroy(fdtd_batch *b)
         launch_set_i64(c->h.stop, LLONG_MAX, c->cur);
     }
     if (b->graph) cudaGraphExecDestroy(b->graph);
+    close_side(b->side);
     if (b->plan_buf) cudaFree(b->plan_buf);
     if (b->rplan_buf) cudaFree(b->rplan_buf);
     if (b->res_buf) cudaFree(b->res_buf);

@@ -349,7 +349,12 @@ enum Phase : int { kPhaseSlabH = 0, kPhaseFusedZ = 1, kPhaseInterior = 2, kPhase
 
 // Launchers (fdtd_kernels.cu).  All enqueue on `st`.
 cudaError_t launch_phase(const Plan &plan, int prec, int phase, int grid_cap, cudaStream_t st);
-cudaError_t launch_step(const Plan &plan, int prec, int grid_cap, cudaStream_t st);
+// A stream that takes a launch beside the main one, and the events that fork and join it.
+struct SideStream {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t start = nullptr, done = nullptr;
+};
+cudaError_t launch_step(const Plan &plan, int prec, int grid_cap, cudaStream_t st, const SideStream &side);
 // A pair of steps with the two-step pass (depth-2 board, even step); or one of its nine launches.
 constexpr int kPairLaunches = 9;
 constexpr int kPairPhase[kPairLaunches] = {kPhaseSlabH, kPhaseFusedZ, kPhaseInterior, kPhaseSlabE, kPhasePost,

@@ -259,9 +259,9 @@ struct Tile {
 // it cost 2 %).  The interior kernel (ZP false) covers planes
 // [iz0, iz1); the z-UPML kernel
 // covers [zlo, iz0) and [max(iz1, iz0), nz).  kstart is the plane below the
-// segment when the tile recomputes its H~ there, else kb (that plane's H~ is
-// then read from the output: an outer plane, or a z-UPML plane written by the
-// z-UPML launch, which runs first).
+// segment when the tile recomputes its H~ there (always in the interior
+// launch), else kb (that plane's H~ is then read from the output: the wall
+// plane below a z-UPML segment that starts at plane 1).
 template <int TY, int W, bool ZP>
 __device__ __forceinline__ Tile decode_tile(const Plan &plan, long long item)
 {
@@ -300,7 +300,7 @@ __device__ __forceinline__ Tile decode_tile(const Plan &plan, long long item)
     if (!ZP) {
         t.kb = iz0 + tz * zs;
         t.ke = min(t.kb + zs, iz1);
-        t.kstart = t.kb - 1 >= iz0 ? t.kb - 1 : t.kb;
+        t.kstart = t.kb - 1;
     } else {
         // planes [zlo, iz0) and [max(iz1, iz0), nz); a segment starting at
         // plane 0 (zlo = 0) has no plane below, one starting at plane 1
@@ -319,6 +319,16 @@ __device__ __forceinline__ Tile decode_tile(const Plan &plan, long long item)
     return t;
 }
 
+// A value as the storage type holds it.
+template <typename T>
+__device__ __forceinline__ float rnd(float v);
+template <>
+__device__ __forceinline__ float rnd<float>(float v) { return v; }
+template <>
+__device__ __forceinline__ float rnd<__half>(float v) { return __half2float(__float2half_rn(v)); }
+template <typename T>
+__device__ __forceinline__ float2 rnd2(float2 v) { return make_float2(rnd<T>(v.x), rnd<T>(v.y)); }
+
 // Fused H+E kernel over the fused region, fed by TMA, warp-specialised.
 // Warps 0..W-1 compute; warp W (one lane) is the producer, streaming planes
 // kstart..ke of the tile into an NS-stage ring (E^n with a one-node halo,
@@ -333,8 +343,14 @@ __device__ __forceinline__ Tile decode_tile(const Plan &plan, long long item)
 // H~^{n+1/2}(k) at its two columns for the halo row j0-1 and then row by
 // row, so H(j-1) is already in registers; H(i-1) of its first column comes
 // from the lane to its left with a shuffle; then it updates E^{n+1}(k).  H~
-// of halo nodes outside the fused region is read from the slab kernel's
-// output instead.  The plane below the segment is run once for the tile's
+// of halo nodes outside the fused region is, in the z-UPML launch, read from
+// the slab kernel's output.  The interior launch forms it itself: of the
+// components it needs there (H~y, H~z on the x side, H~x, H~z on the y side,
+// H~x, H~y on the plane below) none has an auxiliary, so they are the lossy
+// Yee form of the same staged inputs, rounded as the slab or z-UPML launch
+// stores them.  So the interior launch depends on no other launch of its step
+// and runs beside them (launch_step); without the global reads in its inner
+// loop it also takes 95 instead of 110 us on the 480x380x100 FP16 board.  The plane below the segment is run once for the tile's
 // H~x, H~y there (or read, see decode_tile); the plane above is read for E
 // only.  In z-UPML planes (sigma_z only) H~z carries B~z and E_z carries
 // D~z, while H~x, H~y, E_x, E_y update in the lossy form; those planes use
@@ -475,7 +491,7 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
         float2 hk1x[TYW], hk1y[TYW];   // H~x, H~y of the previous plane, per row
 #pragma unroll
         for (int r = 0; r < TYW; ++r) { hk1x[r] = make_float2(0.f, 0.f); hk1y[r] = make_float2(0.f, 0.f); }
-        if (kstart == kb && kb > 0) {   // plane kb-1 is not recomputed: read its H~ (none below plane 0)
+        if (ZP && kstart == kb && kb > 0) {   // plane kb-1 is not recomputed: read its H~ (none below plane 0)
 #pragma unroll
             for (int r = 0; r < TYW; ++r)
                 if (jb + r < iy1) {
@@ -541,6 +557,32 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
                     hx = sub2(ohx, scx);
                     hy = sub2(ohy, scy);
                     hz = sub2(ohz, scz);
+                    if (!ZP) {
+                        auto lossy = [](const Coef &c, float h, float sc) {
+                            return rnd<T>(__fmaf_rn(-c.g, sc, __fmul_rn(c.b1, h)));
+                        };
+                        if (k < iz0) {   // the plane below the interior
+                            const Coef c = ldcoef(B->cw[2][1] + k);
+                            hx = make_float2(lossy(c, ohx.x, scx.x), lossy(c, ohx.y, scx.y));
+                            hy = make_float2(lossy(c, ohy.x, scy.x), lossy(c, ohy.y, scy.y));
+                        } else {
+                            if (rr == 0 && row_slab) {   // the row below the fused region
+                                const Coef c = ldcoef(B->cw[1][1] + (jb - 1));
+                                hx = make_float2(lossy(c, ohx.x, scx.x), lossy(c, ohx.y, scx.y));
+                                hz = make_float2(lossy(c, ohz.x, scz.x), lossy(c, ohz.y, scz.y));
+                            }
+                            if (slab_a) {                // the columns before it
+                                const Coef c = ldcoef(B->cw[0][1] + ca);
+                                hy.x = lossy(c, ohy.x, scy.x);
+                                hz.x = lossy(c, ohz.x, scz.x);
+                            }
+                            if (slab_b) {
+                                const Coef c = ldcoef(B->cw[0][1] + cb);
+                                hy.y = lossy(c, ohy.y, scy.y);
+                                hz.y = lossy(c, ohz.y, scz.y);
+                            }
+                        }
+                    }
                 } else {
                     // B~z of the node: box row rr; zero outside the fused rows
                     float2 boz = make_float2(A0[rr * AW], A0[rr * AW + 1]);
@@ -553,8 +595,9 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
                     hz.y = fused_hz(ohz.y, scz.y, zb, z, boz.y, nbz.y);
                 }
             };
-            // halo elements outside the fused region come from the slab output
+            // z-UPML launch: halo elements outside the fused region come from the slab output
             auto slab_fix = [&](int rr, float2 &hx, float2 &hy, float2 &hz) {
+                if (!ZP) return;
                 if (jb - 1 + rr >= iy1) return;
                 const T *gq = gp + (long long)rr * X;
                 if (slab_a) { hx.x = Io<T>::ld(gq + 3 * NN); hy.x = Io<T>::ld(gq + 4 * NN); hz.x = Io<T>::ld(gq + 5 * NN); }
@@ -565,7 +608,7 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
 
             float2 px = make_float2(0.f, 0.f), pz = px;   // H~x, H~z at (., j-1)
             if (full_plane) {
-                if (row_slab) {   // row jb-1 lies in the low-y slab: read its H~ (own columns)
+                if (ZP && row_slab) {   // row jb-1 lies in the low-y slab: read its H~ (own columns)
                     if (own_a && own_b) {
                         px = Pair<T>::ldg(gp + 3 * NN);
                         pz = Pair<T>::ldg(gp + 5 * NN);
@@ -709,15 +752,6 @@ struct PairLayout {
     static constexpr int THREADS = 32 * (kPairW1 + kPairW2 + 1);
     static_assert(2 * (BYTES + 1024) <= 232448, "two blocks per SM");
 };
-
-template <typename T>
-__device__ __forceinline__ float rnd(float v);
-template <>
-__device__ __forceinline__ float rnd<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ float rnd<__half>(float v) { return __half2float(__float2half_rn(v)); }
-template <typename T>
-__device__ __forceinline__ float2 rnd2(float2 v) { return make_float2(rnd<T>(v.x), rnd<T>(v.y)); }
 
 struct PairTile {
     const Board *B;
@@ -1884,13 +1918,26 @@ cudaError_t launch_pair(const Plan &plan, int prec, int grid_cap, cudaStream_t s
     return cudaSuccess;
 }
 
-cudaError_t launch_step(const Plan &plan, int prec, int grid_cap, cudaStream_t st)
+// One step.  The interior launch depends on no other launch of the step, so it
+// runs on the side stream beside slab H and the z-UPML launch: the blocks of
+// one fill the SMs that the others' last waves leave (880x680x100 669 us a step
+// one after the other, 643 so; 480x380x100 FP16 239 and 220, 280x230x100 FP16
+// 136 and 119).
+cudaError_t launch_step(const Plan &plan, int prec, int grid_cap, cudaStream_t st, const SideStream &side)
 {
-    for (int ph = 0; ph < kNumPhases; ++ph) {
-        cudaError_t e = launch_phase(plan, prec, ph, grid_cap, st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    auto run = [&](int ph, cudaStream_t on) { if (e == cudaSuccess) e = launch_phase(plan, prec, ph, grid_cap, on); };
+    auto ok = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+    ok(cudaEventRecord(side.start, st));
+    ok(cudaStreamWaitEvent(side.stream, side.start, 0));
+    run(kPhaseSlabH, st);
+    run(kPhaseInterior, side.stream);
+    run(kPhaseFusedZ, st);
+    ok(cudaEventRecord(side.done, side.stream));
+    ok(cudaStreamWaitEvent(st, side.done, 0));
+    run(kPhaseSlabE, st);
+    run(kPhasePost, st);
+    return e;
 }
 
 bool fused_tile_supported(int tx, int ty) { return (tx == 62 || tx == 124) && (ty == 4 || ty == 8); }
