@@ -387,7 +387,8 @@ void fdtd_batch_destroy(fdtd_batch *b);
  * columns: 62 or 124, i.e. one or two strips of 62 columns; tile_y rows: 4
  * or 8; a 62x8 tile is worked by four compute warps of 2 rows, a 124x8 tile
  * by two warps of 4 rows per strip; default 62x8), the z-segment length
- * (planes one tile marches before the next work item; default 10) and the
+ * (planes one tile marches before the next work item; default 10, 6 or 4 by
+ * the number of work items) and the
  * number of steps per CUDA graph (default 16).  depth is the number of
  * leapfrog steps one sweep over the interior region advances (time blocking,
  * Model section: the leapfrog's H and E updates of two steps in one pass):

@@ -97,7 +97,7 @@ struct fdtd_ctx {
     long long host_step = 0;
     fdtd_batch *batch = nullptr;
     // single-board plan and graph
-    fdtd_tuning tune{62, 8, 10, 16, 1, 38};
+    fdtd_tuning tune{62, 8, 0, 16, 1, 38};   // zseg 0: by the plan (auto_zseg)
     bool plan_dirty = true;          // neither plan below holds any more
     bool plan_ok = false, rplan_ok = false;
     Plan plan{};                     // tiled launches
@@ -134,7 +134,7 @@ struct fdtd_batch {
     bool own_stream = false;
     std::vector<fdtd_ctx *> members;
     std::vector<long long> remaining;
-    fdtd_tuning tune{62, 8, 10, 16, 1, 38};
+    fdtd_tuning tune{62, 8, 0, 16, 1, 38};   // zseg 0: by the plan (auto_zseg)
     bool dirty = true;
     Plan plan{};
     long long *plan_buf = nullptr;
@@ -822,6 +822,26 @@ long long fused_items(const Board &h, const fdtd_tuning &t, bool zp)
     return ((Lx + t.tile_x - 1) / t.tile_x) * ((Ly + t.tile_y - 1) / t.tile_y) * nseg;
 }
 
+// z-segment length of the fused launches where the caller set none: 10 planes (a
+// segment restages two), shorter where the boards then give the interior launch
+// too few items for its resident blocks (four on each of 152 SMs) to end
+// together.  Measured, us a step at 4 / 6 / 8 / 10 planes, FP16: 232x192x39 (88
+// tiles of 19 planes) 50.2 / 52.5 / 54.1 / 56.4, 280x230x100 (130 of 76) 112 /
+// 109 / 111 / 119, 480x380x100 (360 of 76) 234 / 227 / 218 / 220, 880x680x100
+// (1148 of 76) 576 / 546 / 532 / 524.
+int auto_zseg(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &t)
+{
+    const long long slots = 4 * 152;
+    for (int zs : {10, 6, 4}) {
+        fdtd_tuning u = t;
+        u.zseg = zs;
+        long long items = 0;
+        for (const fdtd_ctx *c : boards) items += fused_items(c->h, u, false);
+        if (items >= (zs == 10 ? 3 : 2) * slots) return zs;
+    }
+    return 4;
+}
+
 // Two-step items of a board: 60 x 8 tiles x z segments of pair_zseg planes of I.
 long long pair_items(const Board &h, const fdtd_tuning &t)
 {
@@ -837,10 +857,12 @@ long long dft_items(const Board &h)
 }
 
 // Lay out plan arrays [boards | int_prefix | zp_prefix | slab_prefix | dft_prefix | work | slab blocks] in buf.
-int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &t, bool tiled, long long *&buf, size_t &cap,
+int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, bool tiled, long long *&buf, size_t &cap,
                Plan &plan, cudaStream_t st, std::vector<long long> &host)
 {
     const int nb = (int)boards.size();
+    fdtd_tuning t = tune;
+    if (t.zseg <= 0) t.zseg = auto_zseg(boards, t);
     for (int b = 0; b < nb && tiled; ++b)
         if (!fused_maps_match(boards[b]->h, t.tile_x, t.tile_y))
             return fail(FDTD_EINVAL, "fused tile " + std::to_string(t.tile_x) + "x" + std::to_string(t.tile_y) +
