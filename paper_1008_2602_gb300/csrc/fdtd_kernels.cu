@@ -1518,6 +1518,7 @@ __global__ void k_post(Plan plan)
 {
     const int b = blockIdx.x;
     if (b >= plan.nb) return;
+    if (b == 0 && threadIdx.x < 3) plan.work[threadIdx.x] = 0;   // for the next step's launches
     Board *B = plan.boards[b];
     // What does not depend on the step is loaded before the step counter, so
     // the descriptors, the field pointers and the counters arrive together
@@ -1554,9 +1555,9 @@ __global__ void k_post(Plan plan)
         for (int s = par_src ? tid : 0; s < n_src; s += par_src ? (int)blockDim.x : 1) {
             const Source S = (par_src && s == tid) ? s0 : src[s];
             if (skip_i && in_interior(B, S.i, S.j, S.k)) continue;
-            const double w = src_pulse(S, step, dt);
             T *e = field(out, S.comp) + S.node;
-            Io<T>::st(e, src_apply(S, w, Io<T>::ldw(e), Io<T>::ldw((const T *)field(in, S.comp) + S.node)));
+            const float ep = Io<T>::ldw(e), en = Io<T>::ldw((const T *)field(in, S.comp) + S.node);   // before the pulse's FP64 chain
+            Io<T>::st(e, src_apply(S, src_pulse(S, step, dt), ep, en));
         }
     }
     __syncthreads();
@@ -1843,16 +1844,10 @@ static cudaError_t phase_t(const Plan &plan, int phase, int grid_cap, cudaStream
             k_slab_h<T><<<(int)(plan.n_slab < kMaxGrid ? plan.n_slab : kMaxGrid), kSlabThreads, 0, st>>>(plan);
         break;
     case kPhaseFusedZ:
-        if (plan.n_zp > 0) {
-            cudaMemsetAsync(plan.work + 1, 0, sizeof(int), st);
-            launch_fused<T, true>(plan, st);
-        }
+        if (plan.n_zp > 0) launch_fused<T, true>(plan, st);
         break;
     case kPhaseInterior:
-        if (plan.n_int > 0) {
-            cudaMemsetAsync(plan.work, 0, sizeof(int), st);
-            launch_fused<T, false>(plan, st);
-        }
+        if (plan.n_int > 0) launch_fused<T, false>(plan, st);
         break;
     case kPhaseSlabE:
         if (plan.n_slab > 0)
@@ -1883,10 +1878,7 @@ static cudaError_t pair_t(const Plan &plan, int idx, int grid_cap, cudaStream_t 
     Plan p = plan;
     switch (idx) {
     case 2:
-        if (plan.n_pair > 0) {
-            cudaMemsetAsync(plan.work + 2, 0, sizeof(int), st);
-            PairCfg<T>::launch(plan, st);
-        }
+        if (plan.n_pair > 0) PairCfg<T>::launch(plan, st);
         return cudaGetLastError();
     case 4: p.first_of_pair = 1; return phase_t<T>(p, kPhasePost, grid_cap, st);
     case 5:   // the band's H+E blocks sit just before the slab blocks in the table
