@@ -237,7 +237,7 @@ struct Plan {
     const SlabBlock *slab_blk;    // [n_slab] per-block descriptors
     const long long *dft_prefix;  // [nb + 1] DFT warps
     long long n_int, n_zp, n_slab, n_dft;
-    int *work;                    // fused-kernel work counters [interior, z-UPML, two-step] (zeroed before every launch)
+    int *work;                    // fused-kernel work counters [interior, z-UPML, two-step]; k_post leaves them at zero
     int slots;                    // resident blocks of the fused launch (set by its launcher; orders the items)
     // two-step passes (single-board plans of a depth-2 board)
     long long n_pair;             // two-step items (60 x 8 tiles x z segments of pair_zseg planes)

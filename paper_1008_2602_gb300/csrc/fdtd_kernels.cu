@@ -1375,6 +1375,26 @@ __device__ __forceinline__ C4 quad_factors(const Coef *p, int i, int n, bool gra
               F4{make_float2(a.ap, b.ap), make_float2(c.ap, d.ap)}, F4{make_float2(a.am, b.am), make_float2(c.am, d.am)}};
 }
 
+// Boards whose field sets do not stay in L2 from one launch to the next fetch
+// the next plane's lines into it while a plane is worked: no registers, and a
+// plane waits for L2 instead of HBM (us a step without and with it: FP16
+// 280x230x100 110.9 and 101.7, 480x380x100 221.4 and 210.2, 880x680x100 525 and
+// 507; FP32 at 880x680x100 641.5 and 637.0).  A board in L2 only gets more
+// instructions (232x192x39 FP16, field sets of 44 MB: 47.7 and 49.1).  Fetching
+// all of a thread's planes at its start, or runs of 8 planes, took 1 to 6 us
+// more per launch.
+constexpr long long kPrefetchBytes = 100000000;
+template <typename T>
+__device__ __forceinline__ bool slab_prefetch(long long nodes)
+{
+    return 12 * (long long)sizeof(T) * nodes > kPrefetchBytes;
+}
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void prefetch_aux(const float *p, int at)
+{
+    if (p) prefetch_l2(p + at);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kSlabThreads, kSlabBlocks) k_slab_h(Plan plan)
 {
@@ -1384,6 +1404,7 @@ __global__ void __launch_bounds__(kSlabThreads, kSlabBlocks) k_slab_h(Plan plan)
         const Board *const B = t.B;
         const int X = B->pitch, nx = B->nx, ny = B->ny, nz = B->nz;
         const long long P = B->plane, N = B->nodes;
+        const bool cold = slab_prefetch<T>(N);
         const float Sx = B->S[0], Sy = B->S[1], Sz = B->S[2];
         float *const a0 = t.sl->aux[3], *const a1 = t.sl->aux[4], *const a2 = t.sl->aux[5];
         const long long at = (long long)t.k * P + (long long)t.j * X + t.i;
@@ -1399,6 +1420,15 @@ __global__ void __launch_bounds__(kSlabThreads, kSlabBlocks) k_slab_h(Plan plan)
             const float eyi = Io<T>::ldw(e + N + 4), ezi = Io<T>::ldw(e + 2 * N + 4);
             const F4 hx = ld4(e + 3 * N), hy = ld4(e + 4 * N), hz = ld4(e + 5 * N);
             const F4 b0 = slab_aux(a0, ax, t.own, t.whole), b1 = slab_aux(a1, ax, t.own, t.whole), b2 = slab_aux(a2, ax, t.own, t.whole);
+            if (cold && m + 1 < t.count) {
+                const int o1 = ax + t.astep + __ffs(t.own) - 1;   // the quad's first own node: the array may start there
+                prefetch_l2(e + 2 * P);
+                prefetch_l2(e + N + 2 * P);
+                for (int c = 2; c < 6; ++c) prefetch_l2(e + c * N + P);
+                prefetch_aux(a0, o1);
+                prefetch_aux(a1, o1);
+                prefetch_aux(a2, o1);
+            }
             const int k = t.k + m;
             const C4 y0 = row_factors(fy0), y1 = row_factors(fy1), z0 = row_factors(fz0 + m), z1 = row_factors(fz1 + m);
             unsigned mx = t.own, my = t.own, mz = t.own;
@@ -1435,6 +1465,7 @@ __global__ void __launch_bounds__(kSlabThreads, kSlabBlocks) k_slab_e(Plan plan)
         const Board *const B = t.B;
         const int X = B->pitch, nx = B->nx, ny = B->ny, nz = B->nz;
         const long long P = B->plane, N = B->nodes;
+        const bool cold = slab_prefetch<T>(N);
         const float Sx = B->S[0], Sy = B->S[1], Sz = B->S[2];
         float *const a0 = t.sl->aux[0], *const a1 = t.sl->aux[1], *const a2 = t.sl->aux[2];
         const long long at = (long long)t.k * P + (long long)t.j * X + t.i;
@@ -1456,6 +1487,17 @@ __global__ void __launch_bounds__(kSlabThreads, kSlabBlocks) k_slab_e(Plan plan)
             F4 hxj = ld4(o + 3 * N - X), hzj = ld4(o + 5 * N - X);
             const F4 ex = ld4(e), ey = ld4(e + N), ez = ld4(e + 2 * N);
             const F4 d0 = slab_aux(a0, ax, t.own, t.whole), d1 = slab_aux(a1, ax, t.own, t.whole), d2 = slab_aux(a2, ax, t.own, t.whole);
+            if (cold && m + 1 < t.count) {
+                const int o1 = ax + t.astep + __ffs(t.own) - 1;
+                prefetch_l2(cid + (id16 ? 2 * P : P));
+                for (int c = 0; c < 3; ++c) {
+                    prefetch_l2(e + c * N + P);
+                    prefetch_l2(o + (c + 3) * N + P);
+                }
+                prefetch_aux(a0, o1);
+                prefetch_aux(a1, o1);
+                prefetch_aux(a2, o1);
+            }
             const int k = t.k + m;
             const C4 y0 = row_factors(fy0), y1 = row_factors(fy1), z0 = row_factors(fz0 + m), z1 = row_factors(fz1 + m);
             F4 hyl{make_float2(hyi, hy.a.x), make_float2(hy.a.y, hy.b.x)};   // H~y, H~z at i - 1
@@ -1518,7 +1560,10 @@ __global__ void k_post(Plan plan)
 {
     const int b = blockIdx.x;
     if (b >= plan.nb) return;
-    if (b == 0 && threadIdx.x < 3) plan.work[threadIdx.x] = 0;   // for the next step's launches
+    // The work counters of the next step's fused launches (a memset node before
+    // each launch lengthened a step's chain: 50.2 us on the 232x192x39 FP16
+    // board, 47.7 without them).
+    if (b == 0 && threadIdx.x < 3) plan.work[threadIdx.x] = 0;
     Board *B = plan.boards[b];
     // What does not depend on the step is loaded before the step counter, so
     // the descriptors, the field pointers and the counters arrive together
