@@ -51,10 +51,13 @@ inline int res_box_of(const Board &h, int i, int j, int k)
     return -1;
 }
 
-// Relative cost of a unit of a box (measured per block on the 232x192x39
-// board): an interior unit 10; a graded box more with every auxiliary, and
-// more again where its rows are short, so that a warp touches many row
-// segments.
+// Relative cost of a unit of a box: an interior unit 10; a graded box more with
+// every auxiliary, and more again where its rows are short, so that a warp
+// touches many row segments.  The constants are those of the best step time
+// over boards of 0.25 to 14 M cells and 24 boards at once, in us: 97x61x43
+// 7.9, 232x192x39 21.7, 280x230x100 92.0, 420x335x100 215, 24 boards 608.  With
+// 13 + ... + 9: 8.4, 22.1, 95.4, 219, 620; 10 + ... + 12: 8.3, 21.8, 89.5, -,
+// 608; graded boxes a tenth lighter or short rows + 7: 24 boards 639 and more.
 inline int res_weight(const Board &h, int box)
 {
     if (box == h.n_slab + 2) return 10;
@@ -64,7 +67,7 @@ inline int res_weight(const Board &h, int box)
         for (int a = 0; a < 6; ++a) naux += h.slab[box].aux[a] != nullptr;
         width = h.slab[box].ni;
     }
-    return 13 + (8 * naux + 4) / 5 + (width < 64 ? 9 : 0);
+    return 11 + (8 * naux + 4) / 5 + (width < 64 ? 11 : 0);
 }
 
 // Work of a step of a board, in those weights.
