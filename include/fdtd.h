@@ -164,7 +164,7 @@ int fdtd_set_spectrum(fdtd_ctx *ctx, double f_max, int n_total_steps);
 /* Advance n >= 0 leapfrog steps (H^{n+1/2} from E^n, then E^{n+1} from
  * H^{n+1/2} and J^{n+1/2}, then probes and DFT).  Asynchronous on the
  * context's stream; fields stay on the device between calls.  FP32 boards up
- * to 24 Mi grid points at depth 1 run many steps per cooperative launch, the
+ * to 14 Mi grid points at depth 1 run many steps per cooperative launch, the
  * others five launches per step replayed as CUDA graphs; a board's fields and
  * traces are the same bit for bit either way. */
 int fdtd_step(fdtd_ctx *ctx, int n);

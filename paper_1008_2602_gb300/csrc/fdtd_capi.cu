@@ -965,7 +965,10 @@ long long grid_points(const Board &h) { return (long long)(h.nx + 1) * (h.ny + 1
 // Boards up to this many grid points are stepped by resident launches.  Past
 // L2 (about 4 M points) their two passes move 73 B per node and step against
 // the tiled launches' 49, but without those launches' tails and slab launches.
-constexpr long long kResPoints = 24LL << 20;
+// Resident and tiled us a step: 280x230x100 92 and 109, 360x290x100 151 and
+// 171, 400x320x100 178 and 182, 480x380x100 258 and 242, 540x420x100 332 and
+// 276.
+constexpr long long kResPoints = 14LL << 20;
 
 std::vector<ResAt> res_ports(const fdtd_ctx *c)
 {
