@@ -349,10 +349,16 @@ __device__ __forceinline__ float2 rnd2(float2 v) { return make_float2(rnd<T>(v.x
 // H~x, H~y on the plane below) none has an auxiliary, so they are the lossy
 // Yee form of the same staged inputs, rounded as the slab or z-UPML launch
 // stores them.  So the interior launch depends on no other launch of its step
-// and runs beside them (launch_step); without the global reads in its inner
-// loop it also takes 95 instead of 110 us on the 480x380x100 FP16 board.  The plane below the segment is run once for the tile's
-// H~x, H~y there (or read, see decode_tile); the plane above is read for E
-// only.  In z-UPML planes (sigma_z only) H~z carries B~z and E_z carries
+// and runs beside them (launch_step).  The plane below the segment is run once
+// for the tile's H~x, H~y there (or read, see decode_tile); the plane above is
+// read for E only.  What holds for a whole item is tested once per item, not
+// once per row: whether the warp has halo nodes outside the fused region
+// (rim), or lanes that own one of their columns (split), the z-UPML box's
+// pointers.  FP16 is bound by issue slots and FP32 partly: the interior launch
+// took 95 us on the 480x380x100 FP16 board with those tests per row, 86.5 now;
+// 364 and 350 on the 880x680x100 FP32 board (a step 638 and 622).  More blocks
+// an SM at 72 or 96 registers spill: 101 us FP16 interior, 96 us FP16 z-UPML
+// launch (66.5 at 128).  In z-UPML planes (sigma_z only) H~z carries B~z and E_z carries
 // D~z, while H~x, H~y, E_x, E_y update in the lossy form; those planes use
 // the scalar update helpers per element, every other plane the paired form.
 template <typename T, int TY, int W, int NS, bool ZP, int R>
@@ -475,11 +481,13 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
         const int g = (wlo - 1) & ~1;
         const int ca = g + 2 * lx, cb = ca + 1;            // this lane's columns
         const bool own_a = ca >= wlo && ca < whi, own_b = cb >= wlo && cb < whi;
+        const bool own_2 = own_a && own_b, split = __any_sync(0xffffffffu, own_a != own_b);
         const bool slab_a = ca < ix0, slab_b = cb < ix0;  // halo column outside the fused region
         const int ecol = (g - ((i0 - 1) & ~7)) + 2 * lx;   // column of ca in the E/H boxes (even)
         const int xc0 = id16 ? (i0 & ~7) : (i0 & ~15);
-        const int ida = max(ca - xc0, 0), idb = cb - xc0;  // columns in the id box (clamped into it)
+        const int ida = max(ca - xc0, 0);                  // column of ca in the id box (clamped into it, even)
         const bool row_slab = (jb - 1 < iy0);
+        const bool rim_x = __any_sync(0xffffffffu, slab_a || slab_b), rim = rim_x || row_slab;   // slab nodes in the warp's halo
         // element (ca, jb-1, kstart) of component 0 in the output set, advanced by P per plane
         T *gp = (T *)B->f[oset][0] + ((long long)kstart * P + (long long)(jb - 1) * X + ca);
         const int zrow = B->zpitch;
@@ -487,6 +495,10 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
         const long long zcol = (long long)(jb - iy0) * zrow + (ca - ix0);   // aux index of (ca, jb) in a plane
         const int acol = (ca - ix0) - ((((i0 - 1) & ~1) - ix0) & ~3);       // column of ca in the aux boxes
         int s0 = sq, s1 = sq + 1 == NS ? 0 : sq + 1;
+        // z-UPML launch: the item's box, and the factors along z
+        const int zbox = ZP && kb >= iz1 ? 1 : 0, kz = ZP ? (zbox ? iz1 : B->zlo) : 0;
+        float *const zdz = ZP ? B->zD[zbox] : nullptr, *const nzbz = ZP ? B->zB[zbox][par ^ 1] : nullptr;
+        const Coef *const cz0 = ZP ? B->cw[2][0] : nullptr, *const cz1 = ZP ? B->cw[2][1] : nullptr;
 
         float2 hk1x[TYW], hk1y[TYW];   // H~x, H~y of the previous plane, per row
 #pragma unroll
@@ -515,14 +527,11 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
             constexpr int AW = St::AW, BCS = St::B_CS;
             const int zb = ZP ? (k < iz0 ? 1 : (k >= iz1 ? 2 : 0)) : 0;
             ZCoef z;
-            float *zdz = nullptr, *nzbz = nullptr;
             long long za = 0;
             if (ZP && zb) {
-                z.zi = B->cw[2][0][k];
-                z.zh = B->cw[2][1][k];
-                za = (long long)(k - (zb == 1 ? B->zlo : iz1)) * zplane + zcol;
-                nzbz = B->zB[zb - 1][par ^ 1];
-                zdz = B->zD[zb - 1];
+                z.zi = ldcoef(cz0 + k);
+                z.zh = ldcoef(cz1 + k);
+                za = (long long)(k - kz) * zplane + zcol;
             }
             const bool full_plane = k >= kb;
             // coefficient rows of the lane's two nodes (ids clamped into the box,
@@ -530,10 +539,16 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
             float4 cea[TYW], ceb[TYW];
 #pragma unroll
             for (int r = 0; r < TYW; ++r) {
-                const int ia = id16 ? (int)reinterpret_cast<const uint16_t *>(C0)[r * St::C16W + ida]
-                                    : (int)C0[r * St::C8W + ida];
-                const int ib = id16 ? (int)reinterpret_cast<const uint16_t *>(C0)[r * St::C16W + idb]
-                                    : (int)C0[r * St::C8W + idb];
+                int ia, ib;   // both nodes' ids in one aligned read: the lane's columns start at an even one
+                if (id16) {
+                    const unsigned v = *reinterpret_cast<const unsigned *>(C0 + 2 * (r * St::C16W + ida));
+                    ia = (int)(v & 0xffffu);
+                    ib = (int)(v >> 16);
+                } else {
+                    const unsigned v = *reinterpret_cast<const uint16_t *>(C0 + r * St::C8W + ida);
+                    ia = (int)(v & 0xffu);
+                    ib = (int)(v >> 8);
+                }
                 cea[r] = __ldg(ctab + ia);
                 ceb[r] = __ldg(ctab + ib);
             }
@@ -557,7 +572,7 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
                     hx = sub2(ohx, scx);
                     hy = sub2(ohy, scy);
                     hz = sub2(ohz, scz);
-                    if (!ZP) {
+                    if (!ZP && (rim || k < iz0)) {
                         auto lossy = [](const Coef &c, float h, float sc) {
                             return rnd<T>(__fmaf_rn(-c.g, sc, __fmul_rn(c.b1, h)));
                         };
@@ -597,7 +612,7 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
             };
             // z-UPML launch: halo elements outside the fused region come from the slab output
             auto slab_fix = [&](int rr, float2 &hx, float2 &hy, float2 &hz) {
-                if (!ZP) return;
+                if (!ZP || !rim_x) return;
                 if (jb - 1 + rr >= iy1) return;
                 const T *gq = gp + (long long)rr * X;
                 if (slab_a) { hx.x = Io<T>::ld(gq + 3 * NN); hy.x = Io<T>::ld(gq + 4 * NN); hz.x = Io<T>::ld(gq + 5 * NN); }
@@ -658,13 +673,15 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
                         if (own_a) { stg1(zdz + a, ndz.x); stg1(nzbz + a, nbz.x); }
                         if (own_b) { stg1(zdz + a + 1, ndz.y); stg1(nzbz + a + 1, nbz.y); }
                     }
-                    if (own_a && own_b) {
+                    if (own_2) {
                         stg2(o + 3 * NN, hx); stg2(o + 4 * NN, hy); stg2(o + 5 * NN, hz);
                         stg2(o, exv); stg2(o + NN, eyv); stg2(o + 2 * NN, ezv);
-                    } else if (own_a) {
+                    }
+                    if (split && own_a && !own_b) {
                         stg1(o + 3 * NN, hx.x); stg1(o + 4 * NN, hy.x); stg1(o + 5 * NN, hz.x);
                         stg1(o, exv.x); stg1(o + NN, eyv.x); stg1(o + 2 * NN, ezv.x);
-                    } else if (own_b) {
+                    }
+                    if (split && own_b && !own_a) {
                         stg1(o + 3 * NN + 1, hx.y); stg1(o + 4 * NN + 1, hy.y); stg1(o + 5 * NN + 1, hz.y);
                         stg1(o + 1, exv.y); stg1(o + NN + 1, eyv.y); stg1(o + 2 * NN + 1, ezv.y);
                     }
