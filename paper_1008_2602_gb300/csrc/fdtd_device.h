@@ -27,12 +27,6 @@ struct Io<__half> {
 };
 
 // ------------------------------------------------------------------ arithmetic
-// Sa (a1 - a0) - Sb (b1 - b0): one component of S * curl.
-__device__ __forceinline__ float curl2(float a1, float a0, float b1, float b0, float Sa, float Sb)
-{
-    return __fmaf_rn(-Sb, __fsub_rn(b1, b0), __fmul_rn(Sa, __fsub_rn(a1, a0)));
-}
-
 // Eq. 8 pulse of a source at the half step n + 1/2: J for a current source,
 // Vs for a voltage source.
 __device__ __forceinline__ double src_pulse(const Source &S, long long step, double dt)
@@ -51,33 +45,6 @@ __device__ __forceinline__ float src_apply(const Source &S, double w, float ep, 
 {
     if (S.kind == kSrcCurrent) return __fsub_rn(ep, (float)(S.coef * w));
     return (float)(((double)ep - S.beta * (double)en - S.gam * w) / (1.0 + S.beta));
-}
-
-// Gedney two-step update of one H~ component (B~ recurrence along w+1, H~
-// recurrence along w+2, B~->H~ along w).  scurl = S * (curl E)_w.  Bo/Bn are
-// the old/new auxiliaries (no auxiliary: pass aux == false).
-__device__ __forceinline__ float upml_h2(float h, float scurl, const Coef &a, const Coef &bb, const Coef &c, bool aux,
-                                         float Bo, float &Bn)
-{
-    if (aux) {
-        Bn = __fmaf_rn(-a.g, scurl, __fmul_rn(a.b1, Bo));
-        return __fmaf_rn(bb.g, __fmaf_rn(c.ap, Bn, -__fmul_rn(c.am, Bo)), __fmul_rn(bb.b1, h));
-    }
-    // no auxiliary: c is trivial and at most one of a, bb is graded, so the
-    // products below are exact
-    return __fmaf_rn(-__fmul_rn(a.g, bb.g), scurl, __fmul_rn(__fmul_rn(a.b1, bb.b1), h));
-}
-
-// Same for E (D~ along w+1, E along w+2, D~->E along w); ce = 1/eps_r.
-__device__ __forceinline__ float upml_e2(float e, float scurl, float ce, const Coef &a, const Coef &bb, const Coef &c,
-                                         bool aux, float Do, float &Dn)
-{
-    if (aux) {
-        Dn = __fmaf_rn(a.g, scurl, __fmul_rn(a.b1, Do));
-        return __fmaf_rn(__fmul_rn(ce, bb.g), __fmaf_rn(c.ap, Dn, -__fmul_rn(c.am, Do)), __fmul_rn(bb.b1, e));
-    }
-    // no auxiliary (see upml_h2)
-    return __fmaf_rn(__fmul_rn(ce, __fmul_rn(a.g, bb.g)), scurl, __fmul_rn(__fmul_rn(a.b1, bb.b1), e));
 }
 
 // Two adjacent elements of one row (8-byte aligned for FP32, 4-byte for the
@@ -103,9 +70,9 @@ struct Pair<__half> {
     static __device__ __forceinline__ void st(__half *p, float2 v) { *reinterpret_cast<__half2 *>(p) = __float22half2_rn(v); }
 };
 
-// Paired forms of curl2 and of h - s.  Per element they round exactly like
-// the scalar forms: a - b == fma(b, -1, a) (the product is exact), and
-// fma(-Sb, d, x) is the same single rounding either way.
+// h - s and one component of S * curl, Sa (a1 - a0) - Sb (b1 - b0), on a pair.
+// a - b == fma(b, -1, a) (the product is exact), so each element rounds as
+// the difference, one product and one fused multiply-add would.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ float2 curl2v(float2 a1, float2 a0, float2 b1, float2 b0, float2 Sa, float2 nSb)
 {
@@ -189,7 +156,11 @@ struct C4 {
 };
 __device__ __forceinline__ C4 fac_one() { return C4{four(1.f), four(1.f), four(1.f), four(1.f)}; }
 
-// upml_h2 and upml_e2 on a quad: the same operations, element by element.
+// Gedney two-step update of one H~ component of a quad (B~ recurrence along
+// w+1, H~ recurrence along w+2, B~->H~ along w).  sc = S * (curl E)_w; Bo/Bn
+// are the old/new auxiliaries.  No auxiliary (aux == false): c is trivial and
+// at most one of a, b is graded, so their products are exact.  Same for E
+// (D~ along w+1, E along w+2, D~->E along w); ce = 1/eps_r.
 __device__ __forceinline__ F4 upml_h4(const F4 &h, const F4 &sc, const C4 &a, const C4 &b, const C4 &c, bool aux, const F4 &Bo,
                                       F4 &Bn)
 {

@@ -19,9 +19,9 @@
 // steps replaces the two interior launches by one two-step pass (k_pair) and
 // lets the slab kernels finish the interior region's outer layer.
 //
-// All curl and update arithmetic goes through curl2()/the update helpers (or
-// their paired FFMA2 forms) with explicit round-to-nearest intrinsics, so a
-// value recomputed as a halo is bit-identical to the one its owner stores.
+// All curl and update arithmetic is written with explicit round-to-nearest
+// intrinsics (paired FFMA2 forms), so a value recomputed as a halo is
+// bit-identical to the one its owner stores.
 #include "fdtd_device.h"
 
 namespace fdtd {
@@ -55,57 +55,16 @@ __device__ __forceinline__ bool in_interior(const Board *B, int i, int j, int k)
 }
 
 // ------------------------------------------------------------------ fused region
-// H~^{n+1/2} components at node q straight from global memory (input parity);
-// used once per z-segment for the plane below the segment.
-template <typename T>
-struct Fields {
-    const T *__restrict__ ex, *__restrict__ ey, *__restrict__ ez;
-    const T *__restrict__ hx, *__restrict__ hy, *__restrict__ hz;
-    T *__restrict__ oex, *__restrict__ oey, *__restrict__ oez;
-    T *__restrict__ ohx, *__restrict__ ohy, *__restrict__ ohz;
-    Fields() = default;
-};
-
 __device__ __forceinline__ int cid_at(const Board *B, long long idx)
 {
     return B->id16 ? (int)__ldg((const uint16_t *)B->cid + idx) : (int)__ldg((const uint8_t *)B->cid + idx);
 }
 
-__device__ __constant__ Coef kOne = {1.0f, 1.0f, 1.0f, 1.0f};
-
-// z-UPML plane kinds of the fused region: 0 none, 1 lower box, 2 upper box.
-__device__ __forceinline__ int zbox_of(const Board *B, int k) { return k < B->iz0 ? 1 : (k >= B->iz1 ? 2 : 0); }
-
-__device__ __forceinline__ long long zaux_index(const Board *B, int box, int i, int j, int k)
-{
-    const int k0 = box == 1 ? B->zlo : B->iz1;
-    return ((long long)(k - k0) * (B->iy1 - B->iy0) + (j - B->iy0)) * (long long)B->zpitch + (i - B->ix0);
-}
-
-// New H~x, H~y, H~z at a fused-region node from already-fetched operands.
-// In z-UPML planes only sigma_z is non-zero: H~x and H~y update in the lossy
-// form (no auxiliary), H~z carries B~z.
+// In z-UPML planes only sigma_z is non-zero: H~x, H~y, E_x, E_y update in the
+// lossy form (no auxiliary), H~z carries B~z and E_z carries D~z.
 struct ZCoef {
     Coef zi, zh;   // z factors at the node's integer and half positions
 };
-
-__device__ __forceinline__ float fused_hx(float h, float sc, int zb, const ZCoef &z)
-{
-    float dummy;
-    if (!zb) return __fsub_rn(h, sc);
-    return upml_h2(h, sc, kOne, z.zh, kOne, false, 0.f, dummy);
-}
-__device__ __forceinline__ float fused_hy(float h, float sc, int zb, const ZCoef &z)
-{
-    float dummy;
-    if (!zb) return __fsub_rn(h, sc);
-    return upml_h2(h, sc, z.zh, kOne, kOne, false, 0.f, dummy);
-}
-__device__ __forceinline__ float fused_hz(float h, float sc, int zb, const ZCoef &z, float Bo, float &Bn)
-{
-    if (!zb) return __fsub_rn(h, sc);
-    return upml_h2(h, sc, kOne, kOne, z.zi, true, Bo, Bn);
-}
 
 // ------------------------------------------------------------------ TMA + mbarrier
 __device__ __forceinline__ uint32_t s_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -358,9 +317,12 @@ __device__ __forceinline__ float2 rnd2(float2 v) { return make_float2(rnd<T>(v.x
 // took 95 us on the 480x380x100 FP16 board with those tests per row, 86.5 now;
 // 364 and 350 on the 880x680x100 FP32 board (a step 638 and 622).  More blocks
 // an SM at 72 or 96 registers spill: 101 us FP16 interior, 96 us FP16 z-UPML
-// launch (66.5 at 128).  In z-UPML planes (sigma_z only) H~z carries B~z and E_z carries
-// D~z, while H~x, H~y, E_x, E_y update in the lossy form; those planes use
-// the scalar update helpers per element, every other plane the paired form.
+// launch (66.5 at 128).  In z-UPML planes (sigma_z only) H~z carries B~z and
+// E_z carries D~z, while H~x, H~y, E_x, E_y update in the lossy form; all in
+// paired arithmetic, with paired auxiliaries where the fused region starts at
+// an even column (per element with the general factors: FP16 66.3 us on the
+// 480x380x100 board, now 65.4, a step 197.3 and 195.6; FP32 183 and 184 on
+// 880x680x100, where HBM latency at three blocks an SM bounds it).
 template <typename T, int TY, int W, int NS, bool ZP, int R>
 __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP, R>::MINB)) k_fused(Plan plan)
 {
@@ -496,6 +458,7 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
         const int acol = (ca - ix0) - ((((i0 - 1) & ~1) - ix0) & ~3);       // column of ca in the aux boxes
         int s0 = sq, s1 = sq + 1 == NS ? 0 : sq + 1;
         // z-UPML launch: the item's box, and the factors along z
+        const bool zeven = (ix0 & 1) == 0;   // a lane's auxiliaries are 8-byte aligned
         const int zbox = ZP && kb >= iz1 ? 1 : 0, kz = ZP ? (zbox ? iz1 : B->zlo) : 0;
         float *const zdz = ZP ? B->zD[zbox] : nullptr, *const nzbz = ZP ? B->zB[zbox][par ^ 1] : nullptr;
         const Coef *const cz0 = ZP ? B->cw[2][0] : nullptr, *const cz1 = ZP ? B->cw[2][1] : nullptr;
@@ -600,14 +563,12 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
                     }
                 } else {
                     // B~z of the node: box row rr; zero outside the fused rows
-                    float2 boz = make_float2(A0[rr * AW], A0[rr * AW + 1]);
+                    float2 boz = zeven ? *reinterpret_cast<const float2 *>(A0 + rr * AW) : make_float2(A0[rr * AW], A0[rr * AW + 1]);
                     if (!in_f) boz = make_float2(0.f, 0.f);
-                    hx.x = fused_hx(ohx.x, scx.x, zb, z);
-                    hx.y = fused_hx(ohx.y, scx.y, zb, z);
-                    hy.x = fused_hy(ohy.x, scy.x, zb, z);
-                    hy.y = fused_hy(ohy.y, scy.y, zb, z);
-                    hz.x = fused_hz(ohz.x, scz.x, zb, z, boz.x, nbz.x);
-                    hz.y = fused_hz(ohz.y, scz.y, zb, z, boz.y, nbz.y);
+                    hx = __ffma2_rn(two(-z.zh.g), scx, __fmul2_rn(two(z.zh.b1), ohx));
+                    hy = __ffma2_rn(two(-z.zh.g), scy, __fmul2_rn(two(z.zh.b1), ohy));
+                    nbz = sub2(boz, scz);
+                    hz = __ffma2_rn(__ffma2_rn(two(z.zi.ap), nbz, __fmul2_rn(two(-z.zi.am), boz)), two(1.f), ohz);
                 }
             };
             // z-UPML launch: halo elements outside the fused region come from the slab output
@@ -662,16 +623,19 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
                     } else {
                         const long long a = za + (long long)r * zrow;
                         const float *dzo = A0 + BCS + r * AW;   // D~z of the node (box row r)
-                        float nd;
-                        float2 ndz;
-                        exv.x = upml_e2(ex.x, scx.x, cea[r].x, kOne, z.zi, kOne, false, 0.f, nd);
-                        exv.y = upml_e2(ex.y, scx.y, ceb[r].x, kOne, z.zi, kOne, false, 0.f, nd);
-                        eyv.x = upml_e2(ey.x, scy.x, cea[r].y, z.zi, kOne, kOne, false, 0.f, nd);
-                        eyv.y = upml_e2(ey.y, scy.y, ceb[r].y, z.zi, kOne, kOne, false, 0.f, nd);
-                        ezv.x = upml_e2(ez.x, scz.x, cea[r].z, kOne, kOne, z.zh, true, dzo[0], ndz.x);
-                        ezv.y = upml_e2(ez.y, scz.y, ceb[r].z, kOne, kOne, z.zh, true, dzo[1], ndz.y);
-                        if (own_a) { stg1(zdz + a, ndz.x); stg1(nzbz + a, nbz.x); }
-                        if (own_b) { stg1(zdz + a + 1, ndz.y); stg1(nzbz + a + 1, nbz.y); }
+                        const float2 doz = zeven ? *reinterpret_cast<const float2 *>(dzo) : make_float2(dzo[0], dzo[1]);
+                        const float2 cx = make_float2(cea[r].x, ceb[r].x), cy = make_float2(cea[r].y, ceb[r].y);
+                        const float2 cz = make_float2(cea[r].z, ceb[r].z);
+                        exv = __ffma2_rn(__fmul2_rn(cx, two(z.zi.g)), scx, __fmul2_rn(two(z.zi.b1), ex));
+                        eyv = __ffma2_rn(__fmul2_rn(cy, two(z.zi.g)), scy, __fmul2_rn(two(z.zi.b1), ey));
+                        const float2 ndz = __ffma2_rn(scz, two(1.f), doz);
+                        ezv = __ffma2_rn(cz, __ffma2_rn(two(z.zh.ap), ndz, __fmul2_rn(two(-z.zh.am), doz)), ez);
+                        if (zeven && own_2) { stg2(zdz + a, ndz); stg2(nzbz + a, nbz); }
+                        if (!zeven || split) {
+                            const bool one = !zeven || !own_2;
+                            if (one && own_a) { stg1(zdz + a, ndz.x); stg1(nzbz + a, nbz.x); }
+                            if (one && own_b) { stg1(zdz + a + 1, ndz.y); stg1(nzbz + a + 1, nbz.y); }
+                        }
                     }
                     if (own_2) {
                         stg2(o + 3 * NN, hx); stg2(o + 4 * NN, hy); stg2(o + 5 * NN, hz);
