@@ -3,8 +3,9 @@
 // Host side of the CUDA path: validates the problem, precomputes what the
 // kernels read (per-edge permittivity -> <=256-entry coefficient table +
 // uint8 id per node, Eq. 5 grading -> 1D UPML factors per axis, Eq. 7 time
-// step, slab decomposition of the UPML), owns device memory, captures chunks
-// of steps into CUDA graphs and batches boards into one launch per phase.
+// step, slab decomposition of the UPML), owns device memory, and runs steps: many
+// to a cooperative launch (fdtd_resident.cu, resident_plan.h) or one launch per
+// phase in CUDA graphs of a chunk of steps; boards of a batch share launches.
 #include <nvtx3/nvToolsExt.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

@@ -38,7 +38,7 @@
 // [iz1,nz)) have sigma_z only, so they carry D~z (updated in place) and B~z
 // (ping-ponged, since neighbouring tiles recompute halo H from it) in compact
 // [k][j][i] boxes.  Everything else (x/y UPML slabs with their
-// edges and corners, and the outer z planes) is updated by generic slab
+// edges and corners, and the outer z planes) is updated by the slab
 // kernels whose auxiliary D~/B~ live in compact [k][j][i] boxes per slab, only
 // for components whose recurrence there is not trivial.
 #pragma once

@@ -1,7 +1,10 @@
-// fdtd_kernels.cu -- sm_103a kernels of the Yee + UPML leapfrog step.
+// fdtd_kernels.cu -- sm_103a kernels of the Yee + UPML leapfrog step, one
+// launch per phase.
 //
-// One step (Model section: H at half steps from E, then E from H and J) is
-// five launches over a Plan (one board or a batch of boards):
+// One step (Model section: H at half steps from E, then E from H and J) of a
+// board past the limit of the resident launches (fdtd_resident.cu), in 16-bit
+// storage or at depth 2 is five launches over a Plan (one board or a batch of
+// boards), the interior one beside the first two (launch_step):
 //   k_slab_h        H^{n+1/2} (and B~) on the x/y UPML slabs and the outer
 //                   z planes                                        (Eqs. 1-5)
 //   k_fused<..,1>   fused H^{n+1/2} and E^{n+1} on the interior columns'
