@@ -1269,9 +1269,10 @@ __global__ void __launch_bounds__(PairLayout<T>::THREADS, 2) k_pair(Plan plan)
 // storage) without staging.  Bound by the latency of those loads: 12 warps an
 // SM at 168 registers keep some 60 KB in flight.  (One node a thread with
 // 4-byte cp.async words into shared-memory rings, as before, took slab H + E
-// 68.5 + 82.6 us on the 880x680x100 board, now 56.5 + 66.9; FP16 at 480x380x100
-// 42.7 + 47.7, now 39.4 + 41.0.  Four blocks an SM at 128 registers spill: 58 +
-// 80; runs of 8 planes instead of 4: the same in FP32, 43.6 + 44.8 in FP16.)
+// 68.5 + 82.6 us on the 880x680x100 board, now 54.8 + 64.8; FP16 at 480x380x100
+// 42.7 + 47.7, now 32.6 + 36.2.  Before the prefetch, 56.5 + 66.9 and 39.4 +
+// 41.0: four blocks an SM at 128 registers spill, 58 + 80; runs of 8 planes
+// instead of 4 the same in FP32, 43.6 + 44.8 in FP16.)
 //
 // Neighbours past the grid's last column, row or plane, or before its first,
 // are read from the adjoining component's memory: in bounds (a set's six
@@ -1941,9 +1942,9 @@ cudaError_t launch_pair(const Plan &plan, int prec, int grid_cap, cudaStream_t s
 
 // One step.  The interior launch depends on no other launch of the step, so it
 // runs on the side stream beside slab H and the z-UPML launch: the blocks of
-// one fill the SMs that the others' last waves leave (880x680x100 669 us a step
-// one after the other, 643 so; 480x380x100 FP16 239 and 220, 280x230x100 FP16
-// 136 and 119).
+// one fill the SMs that the others' last waves leave (when the launches took 10
+// % longer than now: 880x680x100 669 us a step one after the other, 643 so;
+// 480x380x100 FP16 239 and 220, 280x230x100 FP16 136 and 119).
 cudaError_t launch_step(const Plan &plan, int prec, int grid_cap, cudaStream_t st, const SideStream &side)
 {
     cudaError_t e = cudaSuccess;

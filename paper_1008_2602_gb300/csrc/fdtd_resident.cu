@@ -10,14 +10,15 @@
 // barrier ends each (1.2 us measured over 152 blocks).  Nothing is recomputed
 // and nothing is staged: all reads of a phase are of values the phases before
 // it finished, so every warp issues its loads at once and L2 serves them
-// (12-13.7 TB/s measured up to 90 MB); there a phase is bound by L2 latency
-// (small boards) or L2 bandwidth, past L2 by HBM at 73 B a node and step.
+// (12-13.7 TB/s measured up to 90 MB).  A phase is bound by L2 latency and the
+// barrier on small boards, by the load pipe's wavefronts in the middle (with
+// H held in shared memory 232x192x39 gained only 1 %), past L2 by HBM at 73 B a
+// node and step.
 //
-// Measured (us a step, launch-per-phase path -> here): 38x33x20 57 -> 4.5 and
-// 56x48x30 62 -> 4.5 (k_pinned), 181x131x6 34 -> 5.9, 232x192x39 90 -> 22.1,
-// 280x230x100 160 -> 95, 480x380x100 294 -> 259; a batch of 24 boards (41 M
-// cells) 852 -> 618.  At 880x680x100 the tiled launches' 49 B a node win (697
-// against 902).
+// Measured (us a step, launch-per-phase path as it was before this file ->
+// here): 38x33x20 57 -> 4.5 and 56x48x30 62 -> 4.5 (k_pinned), 181x131x6 34 ->
+// 5.9, 232x192x39 90 -> 21.7, 280x230x100 160 -> 92; a batch of 24 boards (41 M
+// cells) 852 -> 607.  Larger boards: see kResPoints.
 //
 // The work is cut into units of 32 column quads (128 nodes), taken in x, y, z
 // order from one box at a time.  The boxes are the board's own (slab boxes,
