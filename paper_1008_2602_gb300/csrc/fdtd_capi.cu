@@ -857,7 +857,7 @@ long long dft_items(const Board &h)
     return (long long)h.n_bins * ((h.n_probe + kDftProbeGroup - 1) / kDftProbeGroup);
 }
 
-// Lay out plan arrays [boards | int_prefix | zp_prefix | slab_prefix | dft_prefix | work | slab blocks] in buf.
+// Lay out plan arrays [boards | int_prefix | zp_prefix | slab block counts | dft_prefix | work | slab blocks] in buf.
 int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, bool tiled, long long *&buf, size_t &cap,
                Plan &plan, cudaStream_t st, std::vector<long long> &host)
 {
@@ -933,7 +933,6 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, b
     plan.boards = (Board *const *)buf;
     plan.int_prefix = buf + nb;
     plan.zp_prefix = buf + nb + (nb + 1);
-    plan.slab_prefix = buf + nb + 2 * (nb + 1);
     plan.dft_prefix = buf + nb + 3 * (nb + 1);
     plan.n_int = ip[nb];
     plan.n_zp = zp[nb];

@@ -233,7 +233,6 @@ struct Plan {
     Board *const *boards;         // [nb] device pointers
     const long long *int_prefix;  // [nb + 1] interior-kernel items (planes [iz0, iz1))
     const long long *zp_prefix;   // [nb + 1] z-UPML-kernel items (planes [zlo, iz0) and [iz1, nz))
-    const long long *slab_prefix; // [nb + 1] slab blocks
     const SlabBlock *slab_blk;    // [n_slab] per-block descriptors
     const long long *dft_prefix;  // [nb + 1] DFT warps
     long long n_int, n_zp, n_slab, n_dft;

@@ -39,11 +39,6 @@ __device__ __forceinline__ int find_board(const long long *prefix, int nb, long 
     return lo;
 }
 
-__device__ __forceinline__ bool board_active(const Board *B)
-{
-    return *((volatile long long *)B->step) < *((volatile long long *)B->stop);
-}
-
 // The step counters as seen by the field kernels: written only by other
 // launches (k_post, the host's stop updates), so within one launch they are
 // read-only and every warp may read them through the cached read-only path
@@ -111,7 +106,6 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
         "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(s_addr(bar))
         : "memory");
 }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 
 template <typename T>
