@@ -1939,16 +1939,33 @@ cudaError_t launch_pair(const Plan &plan, int prec, int grid_cap, cudaStream_t s
 // one fill the SMs that the others' last waves leave (when the launches took 10
 // % longer than now: 880x680x100 669 us a step one after the other, 643 so;
 // 480x380x100 FP16 239 and 220, 280x230x100 FP16 136 and 119).
+//
+// Whose last wave is filled: with the fork before slab H the interior launch
+// fills slab H's and leaves the z-UPML launch's bare; with the fork after it
+// the z-UPML launch comes first and the interior fills up behind it.  The
+// second way wins while the z-UPML launch is a few waves of its 456 blocks (us
+// a step, first and second way: FP16 232x192x39, 528 items, 45.4 and 43.4;
+// 280x230x100, 540, 95.6 and 89.7; 480x380x100, 1440, 195.8 and 190.7; FP32
+// 480x380x100 241.4 and 240.6; 640x500x100, 2400, 367.2 and 366.2), not past
+// that (880x680x100, 4648, 624.9 and 631.8; FP16 471 and 474).
+constexpr long long kZFirstItems = 3000;
 cudaError_t launch_step(const Plan &plan, int prec, int grid_cap, cudaStream_t st, const SideStream &side)
 {
     cudaError_t e = cudaSuccess;
     auto run = [&](int ph, cudaStream_t on) { if (e == cudaSuccess) e = launch_phase(plan, prec, ph, grid_cap, on); };
     auto ok = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    ok(cudaEventRecord(side.start, st));
-    ok(cudaStreamWaitEvent(side.stream, side.start, 0));
-    run(kPhaseSlabH, st);
-    run(kPhaseInterior, side.stream);
-    run(kPhaseFusedZ, st);
+    auto fork = [&] { ok(cudaEventRecord(side.start, st)); ok(cudaStreamWaitEvent(side.stream, side.start, 0)); };
+    if (plan.n_zp > 0 && plan.n_zp < kZFirstItems) {
+        run(kPhaseSlabH, st);
+        fork();
+        run(kPhaseFusedZ, st);
+        run(kPhaseInterior, side.stream);
+    } else {
+        fork();
+        run(kPhaseSlabH, st);
+        run(kPhaseInterior, side.stream);
+        run(kPhaseFusedZ, st);
+    }
     ok(cudaEventRecord(side.done, side.stream));
     ok(cudaStreamWaitEvent(st, side.done, 0));
     run(kPhaseSlabE, st);
