@@ -1446,11 +1446,12 @@ int fdtd_create(const fdtd_grid *grid, const uint8_t *mat_ids, const double *eps
     if (r) { fdtd_destroy(c); return r; }
     if ((r = set_geometry(c, mat_ids))) { fdtd_destroy(c); return r; }
 
-    // UPML factors: one allocation, one upload
+    // UPML factors: one allocation, one upload (read from `all` by the time the
+    // stream is waited for, at the end)
     Axes A;
     build_axes(c, A);
+    std::vector<Coef> all;
     {
-        std::vector<Coef> all;
         for (int w = 0; w < 3; ++w)
             for (int s = 0; s < 2; ++s) all.insert(all.end(), A.cw[w][s].begin(), A.cw[w][s].end());
         Coef *d = nullptr;

@@ -1,0 +1,184 @@
+// The library's host code (csrc/fdtd_capi.cu) over a CUDA runtime of its own:
+// device memory is host memory, and what is queued on a stream runs only when
+// the stream is waited for, as a runtime may do it.  The kernels are replaced
+// by launches that advance the step counters and note which path they belong
+// to.  Host memory that is freed is overwritten and kept, so that a copy
+// queued from it shows.  One scenario per run, named by the first argument.
+#include <cstdio>
+#include <cstdlib>
+#include <functional>
+#include <malloc.h>
+#include <new>
+
+void *operator new(size_t n) { return std::malloc(n ? n : 1); }
+void operator delete(void *p) noexcept { if (p) __builtin_memset(p, 0xA5, malloc_usable_size(p)); }
+void operator delete(void *p, size_t) noexcept { operator delete(p); }
+
+#include "fdtd_capi.cu"
+
+typedef std::vector<std::function<void()>> Ops;
+static Ops queued, *recording = nullptr;
+static void later(std::function<void()> f) { (recording ? *recording : queued).push_back(std::move(f)); }
+static void drain()
+{
+    for (size_t i = 0; i < queued.size(); ++i) queued[i]();
+    queued.clear();
+}
+
+extern "C" {
+cudaError_t cudaMalloc(void **p, size_t n) { *p = std::aligned_alloc(256, (n + 255) / 256 * 256); return cudaSuccess; }
+cudaError_t cudaFree(void *) { drain(); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t)
+{
+    later([=] { std::memcpy(d, s, n); });
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { drain(); std::memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) { later([=] { std::memset(p, v, n); }); return cudaSuccess; }
+static void copy2d(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h)
+{
+    for (size_t r = 0; r < h; ++r) std::memcpy((char *)d + r * dp, (const char *)s + r * sp, w);
+}
+cudaError_t cudaMemcpy2DAsync(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind, cudaStream_t)
+{
+    later([=] { copy2d(d, dp, s, sp, w, h); });
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpy2D(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind)
+{
+    drain();
+    copy2d(d, dp, s, sp, w, h);
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpy3DPeerAsync(const cudaMemcpy3DPeerParms *q, cudaStream_t)
+{
+    const cudaMemcpy3DPeerParms p = *q;
+    later([=] { copy2d(p.dstPtr.ptr, p.dstPtr.pitch, p.srcPtr.ptr, p.srcPtr.pitch, p.extent.width, p.extent.height); });
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) { drain(); return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = (cudaStream_t)std::malloc(1); return cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { recording = new Ops; return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g)
+{
+    *g = (cudaGraph_t)recording;
+    recording = nullptr;
+    return cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t g, unsigned long long) { *e = (cudaGraphExec_t)g; return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t)
+{
+    for (auto &f : *(Ops *)e) queued.push_back(f);
+    return cudaSuccess;
+}
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *) { return cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *, unsigned) { return cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 0.f; return cudaSuccess; }
+cudaError_t cudaHostRegister(void *, size_t, unsigned) { return cudaErrorNotSupported; }
+cudaError_t cudaHostUnregister(void *) { return cudaSuccess; }
+cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+const char *cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **p, unsigned, unsigned long long, cudaDriverEntryPointQueryResult *q)
+{
+    static auto encode = [](CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
+                            const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                            CUtensorMapL2promotion, CUtensorMapFloatOOBfill) { return CUDA_SUCCESS; };
+    *p = (void *)(PFN_cuTensorMapEncodeTiled_v12000)encode;
+    *q = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
+}
+
+// The kernels: which path advanced a board by how many steps.
+static long long tiled_steps, resident_steps;
+static void advance(Board *const *boards, int b, int n, long long &count)
+{
+    Board *const B = boards[b];
+    const long long did = std::max(0LL, std::min<long long>(n, *B->stop - *B->step));
+    *B->step += did;
+    count += did;
+}
+namespace fdtd {
+cudaError_t launch_step(const Plan &p, int, int, cudaStream_t, const SideStream &)
+{
+    later([p] { for (int b = 0; b < p.nb; ++b) advance(p.boards, b, 1, tiled_steps); });
+    return cudaSuccess;
+}
+cudaError_t launch_phase(const Plan &p, int prec, int phase, int cap, cudaStream_t st)
+{
+    return phase == kPhasePost ? launch_step(p, prec, cap, st, SideStream{}) : cudaSuccess;
+}
+cudaError_t launch_pair(const Plan &p, int, int, cudaStream_t)
+{
+    later([p] { advance(p.boards, 0, 2, tiled_steps); });
+    return cudaSuccess;
+}
+cudaError_t launch_pair_part(const Plan &p, int prec, int i, int cap, cudaStream_t st) { return launch_phase(p, prec, kPairPhase[i], cap, st); }
+cudaError_t launch_resident(const ResPlan &p, int n, cudaStream_t)
+{
+    later([p, n] {
+        for (int b = 0; b < p.n_blocks; ++b)
+            if (p.blocks[b].first) advance(p.boards, p.teams[p.blocks[b].team].board, n, resident_steps);
+    });
+    return cudaSuccess;
+}
+size_t resident_smem(const ResPlan &) { return 0; }
+size_t resident_arrive_bytes(int n) { return (size_t)n * 128; }
+cudaError_t resident_set_smem_limit() { return cudaSuccess; }
+cudaError_t launch_dft(const Plan &, int, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_set_i64(long long *p, long long v, cudaStream_t) { later([=] { *p = v; }); return cudaSuccess; }
+cudaError_t launch_energy(const Board *, const Board &, double *, int, double *, cudaStream_t) { return cudaSuccess; }
+int energy_partials(const Board &) { return 1; }
+cudaError_t fused_set_smem_limits() { return cudaSuccess; }
+bool fused_tile_supported(int tx, int ty) { return (tx == 62 || tx == 124) && (ty == 4 || ty == 8); }
+cudaError_t launch_wait_selftest(int *status, unsigned, cudaStream_t) { later([=] { *status = 2; }); return cudaSuccess; }
+}
+
+static int bad = 0;
+static void expect(bool ok, const char *what)
+{
+    if (!ok) {
+        std::printf("not so: %s\n", what);
+        ++bad;
+    }
+}
+
+static fdtd_ctx *board(int nx, int ny, int nz, int depth, int prec = FDTD_FP32)
+{
+    fdtd_grid g{nx, ny, nz, 1e-3, 1e-3, 1e-3, 0.99, 0.0};
+    fdtd_boundary b{};
+    for (int f = 0; f < 6; ++f) b.depth[f] = depth;
+    b.m = 3.0; b.R0 = 1e-6; b.kappa_max = 1.0;
+    const std::vector<uint8_t> mat((size_t)nx * ny * nz, 0);
+    const double eps = 1.0;
+    fdtd_ctx *c = nullptr;
+    expect(fdtd_create(&g, mat.data(), &eps, 1, nullptr, 0, nullptr, &b, prec, nullptr, &c) == FDTD_OK, "the board is created");
+    return c;
+}
+
+static void factors()
+{
+    fdtd_ctx *c = board(30, 24, 20, 4);
+    Axes A;
+    build_axes(c, A);
+    for (int w = 0; w < 3; ++w)
+        for (int s = 0; s < 2; ++s)
+            expect(!std::memcmp(c->h.cw[w][s], A.cw[w][s].data(), sizeof(Coef) * A.cw[w][s].size()), "the UPML factors arrive");
+    fdtd_destroy(c);
+}
+
+int main(int, char **argv)
+{
+    const std::string s = argv[1];
+    if (s == "factors") factors();
+    else expect(false, "a known scenario");
+    return bad;
+}
