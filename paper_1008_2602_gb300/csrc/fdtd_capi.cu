@@ -115,6 +115,7 @@ struct fdtd_ctx {
     size_t rplan_cap = 0;
     bool ports_in_boxes = true;         // every source and probe edge belongs to a box
     bool halo = false;                  // a plane of the state was written from outside
+    bool res_refused = false;           // the device does not take the board's resident launch
     long long *res_buf = nullptr;
     size_t res_cap = 0;
     size_t fbytes = 0;                  // bytes of one field component
@@ -987,8 +988,8 @@ std::vector<ResAt> res_ports(const fdtd_ctx *c)
 bool resident_board(const fdtd_ctx *c, long long n)
 {
     const Board &h = c->h;
-    return c->prec == FDTD_FP32 && !h.pair_ok && grid_points(h) <= kResPoints && 6 * h.nodes < (1LL << 31) &&
-           c->ports_in_boxes && c->src.size() + c->probe.size() <= 512 && h.nx + h.ny + h.nz <= 3000 && (n <= 1 || !c->halo);
+    return c->prec == FDTD_FP32 && !c->res_refused && !h.pair_ok && grid_points(h) <= kResPoints &&
+           6 * h.nodes < (1LL << 31) && c->ports_in_boxes && c->src.size() + c->probe.size() <= 512 && h.nx + h.ny + h.nz <= 3000 && (n <= 1 || !c->halo);
 }
 
 // Upload a resident plan ([arrival counters | teams | blocks | pieces | ports]).
@@ -1656,7 +1657,7 @@ int fdtd_step(fdtd_ctx *c, int n)
     if (int r = finalize(c)) return r;
     const bool resident = resident_board(c, n);
     if (int r = prepare_single(c, !resident)) return r;
-    if (resident) {
+    if (resident && !c->res_refused) {
         if (int r = run_resident(&c->res, 1, c->rplan, c->grid_cap, n, resident_chunk(c->h.nodes), c->cur)) return r;
     } else if (c->h.pair_ok) {
         if (int r = run_depth2(c->plan, c->prec, c->grid_cap, c->host_step, n, c->tune.graph_chunk, c->graph2,
@@ -1670,7 +1671,8 @@ int fdtd_step(fdtd_ctx *c, int n)
 }
 
 // Build what the next launches of a single board need: the plan of the tiled
-// launches, or that of the resident launches.
+// launches, or that of the resident launches (the tiled one all the same where
+// the device does not take those).
 static int prepare_single(fdtd_ctx *c, bool tiled)
 {
     if (int r = finalize(c)) return r;
@@ -1686,6 +1688,10 @@ static int prepare_single(fdtd_ctx *c, bool tiled)
         if (int r = build_resident(c, c->rplan.boards, c->res_buf, c->res_cap, c->res, c->cur, rhost)) return r;
     }
     CK(cudaStreamSynchronize(c->cur));
+    if (!tiled && !resident_fits(c->res)) {
+        c->res_refused = true;
+        return prepare_single(c, true);
+    }
     if (tiled) {
         if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
         if (c->graph2) { cudaGraphExecDestroy(c->graph2); c->graph2 = nullptr; }
@@ -2363,6 +2369,11 @@ static int prepare_batch(fdtd_batch *b)
         b->res_chunk = resident_chunk((long long)(work / (double)b->res.size()) + 1);
     }
     CK(cudaStreamSynchronize(b->stream));
+    for (const ResPlan &p : b->res)
+        if (!resident_fits(p)) {
+            for (fdtd_ctx *c : res) c->res_refused = true;
+            return prepare_batch(b);
+        }
     if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
     b->dirty = false;
     return FDTD_OK;

@@ -363,6 +363,7 @@ cudaError_t launch_pair_part(const Plan &plan, int prec, int idx, int grid_cap, 
 size_t resident_smem(const ResPlan &plan);
 size_t resident_arrive_bytes(int n_teams);
 cudaError_t resident_set_smem_limit();
+bool resident_fits(const ResPlan &plan);   // whether the device takes the plan's cooperative launch
 cudaError_t launch_resident(const ResPlan &plan, int nsteps, cudaStream_t st);
 cudaError_t launch_dft(const Plan &plan, int grid_cap, cudaStream_t st);
 cudaError_t launch_set_i64(long long *p, long long v, cudaStream_t st);

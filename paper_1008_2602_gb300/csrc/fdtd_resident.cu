@@ -832,16 +832,31 @@ cudaError_t resident_set_smem_limit()
 
 size_t resident_arrive_bytes(int n_teams) { return (size_t)n_teams * 128; }
 
+static bool pins(const ResPlan &plan) { return plan.max_units <= kPinWarps; }
+static const void *kernel_of(const ResPlan &plan) { return pins(plan) ? (const void *)k_pinned : (const void *)k_resident; }
+static int threads_of(const ResPlan &plan) { return pins(plan) ? kPinThreads : kResThreads; }
+
+// The driver refuses a cooperative launch whose blocks cannot all be resident
+// at once (too few SMs for this process, or too little of each).
+bool resident_fits(const ResPlan &plan)
+{
+    int dev = 0, coop = 0, sms = 0, per = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of(plan), threads_of(plan), resident_smem(plan)) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return coop != 0 && plan.n_blocks <= sms * per;
+}
+
 cudaError_t launch_resident(const ResPlan &plan, int nsteps, cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(plan.arrive, 0, resident_arrive_bytes(plan.all_teams), st);
     if (e != cudaSuccess) return e;
     ResPlan p = plan;
     void *args[] = {&p, &nsteps};
-    const bool pin = plan.max_units <= kPinWarps;
-    const void *const kernel = pin ? (const void *)k_pinned : (const void *)k_resident;
-    return cudaLaunchCooperativeKernel(kernel, dim3(plan.n_blocks), dim3(pin ? kPinThreads : kResThreads), args,
-                                       resident_smem(plan), st);
+    return cudaLaunchCooperativeKernel(kernel_of(plan), dim3(plan.n_blocks), dim3(threads_of(plan)), args, resident_smem(plan), st);
 }
 
 }  // namespace fdtd

@@ -99,6 +99,7 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **p, unsigned, u
 
 // The kernels: which path advanced a board by how many steps.
 static long long tiled_steps, resident_steps;
+static bool refuse_cooperative;   // the device takes no resident launch
 static void advance(Board *const *boards, int b, int n, long long &count)
 {
     Board *const B = boards[b];
@@ -122,8 +123,10 @@ cudaError_t launch_pair(const Plan &p, int, int, cudaStream_t)
     return cudaSuccess;
 }
 cudaError_t launch_pair_part(const Plan &p, int prec, int i, int cap, cudaStream_t st) { return launch_phase(p, prec, kPairPhase[i], cap, st); }
+bool resident_fits(const ResPlan &) { return !refuse_cooperative; }
 cudaError_t launch_resident(const ResPlan &p, int n, cudaStream_t)
 {
+    if (refuse_cooperative) return cudaErrorCooperativeLaunchTooLarge;
     later([p, n] {
         for (int b = 0; b < p.n_blocks; ++b)
             if (p.blocks[b].first) advance(p.boards, p.teams[p.blocks[b].team].board, n, resident_steps);
@@ -175,10 +178,46 @@ static void factors()
     fdtd_destroy(c);
 }
 
+// Steps of a call, by path.
+struct Took {
+    long long tiled, resident;
+    Took() : tiled(-tiled_steps), resident(-resident_steps) {}
+    bool is(long long t, long long r)
+    {
+        drain();
+        return tiled + tiled_steps == t && resident + resident_steps == r;
+    }
+};
+
+static void refused()
+{
+    fdtd_ctx *a = board(30, 24, 20, 4), *c[2] = {board(30, 24, 20, 4), board(25, 24, 20, 4)};
+    {
+        Took t;
+        expect(fdtd_step(a, 20) == FDTD_OK && t.is(0, 20), "the board takes resident launches");
+    }
+    refuse_cooperative = true;
+    a->plan_dirty = true;
+    Took t;
+    expect(fdtd_step(a, 20) == FDTD_OK && t.is(20, 0), "a board steps where the device takes no resident launch");
+    Took u;
+    expect(fdtd_step(a, 5) == FDTD_OK && u.is(5, 0), "and goes on so");
+    fdtd_batch *b = nullptr;
+    int done = 0;
+    expect(fdtd_batch_create(nullptr, &b) == FDTD_OK, "the batch is created");
+    for (fdtd_ctx *m : c) expect(fdtd_batch_add(b, m, 20) == FDTD_OK, "a board joins");
+    Took v;
+    expect(fdtd_batch_step(b, 20, &done) == FDTD_OK && v.is(40, 0) && done == 2, "a batch steps there");
+    fdtd_batch_destroy(b);
+    for (fdtd_ctx *m : c) fdtd_destroy(m);
+    fdtd_destroy(a);
+}
+
 int main(int, char **argv)
 {
     const std::string s = argv[1];
     if (s == "factors") factors();
+    else if (s == "refused") refused();
     else expect(false, "a known scenario");
     return bad;
 }
