@@ -164,10 +164,23 @@ int fdtd_set_spectrum(fdtd_ctx *ctx, double f_max, int n_total_steps);
 /* Advance n >= 0 leapfrog steps (H^{n+1/2} from E^n, then E^{n+1} from
  * H^{n+1/2} and J^{n+1/2}, then probes and DFT).  Asynchronous on the
  * context's stream; fields stay on the device between calls.  FP32 boards up
- * to 14 Mi grid points at depth 1 run many steps per cooperative launch, the
- * others five launches per step replayed as CUDA graphs; a board's fields and
- * traces are the same bit for bit either way. */
+ * to 14 Mi grid points at depth 1 run many steps per cooperative launch
+ * ("resident"; also at most 512 sources and probes, nx + ny + nz <= 3000, and
+ * no plane written by fdtd_halo_unpack or _copy where n > 1), the others five
+ * launches per step replayed as CUDA graphs ("tiled"); a board's fields and
+ * traces are the same bit for bit either way.  A device that cannot hold a
+ * resident launch runs the tiled ones. */
 int fdtd_step(fdtd_ctx *ctx, int n);
+
+/* A resident launch needs every SM to itself: it starts once the kernels of
+ * other streams have left them, and they wait for it.  A program whose other
+ * kernels stay on the GPU for long, or wait for this board's results there,
+ * sets `on`: the context then steps by tiled launches alone, in a batch too,
+ * from the next call until it is set back to 0 (the default).
+ * fdtd_is_resident says in *resident whether the next fdtd_step(ctx, n), n >= 1
+ * (or its batch's next step), goes by resident launches. */
+int fdtd_set_tiled(fdtd_ctx *ctx, int on);
+int fdtd_is_resident(fdtd_ctx *ctx, int n, int *resident);
 
 /* fdtd_step with every phase launched directly (no CUDA graph) and timed
  * with CUDA events on the context's stream: phase_ms[0..5] receive the summed

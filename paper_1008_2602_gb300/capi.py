@@ -67,6 +67,8 @@ _SIGS = {
     "fdtd_get_plane": (c_int, [c_void_p, c_int, c_int, c_void_p]),
     "fdtd_set_spectrum": (c_int, [c_void_p, c_double, c_int]),
     "fdtd_step": (c_int, [c_void_p, c_int]),
+    "fdtd_set_tiled": (c_int, [c_void_p, c_int]),
+    "fdtd_is_resident": (c_int, [c_void_p, c_int, P(c_int)]),
     "fdtd_step_profiled": (c_int, [c_void_p, c_int, P(c_double)]),
     "fdtd_probe_spectra": (c_int, [c_void_p, c_void_p, c_int, P(c_int)]),
     "fdtd_probe_trace": (c_int, [c_void_p, c_int, c_void_p, c_int, P(c_int)]),

@@ -116,6 +116,7 @@ struct fdtd_ctx {
     bool ports_in_boxes = true;         // every source and probe edge belongs to a box
     bool halo = false;                  // a plane of the state was written from outside
     bool res_refused = false;           // the device does not take the board's resident launch
+    bool tiled_only = false;            // fdtd_set_tiled
     long long *res_buf = nullptr;
     size_t res_cap = 0;
     size_t fbytes = 0;                  // bytes of one field component
@@ -667,9 +668,24 @@ int upload_board(fdtd_ctx *c)
     return FDTD_OK;
 }
 
+// Source and probe edges of a board, as a resident plan places them.
+std::vector<ResAt> res_ports(const fdtd_ctx *c)
+{
+    std::vector<ResAt> at;
+    for (size_t s = 0; s < c->src.size(); ++s) at.push_back({c->src[s].i, c->src[s].j, c->src[s].k, c->src[s].comp, 0, (int)s});
+    for (size_t p = 0; p < c->probe.size(); ++p)
+        at.push_back({c->probe[p].i, c->probe[p].j, c->probe[p].k, c->probe[p].comp, 1, (int)p});
+    return at;
+}
+bool ports_in_boxes(const fdtd_ctx *c)
+{
+    for (const ResAt &a : res_ports(c))
+        if (res_box_of(c->h, a.i, a.j, a.k) < 0) return false;
+    return true;
+}
+
 // Decide the storage scale, upload sources/probes/trace buffers and the
 // descriptor; called once before the first step.
-std::vector<ResAt> res_ports(const fdtd_ctx *c);
 int finalize(fdtd_ctx *c)
 {
     if (c->started) return FDTD_OK;
@@ -717,7 +733,7 @@ int finalize(fdtd_ctx *c)
         c->h.trace = tr;
         c->h.dft = dft;
     }
-    for (const ResAt &a : res_ports(c)) c->ports_in_boxes = c->ports_in_boxes && res_box_of(c->h, a.i, a.j, a.k) >= 0;
+    c->ports_in_boxes = ports_in_boxes(c);
     c->started = true;
     c->plan_dirty = true;
     return upload_board(c);
@@ -971,15 +987,6 @@ long long grid_points(const Board &h) { return (long long)(h.nx + 1) * (h.ny + 1
 // 276.
 constexpr long long kResPoints = 14LL << 20;
 
-std::vector<ResAt> res_ports(const fdtd_ctx *c)
-{
-    std::vector<ResAt> at;
-    for (size_t s = 0; s < c->src.size(); ++s) at.push_back({c->src[s].i, c->src[s].j, c->src[s].k, c->src[s].comp, 0, (int)s});
-    for (size_t p = 0; p < c->probe.size(); ++p)
-        at.push_back({c->probe[p].i, c->probe[p].j, c->probe[p].k, c->probe[p].comp, 1, (int)p});
-    return at;
-}
-
 // Whether n steps of a board go to resident launches.  The limits on ports and
 // extents bound their shared-memory tables; a probe on a high wall plane lies in
 // no box; and a plane written from outside (fdtd_halo_unpack, _copy) may be a
@@ -988,7 +995,7 @@ std::vector<ResAt> res_ports(const fdtd_ctx *c)
 bool resident_board(const fdtd_ctx *c, long long n)
 {
     const Board &h = c->h;
-    return c->prec == FDTD_FP32 && !c->res_refused && !h.pair_ok && grid_points(h) <= kResPoints &&
+    return c->prec == FDTD_FP32 && !c->tiled_only && !c->res_refused && !h.pair_ok && grid_points(h) <= kResPoints &&
            6 * h.nodes < (1LL << 31) && c->ports_in_boxes && c->src.size() + c->probe.size() <= 512 && h.nx + h.ny + h.nz <= 3000 && (n <= 1 || !c->halo);
 }
 
@@ -1644,6 +1651,22 @@ int fdtd_set_tuning(fdtd_ctx *c, const fdtd_tuning *t)
         if (int r = set_time_depth(c, n.depth)) return r;
     c->tune = n;
     c->plan_dirty = true;
+    return FDTD_OK;
+}
+
+int fdtd_set_tiled(fdtd_ctx *c, int on)
+{
+    if (!c) return fail(FDTD_EINVAL, "NULL context");
+    c->tiled_only = on != 0;
+    if (c->batch) c->batch->dirty = true;
+    return FDTD_OK;
+}
+
+int fdtd_is_resident(fdtd_ctx *c, int n, int *resident)
+{
+    if (!c || !resident) return fail(FDTD_EINVAL, "NULL argument");
+    if (n < 1) return fail(FDTD_EINVAL, "n must be >= 1");
+    *resident = resident_board(c, c->batch ? 2 : n) && (c->started || ports_in_boxes(c));
     return FDTD_OK;
 }
 

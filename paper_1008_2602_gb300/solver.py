@@ -114,6 +114,17 @@ class Solver:
         t = C.fdtd_tuning(tile_x, tile_y, zseg, graph_chunk, depth, pair_zseg)
         C.fdtd_set_tuning(self.ctx, ctypes.byref(t))
 
+    def set_tiled(self, on: bool = True):
+        """Step by the tiled launches alone, beside which other streams' kernels
+        can run (fdtd_set_tiled)."""
+        C.fdtd_set_tiled(self.ctx, int(on))
+
+    def resident(self, n: int = 2) -> bool:
+        """Whether the next step(n) goes by resident launches (fdtd_is_resident)."""
+        r = ctypes.c_int()
+        C.fdtd_is_resident(self.ctx, int(n), ctypes.byref(r))
+        return bool(r.value)
+
     # -- results ---------------------------------------------------------------
     def info(self) -> dict:
         inf = C.fdtd_info_t()

@@ -213,11 +213,48 @@ static void refused()
     fdtd_destroy(a);
 }
 
+static bool resident(fdtd_ctx *c, int n)
+{
+    int r = -1;
+    expect(fdtd_is_resident(c, n, &r) == FDTD_OK && (r == 0 || r == 1), "the path is told");
+    return r == 1;
+}
+
+static void chosen()
+{
+    fdtd_ctx *a = board(30, 24, 20, 4), *b = board(25, 24, 20, 4), *h = board(25, 24, 20, 4, FDTD_FP16_STORE);
+    expect(resident(a, 1) && resident(a, 20) && !resident(h, 20), "the rule before the first step");
+    for (int on : {1, 0}) {
+        fdtd_set_tiled(a, on);
+        Took t;
+        expect(resident(a, 20) == !on && fdtd_step(a, 20) == FDTD_OK && t.is(on ? 20 : 0, on ? 0 : 20), "a board steps as set");
+    }
+    fdtd_batch *g = nullptr;
+    expect(fdtd_batch_create(nullptr, &g) == FDTD_OK && fdtd_batch_add(g, a, 30) == FDTD_OK && fdtd_batch_add(g, b, 30) == FDTD_OK,
+           "a batch of two");
+    Took t;
+    expect(fdtd_batch_step(g, 10, nullptr) == FDTD_OK && t.is(0, 20), "both members by the rule");
+    fdtd_set_tiled(a, 1);
+    Took u;
+    expect(!resident(a, 10) && resident(b, 10) && fdtd_batch_step(g, 10, nullptr) == FDTD_OK && u.is(10, 10), "each member as set");
+    fdtd_set_tiled(b, 1);
+    Took v;
+    expect(fdtd_batch_step(g, 10, nullptr) == FDTD_OK && v.is(20, 0), "both set");
+    fdtd_batch_destroy(g);
+    // a probe on a high wall plane belongs to no block
+    fdtd_ctx *p = board(25, 24, 20, 4);
+    expect(fdtd_add_probe(p, 25, 3, 3, 2, nullptr) == FDTD_OK && !resident(p, 20), "a port outside the boxes, before the first step");
+    Took w;
+    expect(fdtd_step(p, 3) == FDTD_OK && w.is(3, 0) && !resident(p, 20), "and after it");
+    for (fdtd_ctx *c : {a, b, h, p}) fdtd_destroy(c);
+}
+
 int main(int, char **argv)
 {
     const std::string s = argv[1];
     if (s == "factors") factors();
     else if (s == "refused") refused();
+    else if (s == "chosen") chosen();
     else expect(false, "a known scenario");
     return bad;
 }
