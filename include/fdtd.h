@@ -166,7 +166,8 @@ int fdtd_set_spectrum(fdtd_ctx *ctx, double f_max, int n_total_steps);
  * context's stream; fields stay on the device between calls.  FP32 boards up
  * to 14 Mi grid points at depth 1 run many steps per cooperative launch
  * ("resident"; also at most 512 sources and probes, nx + ny + nz <= 3000, and
- * no plane written by fdtd_halo_unpack or _copy where n > 1), the others five
+ * since the last reset no plane written by fdtd_halo_unpack or _copy, unless
+ * n = 1 and no copy was between contexts of one GPU), the others five
  * launches per step replayed as CUDA graphs ("tiled"); a board's fields and
  * traces are the same bit for bit either way.  A device that cannot hold a
  * resident launch runs the tiled ones. */

@@ -115,6 +115,7 @@ struct fdtd_ctx {
     size_t rplan_cap = 0;
     bool ports_in_boxes = true;         // every source and probe edge belongs to a box
     bool halo = false;                  // a plane of the state was written from outside
+    bool halo_near = false;             // and exchanged with a context on the same GPU
     bool res_refused = false;           // the device does not take the board's resident launch
     bool tiled_only = false;            // fdtd_set_tiled
     long long *res_buf = nullptr;
@@ -991,12 +992,18 @@ constexpr long long kResPoints = 14LL << 20;
 // extents bound their shared-memory tables; a probe on a high wall plane lies in
 // no box; and a plane written from outside (fdtd_halo_unpack, _copy) may be a
 // wall plane no step writes, whose two sets then differ, so steps that work in
-// place may not follow.
+// place may not follow.  Single steps between exchanges may, but parts of one
+// board on one GPU step faster beside one another, which resident launches
+// cannot (us a step of the split board, resident and tiled: 280x230x100 in two
+// parts 201 and 175, in four 236 and 202; 400x330x100 298 and 264, 354 and 301;
+// 232x192x39 123 and 122, 183 and 148; 132x112x31 101 and 103, 138 and 125).  A
+// part with a GPU of its own keeps them (232x192x39, one step a call, 48 and 71).
 bool resident_board(const fdtd_ctx *c, long long n)
 {
     const Board &h = c->h;
     return c->prec == FDTD_FP32 && !c->tiled_only && !c->res_refused && !h.pair_ok && grid_points(h) <= kResPoints &&
-           6 * h.nodes < (1LL << 31) && c->ports_in_boxes && c->src.size() + c->probe.size() <= 512 && h.nx + h.ny + h.nz <= 3000 && (n <= 1 || !c->halo);
+           6 * h.nodes < (1LL << 31) && c->ports_in_boxes && c->src.size() + c->probe.size() <= 512 && h.nx + h.ny + h.nz <= 3000 &&
+           (!c->halo || (n <= 1 && !c->halo_near));
 }
 
 // Upload a resident plan ([arrival counters | teams | blocks | pieces | ports]).
@@ -1886,7 +1893,7 @@ int fdtd_reset(fdtd_ctx *c)
     CK(cudaMemsetAsync(h.step, 0, sizeof(long long), c->cur));
     CK(cudaMemsetAsync(h.dft_done, 0, 2 * sizeof(long long), c->cur));   // and the status word after it
     c->host_step = 0;
-    c->halo = false;
+    c->halo = c->halo_near = false;
     return FDTD_OK;
 }
 
@@ -2107,6 +2114,7 @@ int fdtd_halo_copy(fdtd_ctx *dst, int dst_plane, fdtd_ctx *src, int src_plane, i
     if (int r = finalize(src)) return r;
     if (src->h.scale != dst->h.scale) return fail(FDTD_EINVAL, "the two contexts use different storage scales");
     dst->halo = true;
+    if (src->device == dst->device) src->halo_near = dst->halo_near = true;
     // the copy runs on the destination's stream once the source's queued work is done
     cudaEvent_t ev = nullptr;
     CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));

@@ -82,7 +82,8 @@ cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 0.f; return cudaSuccess; }
 cudaError_t cudaHostRegister(void *, size_t, unsigned) { return cudaErrorNotSupported; }
 cudaError_t cudaHostUnregister(void *) { return cudaSuccess; }
-cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
+static int device;
+cudaError_t cudaGetDevice(int *d) { *d = device; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char *cudaGetErrorString(cudaError_t) { return "error"; }
@@ -181,7 +182,12 @@ static void factors()
 // Steps of a call, by path.
 struct Took {
     long long tiled, resident;
-    Took() : tiled(-tiled_steps), resident(-resident_steps) {}
+    Took()
+    {
+        drain();
+        tiled = -tiled_steps;
+        resident = -resident_steps;
+    }
     bool is(long long t, long long r)
     {
         drain();
@@ -249,12 +255,36 @@ static void chosen()
     for (fdtd_ctx *c : {a, b, h, p}) fdtd_destroy(c);
 }
 
+// Two parts of a split board take a halo plane from each other after every step.
+static void split()
+{
+    for (int far : {0, 1}) {
+        fdtd_ctx *a = board(30, 24, 20, 0);
+        device = far;
+        fdtd_ctx *b = board(30, 24, 20, 0);
+        device = 0;
+        expect(fdtd_step(a, 1) == FDTD_OK && fdtd_step(b, 1) == FDTD_OK, "a first step");
+        expect(fdtd_halo_copy(a, 24, b, 1, 1, 5) == FDTD_OK && fdtd_halo_copy(b, 0, a, 23, 1, 5) == FDTD_OK, "the exchange");
+        Took t;
+        expect(fdtd_step(a, 1) == FDTD_OK && fdtd_step(b, 1) == FDTD_OK && t.is(far ? 0 : 2, far ? 2 : 0),
+               "parts on one GPU step beside each other, parts on two GPUs by resident launches");
+        Took u;
+        expect(fdtd_step(a, 3) == FDTD_OK && u.is(3, 0), "several steps after an exchange");
+        fdtd_reset(a);
+        Took v;
+        expect(fdtd_step(a, 3) == FDTD_OK && v.is(0, 3), "a board that starts again");
+        fdtd_destroy(a);
+        fdtd_destroy(b);
+    }
+}
+
 int main(int, char **argv)
 {
     const std::string s = argv[1];
     if (s == "factors") factors();
     else if (s == "refused") refused();
     else if (s == "chosen") chosen();
+    else if (s == "split") split();
     else expect(false, "a known scenario");
     return bad;
 }
