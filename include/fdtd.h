@@ -401,9 +401,9 @@ void fdtd_batch_destroy(fdtd_batch *b);
  * columns: 62 or 124, i.e. one or two strips of 62 columns; tile_y rows: 4
  * or 8; a 62x8 tile is worked by four compute warps of 2 rows, a 124x8 tile
  * by two warps of 4 rows per strip; default 62x8), the z-segment length
- * (planes one tile marches before the next work item; default 10, 6 or 4 by
- * the number of work items) and the
- * number of steps per CUDA graph (default 16).  depth is the number of
+ * (planes one tile marches before the next work item; default FDTD_ZSEG_AUTO:
+ * 10, 6 or 4 by the number of work items) and the number of steps per CUDA
+ * graph (default 16).  depth is the number of
  * leapfrog steps one sweep over the interior region advances (time blocking,
  * Model section: the leapfrog's H and E updates of two steps in one pass):
  * 1 (default) or 2.  With depth 2 a single board keeps a third field set
@@ -419,8 +419,8 @@ void fdtd_batch_destroy(fdtd_batch *b);
  * of the two-step pass (default 38, >= 2).  Values <= 0 keep the current
  * setting; unsupported tiles are rejected with FDTD_EINVAL.  Applies to
  * launches queued afterwards.  Tile, segment and graph settings shape the
- * tiled launches; boards that step many times per launch (fdtd_step) do not
- * use them. */
+ * tiled launches; resident boards (fdtd_step) do not use them. */
+#define FDTD_ZSEG_AUTO 0x7fffffff
 typedef struct {
     int tile_x, tile_y, zseg, graph_chunk;
     int depth, pair_zseg;

@@ -19,6 +19,7 @@ FDTD_OK, FDTD_EINVAL, FDTD_ENOMEM, FDTD_ECUDA, FDTD_EUNSTABLE, FDTD_ETIMEOUT, FD
 FDTD_FP32, FDTD_FP16_STORE = 0, 1
 FDTD_WALL_PEC, FDTD_WALL_PMC = 0, 1
 FDTD_X, FDTD_Y, FDTD_Z = 0, 1, 2
+FDTD_ZSEG_AUTO = 0x7fffffff
 FDTD_EX, FDTD_EY, FDTD_EZ, FDTD_HX, FDTD_HY, FDTD_HZ = range(6)
 
 

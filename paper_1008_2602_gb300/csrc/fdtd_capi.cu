@@ -1646,7 +1646,7 @@ int fdtd_set_tuning(fdtd_ctx *c, const fdtd_tuning *t)
     fdtd_tuning n = c->tune;
     if (t->tile_x > 0) n.tile_x = t->tile_x;
     if (t->tile_y > 0) n.tile_y = t->tile_y;
-    if (t->zseg > 0) n.zseg = t->zseg;
+    if (t->zseg > 0) n.zseg = t->zseg == FDTD_ZSEG_AUTO ? 0 : t->zseg;
     if (t->graph_chunk > 0) n.graph_chunk = t->graph_chunk;
     if (t->depth > 0) n.depth = t->depth;
     if (t->pair_zseg > 0) n.pair_zseg = t->pair_zseg;
@@ -2329,7 +2329,7 @@ int fdtd_batch_set_tuning(fdtd_batch *b, const fdtd_tuning *t)
     fdtd_tuning n = b->tune;
     if (t->tile_x > 0) n.tile_x = t->tile_x;
     if (t->tile_y > 0) n.tile_y = t->tile_y;
-    if (t->zseg > 0) n.zseg = t->zseg;
+    if (t->zseg > 0) n.zseg = t->zseg == FDTD_ZSEG_AUTO ? 0 : t->zseg;
     if (t->graph_chunk > 0) n.graph_chunk = t->graph_chunk;
     if (t->depth > 1) return fail(FDTD_EINVAL, "a batch steps one leapfrog step per launch set (depth 1)");
     if (!fused_tile_supported(n.tile_x, n.tile_y))

@@ -108,7 +108,8 @@ class Solver:
         C.fdtd_set_materials(self.ctx, self._mat.ctypes.data)
 
     def set_tuning(self, tile_x=0, tile_y=0, zseg=0, graph_chunk=0, depth=0, pair_zseg=0):
-        """Kernel tuning (0 keeps a setting).  depth=2 advances the interior
+        """Kernel tuning (0 keeps a setting; zseg=capi.FDTD_ZSEG_AUTO: by the
+        number of work items).  depth=2 advances the interior
         region two leapfrog steps per pass (time blocking; bit-identical
         results, one more field set in device memory)."""
         t = C.fdtd_tuning(tile_x, tile_y, zseg, graph_chunk, depth, pair_zseg)

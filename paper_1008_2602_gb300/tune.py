@@ -4,11 +4,13 @@ Times candidate configurations on a throwaway copy of the workload (the
 real solvers are never advanced by tuning) and caches the fastest per
 precision and grid class in a JSON file.  The search covers:
 * the fused-tile shapes (tile_x x tile_y columns);
-* the z-segment lengths;
+* the z-segment lengths, the library's own choice among them;
 * the CUDA-graph chunk sizes;
 * for a single board, the blocking depth: one leapfrog step per interior
   sweep, or two (the two-step pass, with its z-segment length).  A batch
   advances one step per sweep.
+The first three shape the tiled launches.  Where every board goes by resident
+launches, which use none of them, they keep their defaults.
 """
 from __future__ import annotations
 
@@ -18,8 +20,10 @@ import os
 import time
 from typing import Dict, Iterable, List, Optional, Sequence
 
+ZSEG_AUTO = 0x7fffffff   # FDTD_ZSEG_AUTO
+DEFAULT = dict(tile_x=62, tile_y=8, zseg=ZSEG_AUTO, graph_chunk=16)
 SHAPES = [(62, 4), (124, 4), (62, 8), (124, 8)]
-ZSEGS = [8, 10, 16, 25]
+ZSEGS = [ZSEG_AUTO, 8, 10, 16, 25]
 CHUNKS = [16, 64]
 PAIR_ZSEGS = [19, 38]   # two-step pass segments tried for a single board
 
@@ -53,6 +57,21 @@ def _save(d: Dict[str, dict]) -> None:
         os.replace(tmp, CACHE)
     except OSError:
         pass
+
+
+def _resident(probs, precision: str) -> bool:
+    """Whether every board goes by resident launches."""
+    from . import solver
+    if precision != "fp32":
+        return False
+    for p in probs:
+        s = solver.Solver(p, precision=precision, spectrum=False)
+        try:
+            if not s.resident():
+                return False
+        finally:
+            s.close()
+    return True
 
 
 def _time_batch(probs, precision: str, cfg: dict, steps: int) -> float:
@@ -95,13 +114,14 @@ def tune(probs: Sequence, precision: str = "fp32", steps: int = 32, shapes=SHAPE
     """Best tuning dict (tile_x, tile_y, zseg, graph_chunk, depth, and for
     depth 2 pair_zseg) for stepping ``probs`` together (one board = a single
     solve, which also tries depth 2)."""
-    key = grid_class(probs, precision)
+    resident = _resident(probs, precision)
+    key = grid_class(probs, precision) + (":resident" if resident else ":tiled")
     cache = _load() if use_cache else {}
     if use_cache and key in cache:
         return dict(cache[key]["tuning"])
-    best, best_t = None, float("inf")
+    best, best_t = dict(DEFAULT), float("inf")
     trials = []
-    for (tx, ty) in shapes:
+    for (tx, ty) in () if resident else shapes:
         for zs in zsegs:
             cfg = dict(tile_x=tx, tile_y=ty, zseg=zs, graph_chunk=chunks[0])
             t = _time_batch(probs, precision, cfg, steps)
@@ -110,7 +130,7 @@ def tune(probs: Sequence, precision: str = "fp32", steps: int = 32, shapes=SHAPE
                 log(f"tune {key} {cfg} {t * 1e3:.2f} ms")
             if t < best_t:
                 best, best_t = cfg, t
-    for ch in chunks[1:]:
+    for ch in () if resident else chunks[1:]:
         cfg = dict(best, graph_chunk=ch)
         t = _time_batch(probs, precision, cfg, steps)
         if log:
@@ -132,7 +152,7 @@ def tune(probs: Sequence, precision: str = "fp32", steps: int = 32, shapes=SHAPE
                 best, best_t = cfg, t
     if use_cache:
         cache = _load()
-        cache[key] = {"tuning": best, "ms_per_step": best_t * 1e3 / steps,
+        cache[key] = {"tuning": best, "ms_per_step": best_t * 1e3 / steps if best_t < float("inf") else None,
                       "trials": [{"ms": t * 1e3, **c} for t, c in trials]}
         _save(cache)
     return dict(best)

@@ -278,6 +278,35 @@ static void split()
     }
 }
 
+static void segments()
+{
+    fdtd_ctx *a = board(200, 190, 60, 6, FDTD_FP16_STORE);
+    fdtd_batch *g = nullptr;
+    expect(fdtd_batch_create(nullptr, &g) == FDTD_OK, "the batch is created");
+    fdtd_step(a, 1);
+    const int rule = a->plan.zseg;
+    fdtd_tuning t{}, back{};
+    t.zseg = 25;
+    back.zseg = FDTD_ZSEG_AUTO;
+    fdtd_set_tuning(a, &t);
+    fdtd_set_tuning(a, &(t = fdtd_tuning{}));
+    fdtd_step(a, 1);
+    expect(rule != 25 && a->plan.zseg == 25, "a length that was set, and kept by 0");
+    fdtd_set_tuning(a, &back);
+    fdtd_step(a, 1);
+    expect(a->plan.zseg == rule, "the rule's length again");
+    fdtd_batch_add(g, a, 9);
+    t.zseg = 25;
+    fdtd_batch_set_tuning(g, &t);
+    fdtd_batch_step(g, 1, nullptr);
+    const int set = g->plan.zseg;
+    fdtd_batch_set_tuning(g, &back);
+    fdtd_batch_step(g, 1, nullptr);
+    expect(set == 25 && g->plan.zseg == rule, "and in a batch");
+    fdtd_batch_destroy(g);
+    fdtd_destroy(a);
+}
+
 int main(int, char **argv)
 {
     const std::string s = argv[1];
@@ -285,6 +314,7 @@ int main(int, char **argv)
     else if (s == "refused") refused();
     else if (s == "chosen") chosen();
     else if (s == "split") split();
+    else if (s == "segments") segments();
     else expect(false, "a known scenario");
     return bad;
 }
