@@ -241,11 +241,12 @@ int fdtd_load(fdtd_ctx *ctx, const void *buf, size_t size);
 
 /* Failure-detection self-test of the bounded device waits.  Launches one
  * block on `stream` (NULL: the default stream) that waits on an mbarrier no
- * one arrives at, with the fused kernel's bounded poll (max_polls polls,
- * 0 = the fused kernel's limit).  The wait must give up and report it:
- * returns FDTD_ETIMEOUT (the expected result), FDTD_OK if the wait did not
+ * one arrives at, with the fused kernel's bounded poll, and one that waits at
+ * the barrier of a resident launch for a block that never comes (max_polls
+ * polls each, 0 = the kernels' own limits).  Both must give up and report it:
+ * returns FDTD_ETIMEOUT (the expected result), FDTD_OK if one of them did not
  * time out, or FDTD_ECUDA.  Nothing faults, traps or hangs, and the device
- * stays usable.  Allocates one int and frees it.  Synchronises. */
+ * stays usable.  Allocates two ints and frees them.  Synchronises. */
 int fdtd_selftest_wait_timeout(void *stream, unsigned max_polls);
 
 /* Replace the material ids of the board (same eps_r table, PEC and ports),

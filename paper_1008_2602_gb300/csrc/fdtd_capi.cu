@@ -1275,10 +1275,12 @@ int check_status(fdtd_ctx *c)
 {
     int st = 0;
     CK(cudaMemcpy(&st, c->h.status, sizeof(int), cudaMemcpyDeviceToHost));
-    if (st & 4) return fail(FDTD_EINVAL, "a fused-kernel launch did not match the board's tensor maps; its items were "
+    if (st & kStatusMaps) return fail(FDTD_EINVAL, "a fused-kernel launch did not match the board's tensor maps; its items were "
                                          "skipped (results of this run are invalid)");
-    if (st & 2) return fail(FDTD_ETIMEOUT, "a fused-kernel TMA wait gave up (results of this run are invalid)");
-    if (st & 1) return fail(FDTD_EUNSTABLE, "non-finite probe sample (unstable run: check the Courant number)");
+    if (st & kStatusTmaWait) return fail(FDTD_ETIMEOUT, "a fused-kernel TMA wait gave up (results of this run are invalid)");
+    if (st & kStatusBarrier)
+        return fail(FDTD_ETIMEOUT, "the barrier of a resident launch gave up (results of this run are invalid)");
+    if (st & kStatusNonFinite) return fail(FDTD_EUNSTABLE, "non-finite probe sample (unstable run: check the Courant number)");
     return FDTD_OK;
 }
 
@@ -2016,17 +2018,19 @@ int fdtd_load(fdtd_ctx *c, const void *buf, size_t size)
 int fdtd_selftest_wait_timeout(void *stream, unsigned max_polls)
 {
     cudaStream_t st = (cudaStream_t)stream;
-    int *d = nullptr;
-    cudaError_t e = cudaMalloc(&d, sizeof(int));
+    int *d = nullptr;   // status, and the barrier's counter
+    cudaError_t e = cudaMalloc(&d, 2 * sizeof(int));
     if (e != cudaSuccess) { cudaGetLastError(); return fail(FDTD_ECUDA, "selftest allocation failed"); }
     int status = 0;
-    e = cudaMemsetAsync(d, 0, sizeof(int), st);
+    e = cudaMemsetAsync(d, 0, 2 * sizeof(int), st);
     if (e == cudaSuccess) e = launch_wait_selftest(d, max_polls ? max_polls : (1u << 21), st);
+    if (e == cudaSuccess) e = launch_barrier_selftest(d, (unsigned *)d + 1, max_polls ? max_polls : kBarrierPolls, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&status, d, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(d);
     if (e != cudaSuccess) return cuda_fail(e, "selftest");
-    if (status & 2) return fail(FDTD_ETIMEOUT, "bounded device wait gave up (self-test: expected)");
+    if ((status & kStatusTmaWait) && (status & kStatusBarrier))
+        return fail(FDTD_ETIMEOUT, "bounded device waits gave up, mbarrier and resident barrier (self-test: expected)");
     return FDTD_OK;
 }
 

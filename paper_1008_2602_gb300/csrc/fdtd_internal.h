@@ -71,6 +71,14 @@ struct Coef {
     float b1, g, ap, am;
 };
 
+// What a kernel reports in a board's status word.
+enum : int {
+    kStatusNonFinite = 1,         // a probe sample
+    kStatusTmaWait = 2,           // a fused kernel's bounded wait gave up
+    kStatusMaps = 4,              // tile and tensor maps differ (item skipped)
+    kStatusBarrier = 8,           // a resident launch's barrier gave up
+};
+
 struct Slab {
     int i0, i1, j0, j1, k0, k1;   // node box, half-open
     int ni, nj;                   // i1 - i0, j1 - j0
@@ -154,8 +162,7 @@ struct Board {
     int n_bins;
     double *dft;                  // [n_probe][n_bins][2]
     long long *dft_done;          // samples already folded into dft
-    int *status;                  // bit 0: non-finite probe sample seen; bit 1: a bounded wait
-                                  // gave up; bit 2: tile / tensor-map mismatch (item skipped)
+    int *status;                  // kStatus... bits
     int pad1;
 };
 
@@ -298,6 +305,7 @@ __host__ __device__ inline int res_quot(int t, unsigned m, int s)
 // against 5.9 at 1151 units with eight warps.
 constexpr int kPinWarps = 6;
 constexpr int kResSmem = 200 << 10;   // shared memory a resident launch may ask for
+constexpr unsigned kBarrierPolls = 1u << 22;   // after which a block gives up its team's barrier
 
 // TMA descriptor slots of a board (3D maps: x, y, plane).
 __host__ __device__ constexpr int tm_e(int set, int c) { return set * 3 + c; }               // E   box_e  x (TY+2)
@@ -375,5 +383,6 @@ bool fused_tile_supported(int tile_x, int tile_y);
 int set_error(int code, const char *msg);
 cudaError_t fused_set_smem_limits();
 cudaError_t launch_wait_selftest(int *status, unsigned max_polls, cudaStream_t st);
+cudaError_t launch_barrier_selftest(int *status, unsigned *count, unsigned max_polls, cudaStream_t st);
 
 }  // namespace fdtd

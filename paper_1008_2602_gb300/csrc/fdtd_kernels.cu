@@ -95,7 +95,7 @@ __device__ __forceinline__ void mbar_wait(uint64_t *b, uint32_t parity, int *sta
     if (*(volatile int *)abort_flag) return;
     for (uint32_t it = 0; it < max_polls; ++it)
         if (mbar_try(b, parity)) return;
-    atomicOr(status, 2);
+    atomicOr(status, kStatusTmaWait);
     *(volatile int *)abort_flag = 1;
 }
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int x, int y, int z, uint64_t *bar)
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(32 * W * R + 32, (FusedLayout<T, TY, W, NS, ZP
             if (item >= n_items) break;
             const Tile t = decode_tile<TY, W, ZP>(plan, item);
             const Board *B = t.B;
-            if (!t.ok && (B->tm_tx != kWarpCols * W || B->tm_ty != TY)) atomicOr(B->status, 4);
+            if (!t.ok && (B->tm_tx != kWarpCols * W || B->tm_ty != TY)) atomicOr(B->status, kStatusMaps);
             const CUtensorMap *tm = B->tm;
             const int id16 = B->id16;
             const int xe0 = (t.i0 - 1) & ~7;
@@ -1590,7 +1590,7 @@ __global__ void k_post(Plan plan)
         const Probe Q = p == tid ? q0 : probe[p];
         const float v = Io<T>::ldw((const T *)field(out, Q.comp) + Q.node) * scale;
         if (rec) B->trace[(long long)p * n_total + step] = v;
-        if (!isfinite(v)) atomicOr(B->status, 1);
+        if (!isfinite(v)) atomicOr(B->status, kStatusNonFinite);
     }
     __syncthreads();
     if (tid == 0) *((volatile long long *)B->step) = step + 1;
@@ -1751,7 +1751,7 @@ __global__ void k_energy_final(const double *partials, int n, double *out2)
 // ------------------------------------------------------------------ failure detection
 // Self-test of the bounded wait: an mbarrier that nothing arrives on, waited
 // on with the same bounded poll as the fused kernel, must give up, set
-// status bit 1 (value 2) and return, leaving the context usable.
+// kStatusTmaWait and return, leaving the context usable.
 __global__ void k_wait_selftest(int *status, uint32_t max_polls)
 {
     __shared__ uint64_t bar;

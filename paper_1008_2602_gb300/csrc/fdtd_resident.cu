@@ -299,7 +299,7 @@ __device__ __forceinline__ void work_ports(int unit, int s, F4 &nx, F4 &ny, F4 &
                 const float f = now * B.scale;
                 const long long n = B.step0 + s;
                 if (n < (long long)B.n_total) B.trace[(long long)p.index * B.n_total + n] = f;
-                if (!isfinite(f)) atomicOr(B.status, 1);
+                if (!isfinite(f)) atomicOr(B.status, kStatusNonFinite);
             } else {
                 const Drive &d = reinterpret_cast<const Drive *>(smem + B.drive)[v];
                 const float f = d.s.kind == kSrcCurrent
@@ -511,15 +511,15 @@ __device__ __forceinline__ void team_arrive(unsigned *bar)
     __syncthreads();
     if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
 }
-__device__ __forceinline__ bool team_wait(unsigned *bar, unsigned target, int *status, int *gave_up)
+__device__ __forceinline__ bool team_wait(unsigned *bar, unsigned target, int *status, int *gave_up,
+                                          unsigned max_polls = kBarrierPolls)
 {
     if (threadIdx.x == 0) {
-        unsigned v = 0;
-        int it = 0;
+        unsigned v = 0, it = 0;
         do asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-        while (v < target && ++it < (1 << 22));
+        while (v < target && ++it < max_polls);
         if (v < target) {
-            atomicOr(status, 2);
+            atomicOr(status, kStatusBarrier);
             *gave_up = 1;
         }
     }
@@ -820,7 +820,22 @@ __global__ void __launch_bounds__(kPinThreads, 1) k_pinned(ResPlan plan, int nst
     if (tid == 0 && nact > 0 && blk.first) *((volatile long long *)board->step) = B.step0 + nact;
 }
 
+// Self-test of that bounded wait: a team of two of which one block arrives.
+__global__ void k_barrier_selftest(int *status, unsigned *count, unsigned max_polls)
+{
+    __shared__ int gave_up;
+    if (threadIdx.x == 0) gave_up = 0;
+    team_arrive(count);
+    team_wait(count, 2, status, &gave_up, max_polls);
+}
+
 }  // namespace
+
+cudaError_t launch_barrier_selftest(int *status, unsigned *count, unsigned max_polls, cudaStream_t st)
+{
+    k_barrier_selftest<<<1, 32, 0, st>>>(status, count, max_polls);
+    return cudaGetLastError();
+}
 
 size_t resident_smem(const ResPlan &p) { return (size_t)layout_of(p).bytes; }
 

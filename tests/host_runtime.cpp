@@ -98,6 +98,15 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **p, unsigned, u
 }
 }
 
+static int bad = 0;
+static void expect(bool ok, const char *what)
+{
+    if (!ok) {
+        std::printf("not so: %s\n", what);
+        ++bad;
+    }
+}
+
 // The kernels: which path advanced a board by how many steps.
 static long long tiled_steps, resident_steps;
 static bool refuse_cooperative;   // the device takes no resident launch
@@ -143,16 +152,13 @@ cudaError_t launch_energy(const Board *, const Board &, double *, int, double *,
 int energy_partials(const Board &) { return 1; }
 cudaError_t fused_set_smem_limits() { return cudaSuccess; }
 bool fused_tile_supported(int tx, int ty) { return (tx == 62 || tx == 124) && (ty == 4 || ty == 8); }
-cudaError_t launch_wait_selftest(int *status, unsigned, cudaStream_t) { later([=] { *status = 2; }); return cudaSuccess; }
-}
-
-static int bad = 0;
-static void expect(bool ok, const char *what)
+static int mbarrier_gives_up = kStatusTmaWait, team_gives_up = kStatusBarrier;
+cudaError_t launch_wait_selftest(int *s, unsigned, cudaStream_t) { later([=] { *s |= mbarrier_gives_up; }); return cudaSuccess; }
+cudaError_t launch_barrier_selftest(int *s, unsigned *n, unsigned, cudaStream_t)
 {
-    if (!ok) {
-        std::printf("not so: %s\n", what);
-        ++bad;
-    }
+    later([=] { expect(*n == 0, "the counter starts at zero"); *s |= team_gives_up; });
+    return cudaSuccess;
+}
 }
 
 static fdtd_ctx *board(int nx, int ny, int nz, int depth, int prec = FDTD_FP32)
@@ -307,6 +313,24 @@ static void segments()
     fdtd_destroy(a);
 }
 
+// What the host makes of a wait that gave up.
+static void waits()
+{
+    fdtd_ctx *c = board(30, 24, 20, 4);
+    expect(fdtd_step(c, 1) == FDTD_OK && fdtd_sync(c) == FDTD_OK, "no wait gave up");
+    *c->h.status = kStatusTmaWait;
+    expect(fdtd_sync(c) == FDTD_ETIMEOUT && std::strstr(fdtd_last_error(), "TMA wait"), "a TMA wait");
+    *c->h.status = kStatusBarrier;
+    expect(fdtd_sync(c) == FDTD_ETIMEOUT && std::strstr(fdtd_last_error(), "barrier of a resident launch"), "a barrier");
+    fdtd_destroy(c);
+    expect(fdtd_selftest_wait_timeout(nullptr, 10) == FDTD_ETIMEOUT, "both kinds gave up");
+    team_gives_up = 0;
+    expect(fdtd_selftest_wait_timeout(nullptr, 10) == FDTD_OK, "the barrier did not");
+    team_gives_up = kStatusBarrier;
+    mbarrier_gives_up = 0;
+    expect(fdtd_selftest_wait_timeout(nullptr, 10) == FDTD_OK, "the mbarrier did not");
+}
+
 int main(int, char **argv)
 {
     const std::string s = argv[1];
@@ -315,6 +339,7 @@ int main(int, char **argv)
     else if (s == "chosen") chosen();
     else if (s == "split") split();
     else if (s == "segments") segments();
+    else if (s == "waits") waits();
     else expect(false, "a known scenario");
     return bad;
 }
