@@ -1907,7 +1907,7 @@ struct CkptHeader {
     int32_t version;
     int32_t nx, ny, nz, pitch, prec, n_probe, n_src, n_total, n_bins, n_slab;
     float scale;
-    int32_t halo;   // a plane of the state was written from outside
+    int32_t pad;
     int64_t nodes, step, dft_done;
     double dt;
 };
@@ -1944,10 +1944,27 @@ CkptHeader ckpt_header(const fdtd_ctx *c)
     H.n_probe = (int)c->probe.size(); H.n_src = (int)c->src.size();
     H.n_total = h.n_total; H.n_bins = h.n_bins; H.n_slab = h.n_slab;
     H.scale = h.scale;
-    H.halo = c->halo ? 1 : 0;
     H.nodes = h.nodes;
     H.dt = c->dt;
     return H;
+}
+
+// Whether a node no step writes holds something in a checkpoint's field sets:
+// the planes behind high PEC walls, which are zero unless written from outside.
+bool wall_planes_hold(const fdtd_ctx *c, const unsigned char *sets)
+{
+    const Board &h = c->h;
+    const size_t es = elem_size(c->prec);
+    const bool ex = h.wall[1] == FDTD_WALL_PEC, ey = h.wall[3] == FDTD_WALL_PEC, ez = h.wall[5] == FDTD_WALL_PEC;
+    auto any = [](const unsigned char *p, size_t n) { return std::any_of(p, p + n, [](unsigned char b) { return b != 0; }); };
+    for (int f = 0; f < 12; ++f)
+        for (int k = 0; k <= h.nz; ++k)
+            for (int j = 0; j <= h.ny; ++j) {
+                const unsigned char *row = sets + (f * (size_t)h.nodes + (size_t)k * h.plane + (size_t)j * h.pitch) * es;
+                const bool whole = (ez && k == h.nz) || (ey && j == h.ny);
+                if (whole ? any(row, (h.nx + 1) * es) : ex && any(row + h.nx * es, es)) return true;
+            }
+    return false;
 }
 
 }  // namespace
@@ -2011,7 +2028,7 @@ int fdtd_load(fdtd_ctx *c, const void *buf, size_t size)
     CK(cudaMemsetAsync(c->h.status, 0, sizeof(int), c->cur));
     CK(cudaStreamSynchronize(c->cur));
     c->host_step = H.step;
-    c->halo = H.halo != 0;
+    c->halo = wall_planes_hold(c, static_cast<const unsigned char *>(buf) + sizeof(CkptHeader));
     return FDTD_OK;
 }
 

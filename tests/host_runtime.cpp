@@ -331,6 +331,35 @@ static void waits()
     expect(fdtd_selftest_wait_timeout(nullptr, 10) == FDTD_OK, "the mbarrier did not");
 }
 
+// A checkpoint's data say whether a plane was written from outside, also those
+// of before resident launches, whose header has 0 in its last word.
+static void checkpoint()
+{
+    fdtd_ctx *a = board(30, 24, 20, 4), *b = board(30, 24, 20, 4);
+    fdtd_step(a, 4);
+    size_t n = 0;
+    fdtd_save(a, nullptr, 0, &n);
+    std::vector<unsigned char> clean(n), wrote(n);
+    expect(fdtd_save(a, clean.data(), n, &n) == FDTD_OK, "a state of steps alone");
+    std::vector<float> plane(2 * 31 * 25, 1.f);
+    const int high[3] = {30, 24, 20};
+    for (int axis = -1; axis < 3; ++axis) {
+        if (axis >= 0) {
+            fdtd_load(a, clean.data(), n);
+            expect(fdtd_halo_unpack(a, axis, high[axis], 5, plane.data()) == FDTD_OK, "a plane from outside");
+            if (axis == 1) fdtd_step(a, 1);   // it then lies in the set of the step before
+        }
+        expect(fdtd_save(a, wrote.data(), n, &n) == FDTD_OK, "the state is saved");
+        std::memset(wrote.data() + offsetof(CkptHeader, scale) + 4, 0, 4);
+        expect(fdtd_load(b, wrote.data(), n) == FDTD_OK, "the checkpoint is taken");
+        const int tiled = axis < 0 ? 0 : 3;
+        Took t;
+        expect(fdtd_step(b, 3) == FDTD_OK && t.is(tiled, 3 - tiled), "the launches that continue it");
+    }
+    fdtd_destroy(a);
+    fdtd_destroy(b);
+}
+
 int main(int, char **argv)
 {
     const std::string s = argv[1];
@@ -340,6 +369,7 @@ int main(int, char **argv)
     else if (s == "split") split();
     else if (s == "segments") segments();
     else if (s == "waits") waits();
+    else if (s == "checkpoint") checkpoint();
     else expect(false, "a known scenario");
     return bad;
 }
