@@ -1120,6 +1120,13 @@ struct NvtxRange {
     ~NvtxRange() { nvtxRangePop(); }
 };
 
+// Waits for a stream on the way out of a block, whichever way that is: declared
+// after host memory that copies queued on the stream read.
+struct StreamWait {
+    cudaStream_t st;
+    ~StreamWait() { cudaStreamSynchronize(st); }
+};
+
 // The side stream of a context or batch, made on its first tiled step.
 int open_side(SideStream &s)
 {
@@ -1712,6 +1719,7 @@ static int prepare_single(fdtd_ctx *c, bool tiled)
     if (c->plan_dirty) c->plan_ok = c->rplan_ok = c->plan_dirty = false;
     if (tiled ? c->plan_ok : c->rplan_ok) return FDTD_OK;
     std::vector<long long> host, rhost;
+    const StreamWait copies{c->cur};
     const std::vector<fdtd_ctx *> one{c};
     if (tiled) {
         if (int r = build_plan(one, c->tune, true, c->plan_buf, c->plan_cap, c->plan, c->cur, host)) return r;
@@ -2409,6 +2417,7 @@ static int prepare_batch(fdtd_batch *b)
         if (r) work += (double)c->h.nodes;
     }
     std::vector<long long> host, rhost, rhost2;
+    const StreamWait copies{b->stream};
     for (fdtd_ctx *m : tiled)
         if (int r = encode_maps(m, b->tune.tile_x, b->tune.tile_y)) return r;
     b->plan.nb = 0;

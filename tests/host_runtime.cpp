@@ -26,7 +26,14 @@ static void drain()
 }
 
 extern "C" {
-cudaError_t cudaMalloc(void **p, size_t n) { *p = std::aligned_alloc(256, (n + 255) / 256 * 256); return cudaSuccess; }
+static int mallocs_left = -1;   // then none succeeds
+cudaError_t cudaMalloc(void **p, size_t n)
+{
+    if (!mallocs_left) return cudaErrorMemoryAllocation;
+    --mallocs_left;
+    *p = std::aligned_alloc(256, (n + 255) / 256 * 256);
+    return cudaSuccess;
+}
 cudaError_t cudaFree(void *) { drain(); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t)
 {
@@ -360,6 +367,30 @@ static void checkpoint()
     fdtd_destroy(b);
 }
 
+// A plan that runs out of memory half-way leaves no copy queued from freed memory.
+static void memory()
+{
+    for (int batched : {0, 1}) {
+        fdtd_ctx *c = board(30, 24, 20, 4);
+        fdtd_batch *g = nullptr;
+        fdtd_step(c, 0);
+        c->plan_dirty = true;
+        long long **const boards = batched ? nullptr : &c->rplan_buf;
+        if (batched) expect(fdtd_batch_create(nullptr, &g) == FDTD_OK && fdtd_batch_add(g, c, 9) == FDTD_OK, "a batch of one");
+        else for (long long **b : {&c->rplan_buf, &c->res_buf}) { cudaFree(*b); *b = nullptr; c->rplan_cap = c->res_cap = 0; }
+        mallocs_left = 1;
+        expect((batched ? fdtd_batch_step(g, 4, nullptr) : fdtd_step(c, 4)) == FDTD_ENOMEM, "the second buffer is refused");
+        mallocs_left = -1;
+        drain();
+        const long long *const buf = boards ? *boards : g->rplan_buf;
+        expect(buf && *buf == (long long)(uintptr_t)c->d, "the first holds what was copied to it");
+        Took t;
+        expect((batched ? fdtd_batch_step(g, 4, nullptr) : fdtd_step(c, 4)) == FDTD_OK && t.is(0, 4), "the next call steps");
+        if (g) fdtd_batch_destroy(g);
+        fdtd_destroy(c);
+    }
+}
+
 int main(int, char **argv)
 {
     const std::string s = argv[1];
@@ -370,6 +401,7 @@ int main(int, char **argv)
     else if (s == "segments") segments();
     else if (s == "waits") waits();
     else if (s == "checkpoint") checkpoint();
+    else if (s == "memory") memory();
     else expect(false, "a known scenario");
     return bad;
 }

@@ -23,7 +23,7 @@ def program(tmp_path_factory):
     return str(exe)
 
 
-@pytest.mark.parametrize("scenario", ["factors", "refused", "chosen", "split", "segments", "waits", "checkpoint"])
+@pytest.mark.parametrize("scenario", ["factors", "refused", "chosen", "split", "segments", "waits", "checkpoint", "memory"])
 def test_host_code(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
