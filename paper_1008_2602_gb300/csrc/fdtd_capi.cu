@@ -875,7 +875,7 @@ long long dft_items(const Board &h)
     return (long long)h.n_bins * ((h.n_probe + kDftProbeGroup - 1) / kDftProbeGroup);
 }
 
-// Lay out plan arrays [boards | int_prefix | zp_prefix | slab block counts | dft_prefix | work | slab blocks] in buf.
+// Lay out plan arrays [boards | int_prefix | zp_prefix | dft_prefix | work | slab blocks] in buf.
 int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, bool tiled, long long *&buf, size_t &cap,
                Plan &plan, cudaStream_t st, std::vector<long long> &host)
 {
@@ -894,11 +894,11 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, b
     const bool band = tiled && nb == 1 && boards[0]->h.pair_ok && boards[0]->h.n_band > 0;
     if (band) n_slab_blk += boards[0]->h.band_blocks;
     static_assert(sizeof(SlabBlock) == 4 * sizeof(long long), "slab block descriptor layout");
-    const size_t head = ((size_t)nb + 4 * ((size_t)nb + 1) + 2 + 1) & ~(size_t)1;   // + four work counters, 16-byte aligned
+    const size_t head = ((size_t)nb + 3 * ((size_t)nb + 1) + 2 + 1) & ~(size_t)1;   // + four work counters, 16-byte aligned
     const size_t words = head + 4 * (size_t)n_slab_blk;
     host.assign(words, 0);
     long long *ptrs = host.data();
-    long long *ip = ptrs + nb, *zp = ip + nb + 1, *sp = zp + nb + 1, *dp = sp + nb + 1;
+    long long *ip = ptrs + nb, *zp = ip + nb + 1, *dp = zp + nb + 1;
     SlabBlock *sb = reinterpret_cast<SlabBlock *>(ptrs + head);
     // a single board's band blocks come first in the table, E-only boxes then
     // H+E boxes, so that a second-step launch starts them before the slab
@@ -906,6 +906,7 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, b
     // their latency to the launch)
     const long long nbb = band ? boards[0]->h.band_blocks : 0;
     const long long nbh = band ? boards[0]->h.band_h_blocks : 0;
+    long long slab0 = nbb;   // table position of a board's first slab block
     for (int b = 0; b < nb; ++b) {
         const Board &h = boards[b]->h;
         ptrs[b] = (long long)(uintptr_t)boards[b]->d;
@@ -913,14 +914,13 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, b
         if (!tiled) continue;   // a plan for resident launches: boards and DFT items only
         ip[b + 1] = ip[b] + fused_items(h, t, false);
         zp[b + 1] = zp[b] + fused_items(h, t, true);
-        sp[b + 1] = sp[b] + h.slab_blocks;
         const int ns = h.n_slab + (band ? h.n_band : 0);
         for (int s = 0; s < ns; ++s) {
             const int end = s + 1 < ns ? (int)h.slab[s + 1].block0 : h.slab_blocks + (band ? h.band_blocks : 0);
             for (int k = (int)h.slab[s].block0; k < end; ++k) {
                 // table position: slab blocks after the band; band H+E blocks
                 // (numbered first) after the E-only ones
-                long long at = sp[b] + k + nbb;
+                long long at = slab0 + k;
                 if (band && k >= h.slab_blocks) at = k - h.slab_blocks < nbh ? (nbb - nbh) + (k - h.slab_blocks)
                                                                               : k - h.slab_blocks - nbh;
                 SlabBlock &e = sb[at];
@@ -931,6 +931,7 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, b
                 e.t0 = (k - (int)h.slab[s].block0) * kSlabThreads;
             }
         }
+        slab0 += h.slab_blocks;
     }
     if (words > cap) {
         if (buf) cudaFree(buf);
@@ -951,12 +952,12 @@ int build_plan(const std::vector<fdtd_ctx *> &boards, const fdtd_tuning &tune, b
     plan.boards = (Board *const *)buf;
     plan.int_prefix = buf + nb;
     plan.zp_prefix = buf + nb + (nb + 1);
-    plan.dft_prefix = buf + nb + 3 * (nb + 1);
+    plan.dft_prefix = buf + nb + 2 * (nb + 1);
     plan.n_int = ip[nb];
     plan.n_zp = zp[nb];
-    plan.n_slab = sp[nb];
+    plan.n_slab = slab0 - nbb;
     plan.n_dft = dp[nb];
-    plan.work = (int *)(buf + nb + 4 * (nb + 1));
+    plan.work = (int *)(buf + nb + 3 * (nb + 1));
     plan.slab_blk = reinterpret_cast<const SlabBlock *>(buf + head) + nbb;
     plan.pair_zseg = t.pair_zseg;
     plan.n_pair = band ? pair_items(boards[0]->h, t) : 0;
@@ -1031,7 +1032,7 @@ int upload_resident(const ResHost &R, Board *const *dev_boards, long long *&buf,
         cap = words;
     }
     CK(cudaMemcpyAsync(buf, host.data(), words * sizeof(long long), cudaMemcpyHostToDevice, st));
-    plan.n_teams = plan.all_teams = (int)R.teams.size();
+    plan.all_teams = (int)R.teams.size();
     plan.n_blocks = (int)R.blocks.size();
     plan.boards = dev_boards;
     plan.arrive = (unsigned *)(buf + oa);
@@ -1092,22 +1093,19 @@ int build_resident_batch(const std::vector<fdtd_ctx *> &boards, Board *const *de
         for (int m : group[g]) work.push_back(res_work(boards[m]->h));
         const std::vector<int> n = res_share(work, sms);
         plans[g].n_blocks = -(int)R.blocks.size();
-        plans[g].n_teams = -(int)R.teams.size();
         R.max_units = 0;
         for (size_t t = 0; t < n.size(); ++t) res_team(boards[group[g][t]]->h, res_ports(boards[group[g][t]]), group[g][t], n[t], R);
         plans[g].n_blocks += (int)R.blocks.size();
-        plans[g].n_teams += (int)R.teams.size();
         plans[g].max_units = R.max_units;
     }
     ResPlan all{};
     if (int r = upload_resident(R, dev_boards, buf, cap, all, st, host)) return r;
     int blk = 0;
     for (ResPlan &p : plans) {
-        const int nb = p.n_blocks, nt = p.n_teams, nu = p.max_units;
+        const int nb = p.n_blocks, nu = p.max_units;
         p = all;   // (a block names its team by its place among all teams, and so its counter)
         p.n_blocks = nb;
         p.blocks = all.blocks + blk;
-        p.n_teams = nt;
         p.max_units = nu;
         blk += nb;
     }

@@ -87,9 +87,9 @@ __device__ __forceinline__ Coef ldcoef(const Coef *p)
     return Coef{v.x, v.y, v.z, v.w};
 }
 
-// Factor of the image of tangential H~ across an outer wall for a neighbour
-// `outside` the grid (PMC: odd mirror, -1; PEC: 0).
-__device__ __forceinline__ float hsign(bool outside, int wall) { return outside ? (wall == 1 ? -1.0f : 0.0f) : 1.0f; }
+// Factor of the image of tangential H~ across an outer wall (PMC: odd mirror,
+// -1; PEC: 0).
+__device__ __forceinline__ float hsign(int wall) { return wall == 1 ? -1.0f : 0.0f; }
 
 // ------------------------------------------------------------------ quads
 struct F4 {       // four neighbouring nodes of a row
@@ -187,8 +187,8 @@ __device__ __forceinline__ unsigned below(int i, int n) { return 15u >> min(max(
 // node's own value, a high wall its - neighbour's.
 __device__ __forceinline__ void image(bool lo, bool hi, int wlo, int whi, float &p, float &m)
 {
-    if (hi) p = hsign(true, whi) * m;
-    if (lo) m = hsign(true, wlo) * p;
+    if (hi) p = hsign(whi) * m;
+    if (lo) m = hsign(wlo) * p;
 }
 __device__ __forceinline__ void image4(bool lo, bool hi, int wlo, int whi, F4 &p, F4 &m)
 {

@@ -277,7 +277,7 @@ struct ResBlock {
     int piece0, n_piece, port0, n_port;
 };
 struct ResPlan {
-    int n_teams, n_blocks, all_teams;
+    int n_blocks, all_teams;      // of the launch; teams of all launches that share `arrive`
     Board *const *boards;
     const ResTeam *teams;
     const ResBlock *blocks;
@@ -289,7 +289,8 @@ struct ResPlan {
 };
 // Length of a UPML factor array in a block's shared memory (n + 1 positions, whole quads).
 __host__ __device__ inline int res_fac_len(int n) { return (n + 1 + 3) & ~3; }
-// Quotients by a fixed divisor d >= 1 for 0 <= t < 2^31: q = (umulhi(t, m) + t) >> s.
+// Quotients by a fixed divisor d >= 1 for 0 <= t < 2^31: q = (umulhi(t, m) + t) >> s
+// (division by an invariant with a rounded-up reciprocal, Granlund and Montgomery 1994).
 __host__ __device__ inline void res_recip(int d, unsigned &m, int &s)
 {
     s = 0;
