@@ -114,7 +114,11 @@ typedef struct {
  *  bnd       UPML depths, grading and outer walls.
  *  precision FDTD_FP32, or FDTD_FP16_STORE (fields stored as FP16 with a
  *            power-of-two scale, arithmetic in FP32; UPML auxiliary D/B
- *            always FP32).  Any other value is FDTD_EINVAL.
+ *            always FP32).  Any other value is FDTD_EINVAL.  FP16 halves the
+ *            memory; it is the faster choice on boards past the resident
+ *            launches (fdtd_step) and no faster below (us a step, FP16 and
+ *            FP32: 56x48x30 32 and 4.5, 232x192x39 44 and 22, 280x230x100 91
+ *            and 92, 880x680x100 509 and 667).
  *  stream    cudaStream_t the context enqueues on; NULL makes the library
  *            create (and later destroy) its own non-blocking stream.
  *  out       receives the context.
@@ -183,8 +187,11 @@ int fdtd_step(fdtd_ctx *ctx, int n);
 int fdtd_set_tiled(fdtd_ctx *ctx, int on);
 int fdtd_is_resident(fdtd_ctx *ctx, int n, int *resident);
 
-/* fdtd_step with every phase launched directly (no CUDA graph) and timed
- * with CUDA events on the context's stream: phase_ms[0..5] receive the summed
+/* n steps by the tiled launches, every phase launched directly (no CUDA graph)
+ * one after the other and timed with CUDA events on the context's stream; the
+ * results are fdtd_step's.  A resident board's fdtd_step makes none of these
+ * launches: the times are then those of the tiled path it would take after
+ * fdtd_set_tiled, several times its own.  phase_ms[0..5] receive the summed
  * device time [ms] of the UPML/boundary slab H kernel, the fused H+E kernel
  * over the z-UPML planes of the interior columns, the fused H+E kernel over
  * the interior planes, the slab E kernel, the source/probe kernel and the
@@ -363,12 +370,13 @@ int fdtd_energy_static(const float *const fields[9], const float *const eps_r[3]
                        int pitch, double dx, double dy, double dz, const int upml_depth[6], void *stream,
                        double *energy, double *max_div_b);
 
-/* ---------------- batching (many boards, one launch per phase) -------------
+/* ---------------- batching (many boards in shared launches) ----------------
  * A batch steps many boards with one kernel launch per phase (UPML H, interior
  * fused H+E, UPML E, sources/probes) over a packed list of (board, tile) work
- * items, replayed as one CUDA graph per chunk of steps.  FP32 members up to 24
- * Mi grid points are worked in groups whose states stay in L2, many steps per
- * cooperative launch, each member by its own share of the blocks.  Each board's
+ * items, replayed as one CUDA graph per chunk of steps.  Members that are
+ * resident by the conditions of fdtd_step (FP32, up to 14 Mi grid points) are
+ * worked in groups whose states stay in L2, many steps per cooperative launch,
+ * each member by its own share of the blocks.  Each board's
  * arithmetic is identical to stepping it alone.  Boards keep their own device
  * state and may join or leave between calls.  All boards must share the
  * batch's stream (the batch uses its own; member contexts must not be

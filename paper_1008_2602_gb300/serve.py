@@ -4,8 +4,9 @@ Requests are boards (``workloads.Request``: arrival time + ``Problem``).  The
 server admits queued requests as soon as a batch slot and enough of the HBM
 budget are free, keeps every admitted board's fields on the device, and
 advances all admitted boards together with ``Batch.step`` in chunks of
-leapfrog steps (one launch per phase for the whole mix, replayed as a CUDA
-graph).  A board that reaches its step count retires at the next chunk
+leapfrog steps (FP32 boards up to 14 Mi grid points in groups, many steps per
+cooperative launch; the others by one launch per phase for all of them,
+replayed as a CUDA graph).  A board that reaches its step count retires at the next chunk
 boundary: its spectra are copied back, its device memory released and its
 latency (retire time - arrival time) recorded.  Requests that arrive while
 others are on the GPU join at the next chunk boundary, so their work overlaps

@@ -3,8 +3,8 @@
 ``Solver(problem)`` creates a board from a ``workloads.Problem`` (material
 volume, eps_r table, PEC boxes, UPML, walls, sources, probes, spectrum) and
 exposes ``step``, ``spectra``, ``traces``, ``field``, ``diagnostics``.
-``Batch`` steps many solvers with one launch per phase.  All arithmetic runs
-in libfdtd.so's CUDA kernels; this module only marshals arguments.
+``Batch`` steps many solvers in shared launches.  All arithmetic runs in
+libfdtd.so's CUDA kernels; this module only marshals arguments.
 """
 from __future__ import annotations
 
@@ -87,7 +87,7 @@ class Solver:
         return self
 
     def step_profiled(self, n: int) -> np.ndarray:
-        """n steps with per-phase CUDA-event timing: [slab H, fused z-UPML,
+        """n steps by the tiled launches with per-phase CUDA-event timing: [slab H, fused z-UPML,
         fused interior, slab E, sources/probes, DFT] summed device
         milliseconds."""
         ms = (ctypes.c_double * 6)()
