@@ -112,3 +112,36 @@ def test_a_tiled_batch_equals_each_board_alone(fdtd, precision):
     b.close()
     for s in sols:
         s.close()
+
+
+@pytest.mark.parametrize("axis,plane,rim,resident", [(0, 0, 0, True), (1, 0, 0, True), (2, 0, 0, True), (1, 17, 0, True),
+                                                     (1, 17, 1, False), (0, 40, 0, False), (1, 33, 0, False), (2, 26, 0, False)])
+def test_restored_planes_go_on_alike(fdtd, axis, plane, rim, resident):
+    """A checkpoint of a board with a plane of E_x, E_z written from outside:
+    only values behind a high PEC wall, which no step writes, keep it from the
+    resident launches (rim: the plane's own edges there have some too); both
+    ways give the same fields."""
+    import torch
+    from paper_1008_2602_gb300 import capi
+    p = W.random_problem(16, 40, 33, 26, upml=3, n_steps=60)
+    a, b, c = (fdtd.Solver(p) for _ in range(3))
+    a.step(9)
+    nodes = [n + 1 for n in (p.nz, p.ny, p.nx)]
+    del nodes[2 - axis]
+    vals = torch.rand([2] + nodes, generator=torch.Generator().manual_seed(1))
+    if not rim:
+        vals[:, -1, :] = vals[:, :, -1] = 0
+    vals = vals.cuda()
+    torch.cuda.synchronize()
+    capi.fdtd_halo_unpack(a.ctx, axis, plane, 0b101, vals.data_ptr())
+    state = a.save()
+    for s in (b, c):
+        s.load(state)
+    assert b.resident() == resident
+    c.set_tiled()
+    for n in (1, 6, 5):
+        b.step(n)
+        c.step(n)
+        _same(b, c)
+    for s in (a, b, c):
+        s.close()
